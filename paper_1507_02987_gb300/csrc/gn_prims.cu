@@ -76,51 +76,82 @@ void DeviceArena::release() {
 }
 
 // --------------------------------------------------------------- packing --
-__device__ __forceinline__ uint32_t base_bits(uint32_t b, uint32_t &bad) {
-    uint32_t c = b & 0xDFu;  // upper case for letters; other bytes stay non-bases
-    uint32_t code = (c == 'C') ? 1u : (c == 'G') ? 2u : (c == 'T' || c == 'U') ? 3u : 0u;
-    bad = (c == 'A' || c == 'C' || c == 'G' || c == 'T' || c == 'U') ? 0u : 1u;
-    return code;
+// Four ASCII bases at once (byte 0 first): their codes in bits 7-0, first base on top, and
+// bits 0-3 of bad for non-bases (whose code is 0).  Of a letter in upper case, bits 2-1 are
+// A 0, C 1, T and U 2, G 3, so v ^ (v >> 1) is the code; the letters that the codes stand for,
+// from one byte permute, tell bases from everything else (T and U differ in bit 0 only).  The
+// multiplications gather one field of each byte into adjacent bits; no two terms overlap.
+__device__ __forceinline__ uint32_t pack4(uint32_t x, uint32_t &bad) {
+    const uint32_t c = x & 0xDFDFDFDFu;  // upper case for letters; other bytes stay non-bases
+    uint32_t v = (c >> 1) & 0x03030303u;
+    v ^= (v >> 1) & 0x01010101u;
+    const uint32_t n = v | (v >> 4);  // nibbles b0 b1 in byte 0, b2 b3 in byte 2
+    const uint32_t want = __byte_perm(0x54474341u, 0u, (n & 0xFFu) | ((n >> 8) & 0xFF00u));  // "ACGT"
+    const uint32_t diff = (c ^ want) & ~(v & (v >> 1) & 0x01010101u);
+    const uint32_t no = ((((diff & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | diff) >> 7) & 0x01010101u;
+    bad = (no * 0x10204080u) >> 28;
+    v &= ~(no * 3u);
+    return (v * 0x40100401u) >> 24;
 }
 
-// One thread packs 32 bases: two code words and one non-base word.
-__global__ void k_pack(const uint8_t *__restrict__ ascii, uint64_t n, uint32_t *__restrict__ pk,
-                       uint32_t *__restrict__ nb, int aligned16) {
-    uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    uint64_t g0 = t * 32;
+// One thread packs 32 bases: two code words and one non-base word; the last one also writes
+// the words after the packed bases (zero codes, all non-bases).  The bytes come in aligned
+// 4-byte words shifted to the first base (16-byte loads where the input allows), and only
+// words that hold a byte of the input are read.  Bound by the instructions of pack4, near the
+// time of its bytes: 400 Mbp in 0.10 ms (0.59 ms one byte at a time; the bytes' floor is 0.08).
+__global__ void __launch_bounds__(256) k_pack(const uint8_t *__restrict__ ascii, uint64_t n, uint32_t *__restrict__ pk,
+                                              uint32_t *__restrict__ nb, uint64_t pk_words, uint64_t nb_words) {
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t g0 = t * 32;
     if (g0 >= n) return;
-    uint8_t buf[32];
-    if (aligned16 && g0 + 32 <= n) {
+    uint32_t w[9];
+    const uint32_t shift = 8u * (uint32_t)((uintptr_t)ascii & 3u);
+    const uint32_t left = (uint32_t)min((uint64_t)32, n - g0);  // bases of this thread
+    if (((uintptr_t)ascii & 15u) == 0 && left == 32) {
         const uint4 *src = reinterpret_cast<const uint4 *>(ascii + g0);
-        uint4 a = __ldg(src), b = __ldg(src + 1);
-        memcpy(buf, &a, 16);
-        memcpy(buf + 16, &b, 16);
+        const uint4 a = __ldg(src), b = __ldg(src + 1);
+        w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+        w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+        w[8] = 0;
     } else {
-        for (int i = 0; i < 32; ++i) buf[i] = (g0 + i < n) ? ascii[g0 + i] : (uint8_t)'N';
+        const uint32_t *src = reinterpret_cast<const uint32_t *>((uintptr_t)ascii & ~(uintptr_t)3) + g0 / 4;
+        const uint32_t bytes = shift / 8 + left;  // from the first word's start
+#pragma unroll
+        for (int i = 0; i < 9; ++i) w[i] = 4u * i < bytes ? __ldg(src + i) : 0u;
     }
     uint32_t w0 = 0, w1 = 0, bw = 0;
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
+    for (int i = 0; i < 8; ++i) {
         uint32_t bad;
-        uint32_t c = base_bits(buf[i], bad);
-        if (i < 16) w0 |= c << (30 - 2 * i);
-        else w1 |= c << (30 - 2 * (i - 16));
-        bw |= bad << i;
+        const uint32_t codes = pack4(__funnelshift_r(w[i], w[i + 1], shift), bad);
+        if (i < 4) w0 |= codes << (24 - 8 * i);
+        else w1 |= codes << (24 - 8 * (i - 4));
+        bw |= bad << (4 * i);
     }
-    pk[2 * t] = w0;
-    pk[2 * t + 1] = w1;
+    if (left < 32) {  // past the input: non-bases
+        bw |= 0xFFFFFFFFu << left;
+        w0 &= left < 16 ? ~(0xFFFFFFFFu >> (2 * left)) : 0xFFFFFFFFu;
+        w1 &= left <= 16 ? 0u : ~(0xFFFFFFFFu >> (2 * (left - 16)));
+    }
+    *reinterpret_cast<uint2 *>(pk + 2 * t) = make_uint2(w0, w1);
     nb[t] = bw;
+    if (g0 + 32 >= n) {
+        for (uint64_t i = 2 * t + 2; i < pk_words; ++i) pk[i] = 0u;
+        for (uint64_t i = t + 1; i < nb_words; ++i) nb[i] = 0xFFFFFFFFu;
+    }
 }
 
 void pack_bases(const uint8_t *ascii_dev, uint64_t n, Packed &out, cudaStream_t s) {
     out.n = n;
-    GN_CUDA(cudaMemsetAsync(out.pk, 0, Packed::pk_words(n) * 4, s));
-    GN_CUDA(cudaMemsetAsync(out.nb, 0xFF, Packed::nb_words(n) * 4, s));
-    if (n == 0) return;
-    uint64_t threads = (n + 31) / 32;
-    int aligned = ((uintptr_t)ascii_dev % 16) == 0;
+    if (n == 0) {
+        GN_CUDA(cudaMemsetAsync(out.pk, 0, Packed::pk_words(n) * 4, s));
+        GN_CUDA(cudaMemsetAsync(out.nb, 0xFF, Packed::nb_words(n) * 4, s));
+        return;
+    }
+    const uint64_t threads = (n + 31) / 32;
     GN_LAUNCH("k_pack", n, s,
-              k_pack<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(ascii_dev, n, out.pk, out.nb, aligned));
+              k_pack<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(ascii_dev, n, out.pk, out.nb, Packed::pk_words(n),
+                                                                     Packed::nb_words(n)));
 }
 
 // ----------------------------------------------------------------- scans --
