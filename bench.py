@@ -50,6 +50,10 @@ BYTES_PER_UNIT = {
     "record_sort_downsweep": 24.0,
     "record_sort_upsweep": 8.0,
     "k_query_codes": 17.0,
+    # one base and one list range read, one record, position and unit count written
+    "k_query_recs": 41.0,
+    # signature scan (units = hits): one 4-byte signature read per hit
+    "k_seed_scan": 4.0,
     # bucket fill (units = hits): one 4-byte occurrence read per hit; the 8-byte writes of the
     # kept hits are added from k_bucket_group's units (kept hits) in roofline()
     "k_bucket_fill": 4.0,
@@ -684,7 +688,7 @@ def run_ours(args, dist):
                 "config": {"workload": desc, "bank_bases": bank.n_bases, "bank_seqs": bank.n_seqs,
                            "n_queries": queries.n, "query_bases_per_rank": M, "k": 11, "stride": args.stride,
                            "mask": args.mask, "band_w": band_w, "autotune": tuned,
-                           "hits_per_step": (kern.get("k_bucket_fill") or kern.get("k_seed_gather") or [0, 0, 0])[2]
+                           "hits_per_step": (kern.get("k_seed_scan") or kern.get("k_bucket_fill") or kern.get("k_seed_gather") or [0, 0, 0])[2]
                            / max(1, args.steps),
                            "parallelism": f"replicas x{dist.world}",
                            "l2": "inputs larger than L2 (postings and hit keys are GBs per step); no flush"},

@@ -24,42 +24,99 @@ __global__ void k_window_counts(const uint64_t *__restrict__ seq_start, uint32_t
 }
 
 constexpr int WIN_J = 8;  // windows per lane per warp chunk
+constexpr int WIN_CHUNK = 32 * WIN_J;
 
-// Pass 1 (flags = true): validity flag of every window + bucket histogram.
-// Pass 2 (flags = false): key (code << 32 | global offset) of every valid window at its compacted slot.
-template <bool FLAGS>
+// Windows of warp chunk c: [c * WIN_CHUNK, ...), lane by lane.  COUNT: the chunk's valid
+// windows (no non-base at a kept position).  Otherwise: the key (code << 32 | global offset)
+// of every valid window, in window order from the chunk's first slot, and the bucket
+// histogram.  One count per chunk and a ballot rank give the slots, so that no flag or slot
+// per window goes through memory (400 Mbp, 36.4 M windows: flags, their scan and the two
+// window passes 0.9 GB, now 0.45 GB).
+template <bool COUNT>
 __global__ void k_bank_windows(const uint64_t *__restrict__ seq_start, const uint64_t *__restrict__ woff,
                                uint32_t n_seqs, uint64_t W, const uint32_t *__restrict__ pk,
-                               const uint32_t *__restrict__ nb, SeedShape sh, int t, uint32_t *__restrict__ flags,
-                               uint32_t *__restrict__ hist, const uint64_t *__restrict__ slot,
+                               const uint32_t *__restrict__ nb, SeedShape sh, int t, uint32_t *__restrict__ count,
+                               uint32_t *__restrict__ hist, const uint64_t *__restrict__ first,
                                uint64_t *__restrict__ keys) {
     const int lane = threadIdx.x & 31;
-    uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint64_t w0 = warp * 32 * WIN_J;
+    const uint64_t chunk = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t w0 = chunk * WIN_CHUNK;
     if (w0 >= W) return;
     uint32_t s = 0;
     if (lane == 0) s = dev_upper_index(woff, n_seqs + 1, w0);
     s = __shfl_sync(0xffffffffu, s, 0);
+    uint64_t slot = COUNT ? 0 : first[chunk];
+    uint32_t total = 0;
 #pragma unroll
     for (int it = 0; it < WIN_J; ++it) {
-        uint64_t w = w0 + (uint64_t)it * 32 + lane;
-        if (w >= W) break;
-        while (woff[s + 1] <= w) ++s;
-        uint64_t g = seq_start[s] + (w - woff[s]) * (uint64_t)t;
-        bool bad = dev_seed_has_nonbase(nb, g, sh);
-        uint32_t code = dev_seed_code(pk, g, sh);
-        if (FLAGS) {
-            flags[w] = bad ? 0u : 1u;
-            if (!bad) atomicAdd(&hist[code], 1u);
-        } else if (!bad) {
-            keys[slot[w]] = ((uint64_t)code << 32) | g;
+        const uint64_t w = w0 + (uint64_t)it * 32 + lane;
+        uint64_t g = 0;
+        bool ok = w < W;
+        if (ok) {
+            while (woff[s + 1] <= w) ++s;
+            g = seq_start[s] + (w - woff[s]) * (uint64_t)t;
+            ok = !dev_seed_has_nonbase(nb, g, sh);
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, ok);
+        if (COUNT) {
+            total += __popc(m);
+        } else {
+            if (ok) {
+                const uint32_t code = dev_seed_code(pk, g, sh);
+                atomicAdd(&hist[code], 1u);
+                keys[slot + __popc(m & ((1u << lane) - 1u))] = ((uint64_t)code << 32) | g;
+            }
+            slot += __popc(m);
         }
     }
+    if (COUNT && lane == 0) count[chunk] = total;
 }
 
-__global__ void k_low_words(const uint64_t *__restrict__ keys, uint64_t n, uint32_t *__restrict__ out) {
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (uint32_t)keys[i];
+// Signature of the occurrence at bank position g.  Fields ahead are taken from the packed
+// bases whatever sequence they belong to and whether they are bases: a field that matches
+// wrongly costs the search one check, none is missed.  Bound by the gather of the bases after
+// g (one or two 32-byte sectors an occurrence).
+__device__ __forceinline__ uint32_t occurrence_sig(uint64_t g, uint64_t n, const uint32_t *__restrict__ pk,
+                                                   const uint32_t *__restrict__ nb, const SeqMap &sm,
+                                                   const SeedShape &sh, int t, int kind) {
+    uint32_t sig = 0;
+    if (kind == SIG_FLANK) {
+        sig = SIG_NO_BASE;
+        if (g > 0 && g < n) {
+            const uint32_t sq = sm.lut ? dev_seq_of(sm, g) : dev_upper_index(sm.start, sm.n_seqs + 1, g);
+            if (sm.start[sq] != g) sig = dev_base(pk, nb, g - 1);
+        }
+        if (g + (uint64_t)sh.span <= n) sig |= sig_flank(pk, g + (uint64_t)sh.span);
+    } else {
+        for (int j = 0; j < SIG_FIELDS; ++j) {
+            const uint64_t x = g + (uint64_t)t * (j + 1);
+            sig |= (x + (uint64_t)sh.span <= n ? sig_hash(dev_seed_code(pk, x, sh)) : SIG_NONE) << (10 * j);
+        }
+    }
+    return sig;
+}
+
+// Occurrences and their signatures from the sorted keys (keys null: signatures of the
+// occurrences that post already holds).  post and sig: post_alloc_entries words.
+__global__ void k_occurrences(const uint64_t *__restrict__ keys, uint64_t n_post, uint32_t *__restrict__ post,
+                              uint32_t *__restrict__ sig, uint64_t n, const uint32_t *__restrict__ pk,
+                              const uint32_t *__restrict__ nb, SeqMap sm, SeedShape sh, int t, int kind) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_post) return;
+    const uint32_t g = keys ? (uint32_t)keys[i] : post[i];
+    if (keys) post[i] = g;
+    if (sig) sig[i] = occurrence_sig(g, n, pk, nb, sm, sh, t, kind);
+}
+
+// Room for the signatures; without it searches take the path that does not read them.
+static void alloc_sigs(gn_index *ix, uint64_t &bytes) {
+    const size_t want = sizeof(uint32_t) * post_alloc_entries(ix->n_postings);
+    if (cudaMalloc(&ix->sig_d, want) == cudaSuccess) {
+        bytes += sizeof(uint32_t) * ix->n_postings;
+    } else {
+        cudaGetLastError();
+        ix->sig_d = nullptr;
+    }
 }
 
 // lut[j] = last sequence s with start[s] <= j << SEQ_LUT_SHIFT (positions past the bank
@@ -169,42 +226,46 @@ static void index_build_shape(const gn_bank *db, int k, int span, uint32_t keep,
     GN_CUDA(cudaMemcpyAsync(&W, woff + ns, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     GN_CUDA(cudaStreamSynchronize(s));
 
-    // K2: window validity + bucket histogram
-    uint32_t *hist = arena.alloc_n<uint32_t>(nbk);
-    GN_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * nbk, s));
-    uint32_t *flags = arena.alloc_n<uint32_t>(W);
-    uint64_t *slot = arena.alloc_n<uint64_t>(W + 1);
-    uint64_t warps = (W + 32 * WIN_J - 1) / (32 * WIN_J);
-    unsigned grid = (unsigned)std::max<uint64_t>(1, (warps * 32 + 255) / 256);
+    // K2: valid windows per chunk and their exclusive scan
+    const uint64_t chunks = (W + WIN_CHUNK - 1) / WIN_CHUNK;
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, (chunks * 32 + 255) / 256);
+    uint32_t *ccnt = arena.alloc_n<uint32_t>(chunks);
+    uint64_t *coff = arena.alloc_n<uint64_t>(chunks + 1);
     if (W) {
-        GN_LAUNCH("k_bank_windows_flags", W, s,
+        GN_LAUNCH("k_bank_windows_count", W, s,
                   k_bank_windows<true><<<grid, 256, 0, s>>>(ix->seq_start_d, woff, ns, W, ix->bank.pk, ix->bank.nb, sh, t,
-                                                  flags, hist, nullptr, nullptr));
+                                                  ccnt, nullptr, nullptr, nullptr));
     }
-    // K3: bucket starts = exclusive scan of the histogram
-    exclusive_scan_u32(hist, ix->off_d, nbk, scan_scr, s);
-    void *scan_scr2 = arena.alloc(scan_scratch_bytes(W));
-    exclusive_scan_u32(flags, slot, W, scan_scr2, s);
+    void *scan_scr2 = arena.alloc(scan_scratch_bytes(chunks));
+    exclusive_scan_u32(ccnt, coff, chunks, scan_scr2, s);
     uint64_t P = 0;
-    GN_CUDA(cudaMemcpyAsync(&P, ix->off_d + nbk, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    GN_CUDA(cudaMemcpyAsync(&P, coff + chunks, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     GN_CUDA(cudaStreamSynchronize(s));
     ix->n_postings = P;
 
-    // K4: stable scatter = stable radix sort of (code, global offset) keys by code
+    // K3: keys of the valid windows and the bucket histogram, whose exclusive scan gives the
+    // bucket starts
+    uint32_t *hist = arena.alloc_n<uint32_t>(nbk);
+    GN_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * nbk, s));
     uint64_t *keys = arena.alloc_n<uint64_t>(P);
     uint64_t *keys_alt = arena.alloc_n<uint64_t>(P);
     if (W) {
         GN_LAUNCH("k_bank_windows_keys", W, s,
                   k_bank_windows<false><<<grid, 256, 0, s>>>(ix->seq_start_d, woff, ns, W, ix->bank.pk, ix->bank.nb, sh, t,
-                                                   nullptr, nullptr, slot, keys));
+                                                   nullptr, hist, coff, keys));
     }
+    exclusive_scan_u32(hist, ix->off_d, nbk, scan_scr, s);
+
+    // K4: stable scatter = stable radix sort of (code, global offset) keys by code
     void *rs = arena.alloc(radix_scratch_bytes(P));
     bool flipped = radix_sort(keys, keys_alt, nullptr, nullptr, P, 32, 32 + 2 * k, rs, s, TAG_INDEX_SORT);
     GN_CUDA(cudaMalloc(&ix->post_d, sizeof(uint32_t) * post_alloc_entries(P)));
     bytes += sizeof(uint32_t) * P;
+    alloc_sigs(ix, bytes);
     if (P) {
-        GN_LAUNCH("k_low_words", P, s,
-                  k_low_words<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(flipped ? keys_alt : keys, P, ix->post_d));
+        GN_LAUNCH("k_occurrences", P, s,
+                  k_occurrences<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(flipped ? keys_alt : keys, P, ix->post_d, ix->sig_d, n,
+                                                                         ix->bank.pk, ix->bank.nb, seq_map(ix), sh, t, sig_kind(k, span, t)));
     }
     uint32_t wst = 0;
     GN_CUDA(cudaMemcpyAsync(&wst, wait_status, 4, cudaMemcpyDeviceToHost, s));
@@ -222,6 +283,7 @@ void index_free(gn_index *ix) {
     cudaFree(ix->bank.nb);
     cudaFree(ix->off_d);
     cudaFree(ix->post_d);
+    cudaFree(ix->sig_d);
 }
 
 void index_export(const gn_index *ix, uint64_t *bucket_start, uint32_t *post_seq, uint32_t *post_pos) {
@@ -353,6 +415,17 @@ void index_load(const char *path, gn_index *ix) {
     uint64_t last = 0;
     GN_CUDA(cudaMemcpy(&last, ix->off_d + (nbk - 1), 8, cudaMemcpyDeviceToHost));
     GN_REQUIRE(last == np, GN_EINVAL, "index file: bucket starts do not end at the occurrence count");
+    // the signatures are not in the file: they follow from the occurrences and the bank (the
+    // lookup table, unchecked file content, is not walked here)
+    alloc_sigs(ix, bytes);
+    if (np && ix->sig_d) {
+        GN_LAUNCH("k_occurrences", np, 0,
+                  k_occurrences<<<(unsigned)((np + 255) / 256), 256>>>(nullptr, np, ix->post_d, ix->sig_d, n, ix->bank.pk,
+                                                                     ix->bank.nb, SeqMap{ix->seq_start_d, nullptr, ix->n_seqs},
+                                                                     seed_shape(ix), ix->t,
+                                                                     sig_kind(ix->k, ix->span, ix->t)));
+        GN_CUDA(cudaDeviceSynchronize());
+    }
     ix->device_bytes = bytes;
 }
 

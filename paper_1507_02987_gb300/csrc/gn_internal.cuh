@@ -258,6 +258,29 @@ __device__ __forceinline__ uint32_t dev_upper_index(const uint64_t *__restrict__
 // any list in aligned 16-byte loads; the entries past n are never used.
 inline uint64_t post_alloc_entries(uint64_t n) { return std::max<uint64_t>(4, (n + 3) & ~3ull); }
 
+// Occurrence signatures: one word per occurrence, beside the occurrence array, that tells
+// from the word alone whether a seed hit can have another hit ahead on its diagonal.
+// Windows of one sequence start t apart, so the next hits of a chain lie t, 2t or 3t bases
+// on.  SIG_AHEAD: three 10-bit fields, field j the hash of the seed code t (j + 1) bases on
+// (SIG_NONE past the bank's end).  Stride 1 without a mask shares all but one base with the
+// next window, so a hash of its code says little; there SIG_FLANK keeps the bases themselves:
+// bits 0-2 the base before the window (SIG_NO_BASE at a sequence start or a non-base), bits
+// 3-30 the 14 bases after it, the first one on top (0 past the bank's end).
+// Hash values of codes stay below SIG_NONE; a query field SIG_NEVER equals no stored field.
+enum SigKind : int { SIG_AHEAD = 0, SIG_FLANK = 1 };
+constexpr uint32_t SIG_NONE = 1022, SIG_NEVER = 1023;
+constexpr uint32_t SIG_NO_BASE = 4, SIG_NO_BASE_QUERY = 5;  // never equal: a window without a predecessor starts a chain
+constexpr int SIG_FLANK_BASES = 14;
+constexpr int SIG_FIELDS = 3;
+__device__ __forceinline__ uint32_t sig_hash(uint32_t code) { return min((code * 0x9E3779B1u) >> 22, SIG_NONE - 1u); }
+__device__ __forceinline__ uint32_t sig_flank(const uint32_t *__restrict__ pk, uint64_t x) {  // the bases from x on
+    const uint64_t w = x >> 4;
+    return __funnelshift_l(pk[w + 1], pk[w], 2u * (uint32_t)(x & 15)) >> 4 << 3;
+}
+// the first f of those bases
+__host__ __device__ __forceinline__ uint32_t sig_flank_mask(int f) { return ((1u << (2 * f)) - 1u) << (31 - 2 * f); }
+inline SigKind sig_kind(int k, int span, int t) { return t == 1 && span == k ? SIG_FLANK : SIG_AHEAD; }
+
 constexpr int SEQ_LUT_SHIFT = 10;
 struct SeqMap {
     const uint64_t *start;  // n_seqs + 1 sequence starts (start[n_seqs] = bank length)
@@ -303,6 +326,7 @@ struct gn_index {
     gn::Packed bank;                  // packed bank + non-base bitmap
     uint64_t *off_d = nullptr;        // 4^k + 1 bucket starts
     uint32_t *post_d = nullptr;       // occurrences: global base offset of the window (post_alloc_entries)
+    uint32_t *sig_d = nullptr;        // occurrence signatures (SigKind), entry for entry; null without room for them
     uint64_t device_bytes = 0;
     // per-phase device times of the most recent search through this handle
     std::vector<std::pair<const char *, float>> last_phases;

@@ -1091,6 +1091,10 @@ __global__ void k_xdrop(DevHsp *__restrict__ h, uint32_t n, const uint32_t *__re
     }
 }
 
+}  // namespace gn
+#include "gn_seed_scan.cuh"
+namespace gn {
+
 // ------------------------------------------- long queries: segments, join --
 // Bases of each segment (block v): len bytes from offset off[v] of query parent[v].
 __global__ void k_segment_bases(const uint8_t *__restrict__ qbases, const uint64_t *__restrict__ qstart,
@@ -2369,6 +2373,15 @@ std::vector<T> to_host(const T *d, size_t n, cudaStream_t s) {
 
 unsigned blocks_for(uint64_t n, unsigned t = 256) { return (unsigned)std::max<uint64_t>(1, (n + t - 1) / t); }
 
+// A hit-storing path is asked for: the path itself, or one of the settings that only the
+// buckets have.
+bool hit_path_forced() {
+    for (const char *v : {"GN_HIT_GROUPING", "GN_TILE_FILTER", "GN_TILE_POS", "GN_TILE_FBITS", "GN_TILE_FBITS2",
+                          "GN_FILL_THREADS", "GN_BUCKET_TARGET", "GN_BUCKET_CAP", "GN_SPILL_ROOM", "GN_MAX_CHUNK_HITS"})
+        if (getenv(v)) return true;
+    return false;
+}
+
 // Lets the kernels with a per-call dynamic shared-memory size use up to the device's opt-in
 // maximum.  Set once per device: concurrent searches (serving threads) launch with different
 // sizes, and a per-call attribute change by one thread could undercut another's launch.
@@ -2526,12 +2539,37 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         hqp.nb = arena.alloc_n<uint32_t>(Packed::nb_words(HM));
         pack_bases(sb, HM, hqp, s);
     }
-    uint32_t *codes = arena.alloc_n<uint32_t>(HM);
+    // Seed lookup and chaining take one of two routes to the same HSPs.  The signature scan
+    // (gn_seed_scan.cuh) reads each occurrence's signature once and stores no hit; it serves
+    // searches in which a chain needs two hits (min_hsp_len > span) at most SIG_FIELDS windows
+    // apart (with SIG_FLANK: windows that overlap or touch), the distances a signature holds.
+    // Everything else, and a search for which a hit-storing path is forced, goes through the
+    // buckets or the global sort below.  Where both serve, the scan is faster at every size
+    // measured (scan and chains against fill, grouping and the sort of its spills): one query of
+    // 2,000 bases on 4 Gbp 29 against 36 us; 4,096 short queries on 400 Mbp 0.18 against 0.60 ms;
+    // 2,000 queries on 4 Gbp 1.46 against 3.70 ms; 500 queries at stride 1 0.13 against 3.2 ms.
+    const int singles = p.min_hsp_len <= (uint32_t)k ? 1 : 0;
+    const SigKind kind = sig_kind(ix->k, ix->span, ix->t);
+    const uint32_t links = p.max_hit_distance / (uint32_t)ix->t;  // windows from one hit to the next, at most
+    const bool scan = ix->sig_d && !singles && !keep_hits && !hit_path_forced() &&
+                      (kind == SIG_FLANK ? links >= 1 && links <= (uint32_t)k : links >= 1 && links <= (uint32_t)SIG_FIELDS);
+    uint32_t *codes = scan ? nullptr : arena.alloc_n<uint32_t>(HM);
     uint32_t *qinfo = arena.alloc_n<uint32_t>(HM);
-    uint32_t *cnt = arena.alloc_n<uint32_t>(HM);
-    uint32_t *src = arena.alloc_n<uint32_t>(HM);
+    uint32_t *cnt = arena.alloc_n<uint32_t>(HM);  // list lengths; scan route: list units
     uint64_t *hoff = arena.alloc_n<uint64_t>(HM + 1);
-    if (HM) {
+    uint32_t *src = scan ? nullptr : arena.alloc_n<uint32_t>(HM);
+    QueryRec *qrec = scan ? arena.alloc_n<QueryRec>(HM) : nullptr;
+    uint64_t *hq_d = arena.alloc_n<uint64_t>(hnq + 1);
+    const int flank = (int)std::min<uint32_t>(SIG_FLANK_BASES, p.min_hsp_len > (uint32_t)k ? p.min_hsp_len - (uint32_t)k : 0u);
+    if (scan) {
+        GN_CUDA(cudaMemsetAsync(hq_d, 0, 8 * (hnq + 1), s));
+        auto kernel = kind == SIG_FLANK ? k_query_recs<SIG_FLANK> : k_query_recs<SIG_AHEAD>;
+        if (HM)
+            GN_LAUNCH("k_query_recs", HM, s,
+                      kernel<<<blocks_for(HM), 256, 0, s>>>(hstart_d, hnq, HM, hqp.pk, hqp.nb, seed_shape(ix), ix->t,
+                                                            (int)links, flank, ix->off_d, qinfo, qrec, cnt,
+                                                            reinterpret_cast<unsigned long long *>(hq_d)));
+    } else if (HM) {
         GN_LAUNCH("k_query_codes", HM, s,
                   k_query_codes<<<blocks_for(HM), 256, 0, s>>>(hstart_d, hnq, HM, hqp.pk, hqp.nb, seed_shape(ix), ix->off_d, codes, qinfo,
                                                               cnt, src));
@@ -2540,11 +2578,20 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         void *scr = arena.alloc(scan_scratch_bytes(HM));
         exclusive_scan_u32(cnt, hoff, HM, scr, s);
     }
-    // hit offsets at query boundaries -> per-query hit counts (chunk plan)
-    uint64_t *hq_d = arena.alloc_n<uint64_t>(hnq + 1);
-    GN_LAUNCH("k_gather_u64", hnq + 1, s,
-              k_gather_u64<<<blocks_for(hnq + 1), 256, 0, s>>>(hoff, hstart_d, hnq + 1, hq_d));
+    // per-query hit counts (limits; the chunk plan of the hit-storing paths), as prefix sums
+    if (!scan)
+        GN_LAUNCH("k_gather_u64", hnq + 1, s,
+                  k_gather_u64<<<blocks_for(hnq + 1), 256, 0, s>>>(hoff, hstart_d, hnq + 1, hq_d));
     std::vector<uint64_t> hq = to_host(hq_d, hnq + 1, s);
+    if (scan) {
+        uint64_t at = 0;
+        for (uint32_t i = 0; i <= hnq; ++i) {
+            const uint64_t h = hq[i];
+            GN_REQUIRE(i == hnq || h < (1ull << 32), GN_ETOOBIG, "a query has 2^32 seed hits or more");
+            hq[i] = at;
+            at += h;
+        }
+    }
     GN_REQUIRE(!o.max_hit_bytes || hq[hnq] * HIT_BYTES <= o.max_hit_bytes, GN_ETOOBIG,
                "the query alone exceeds the server's memory budget");
     timer.mark("query_codes");
@@ -2577,7 +2624,77 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     GN_CUDA(cudaMemsetAsync(status, 0, 4, s));
     std::vector<uint32_t> hits_q;
 
-    uint32_t qa = 0;
+    // appends HSPs through `launch(out, room)`, growing the HSP buffer and relaunching on overflow
+    auto emit = [&](auto launch) {
+        for (int attempt = 0; attempt < 3; ++attempt) {
+            GN_CUDA(cudaMemsetAsync(counter, 0, 4, s));
+            launch(hsp + n_hsp, hsp_cap - n_hsp);
+            uint32_t got = 0;
+            GN_CUDA(cudaMemcpyAsync(&got, counter, 4, cudaMemcpyDeviceToHost, s));
+            GN_CUDA(cudaStreamSynchronize(s));
+            if (n_hsp + (uint64_t)got <= hsp_cap) {
+                n_hsp += got;
+                return;
+            }
+            uint64_t need = (uint64_t)n_hsp + got;
+            GN_REQUIRE(need < (1ull << 32), GN_ETOOBIG, "more than 2^32 HSPs in one call");
+            uint32_t ncap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull,
+                                                         std::max<uint64_t>(need + need / 4, 2ull * hsp_cap));
+            DevHsp *nh = arena.alloc_n<DevHsp>(ncap);
+            if (n_hsp) GN_CUDA(cudaMemcpyAsync(nh, hsp, sizeof(DevHsp) * n_hsp, cudaMemcpyDeviceToDevice, s));
+            hsp = nh;
+            hsp_cap = ncap;
+            GN_CUDA(cudaMemsetAsync(status, 0, 4, s));
+        }
+        throw Error{GN_EINTERNAL, "HSP buffer growth did not converge"};
+    };
+    if (scan && hq[hnq]) {
+        auto kernel = kind == SIG_FLANK ? k_seed_scan<SIG_FLANK> : k_seed_scan<SIG_AHEAD>;
+        auto chain = kind == SIG_FLANK ? k_chain<SIG_FLANK> : k_chain<SIG_AHEAD>;
+        int occ = 0, cocc = 0;
+        GN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, SCAN_THREADS, 0));
+        GN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cocc, chain, SCAN_THREADS, 0));
+        // resident blocks; fewer when the hits (at most 4 a unit, plus an offset's own unit) do not fill them
+        const uint64_t tiles = (hq[hnq] / 4 + 2 * HM) / 64 + 1;
+        const unsigned grid = (unsigned)std::max<uint64_t>(
+            1, std::min<uint64_t>((tiles + SCAN_THREADS / 32 - 1) / (SCAN_THREADS / 32), (uint64_t)num_sms() * std::max(occ, 1)));
+        // room for candidates: about 1 % of the hits at stride 11
+        uint64_t cand_cap = std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 16, hq[hnq] / 32));
+        uint2 *cand = arena.alloc_n<uint2>(cand_cap);
+        uint32_t *sctr = arena.alloc_n<uint32_t>(4);  // candidates, tile counter, candidate counter
+        bool scanned = false;
+        for (int attempt = 0;; ++attempt) {
+            uint32_t n_cand = 0;
+            emit([&](DevHsp *o, uint32_t room) {
+                if (!scanned) {
+                    GN_CUDA(cudaMemsetAsync(sctr, 0, 16, s));
+                    GN_LAUNCH("k_seed_scan", hq[hnq], s,
+                              kernel<<<grid, SCAN_THREADS, 0, s>>>(qrec, hoff, HM, reinterpret_cast<const uint4 *>(ix->sig_d),
+                                                                   post_alloc_entries(ix->n_postings) / 4, flank, cand,
+                                                                   sctr, (uint32_t)cand_cap, sctr + 1));
+                    scanned = true;
+                }
+                GN_CUDA(cudaMemsetAsync(sctr + 2, 0, 4, s));
+                const ScanCtx c{qinfo, hstart_d, ix->post_d, ix->bank.pk, ix->bank.nb, hqp.pk, hqp.nb, seed_shape(ix),
+                                ix->t, (int)links, flank, hit_min_len, seq_map(ix), o, counter, room, status,
+                                ix->n_postings, ix->n_bases, HM};
+                GN_LAUNCH("k_chain", hq[hnq], s,
+                          chain<<<(unsigned)std::min<uint64_t>((cand_cap + SCAN_THREADS - 1) / SCAN_THREADS,
+                                                               (uint64_t)num_sms() * std::max(cocc, 1)),
+                                  SCAN_THREADS, 0, s>>>(c, cand, sctr, (uint32_t)cand_cap, sctr + 2));
+                GN_CUDA(cudaMemcpyAsync(&n_cand, sctr, 4, cudaMemcpyDeviceToHost, s));
+            });
+            if (n_cand <= cand_cap) break;
+            GN_REQUIRE(attempt < 1, GN_EINTERNAL, "candidate list sizing did not converge");
+            n_hsp = 0;  // the rerun emits everything again
+            cand_cap = n_cand;
+            cand = arena.alloc_n<uint2>(cand_cap);
+            scanned = false;
+        }
+        timer.mark("seed_scan");
+    }
+
+    uint32_t qa = scan ? hnq : 0;
     while (qa < hnq) {
         uint32_t qb = qa + 1;
         while (qb < hnq && qb - qa < max_chunk_q && hq[qb + 1] - hq[qa] <= hit_budget) ++qb;
@@ -2589,30 +2706,6 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
             const int gbits = (int)gbits_max;
             const uint32_t nqc = qb - qa;
             DeviceArena carena(s);
-            // appends HSPs through `launch(out, room)`, growing the HSP buffer and relaunching on overflow
-            auto emit = [&](auto launch) {
-                for (int attempt = 0; attempt < 3; ++attempt) {
-                    GN_CUDA(cudaMemsetAsync(counter, 0, 4, s));
-                    launch(hsp + n_hsp, hsp_cap - n_hsp);
-                    uint32_t got = 0;
-                    GN_CUDA(cudaMemcpyAsync(&got, counter, 4, cudaMemcpyDeviceToHost, s));
-                    GN_CUDA(cudaStreamSynchronize(s));
-                    if (n_hsp + (uint64_t)got <= hsp_cap) {
-                        n_hsp += got;
-                        return;
-                    }
-                    uint64_t need = (uint64_t)n_hsp + got;
-                    GN_REQUIRE(need < (1ull << 32), GN_ETOOBIG, "more than 2^32 HSPs in one call");
-                    uint32_t ncap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull,
-                                                                 std::max<uint64_t>(need + need / 4, 2ull * hsp_cap));
-                    DevHsp *nh = arena.alloc_n<DevHsp>(ncap);
-                    if (n_hsp) GN_CUDA(cudaMemcpyAsync(nh, hsp, sizeof(DevHsp) * n_hsp, cudaMemcpyDeviceToDevice, s));
-                    hsp = nh;
-                    hsp_cap = ncap;
-                    GN_CUDA(cudaMemsetAsync(status, 0, 4, s));
-                }
-                throw Error{GN_EINTERNAL, "HSP buffer growth did not converge"};
-            };
             // global path: gather every hit, LSD radix sort by diagonal key, merge sorted runs
             auto sort_path = [&](uint64_t *keys, uint64_t *keys_alt, uint64_t n, int lo_bit, const RadixTag &tag) {
                 void *rs = carena.alloc(radix_scratch_bytes(n));
@@ -2650,7 +2743,6 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
                 }
             } else {
                 // bucket plan: 2^lg buckets per query, about `target` raw hits each
-                const int singles = p.min_hsp_len <= (uint32_t)k ? 1 : 0;
                 const char *fenv = getenv("GN_TILE_FILTER");
                 const int filter = (!singles && p.max_hit_distance <= (uint32_t)BT_MAX_D &&
                                     !(fenv && strcmp(fenv, "0") == 0)) ? 1 : 0;
