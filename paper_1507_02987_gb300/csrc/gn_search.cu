@@ -889,21 +889,6 @@ __device__ __forceinline__ int32_t dev_pair(uint32_t a, uint32_t b, int32_t matc
     return (a < 4u && a == b) ? match : mismatch;
 }
 
-// Walks packed bases one at a time, reloading the code word every 16 bases and the
-// non-base word every 32 (instead of two loads per base).
-struct BaseCursor {
-    const uint32_t *pk, *nb;
-    uint64_t wpk_i = ~0ull, wnb_i = ~0ull;
-    uint32_t wpk = 0, wnb = 0;
-    __device__ __forceinline__ BaseCursor(const uint32_t *p, const uint32_t *n) : pk(p), nb(n) {}
-    __device__ __forceinline__ uint32_t at(uint64_t g) {  // 2-bit code, or 4 for a non-base
-        const uint64_t a = g >> 4, b = g >> 5;
-        if (a != wpk_i) { wpk_i = a; wpk = pk[a]; }
-        if (b != wnb_i) { wnb_i = b; wnb = nb[b]; }
-        return ((wnb >> (g & 31)) & 1u) ? 4u : (wpk >> (30 - 2 * (int)(g & 15))) & 3u;
-    }
-};
-
 // One direction of the X-drop walk, 32 steps per round for a whole warp.  Step e
 // (1-based) compares query base qg(e) with bank base dg(e).  The sequential rule
 // (score += s; if score > best: best = score, ext = e; else if best - score > X:
@@ -1387,111 +1372,20 @@ __device__ __forceinline__ void scan_pair_max(int32_t &v, uint32_t &s, int lane)
 }
 
 
-// Band of at most 64 diagonals: lane l owns the two adjacent band offsets 2l and
-// 2l+1 and keeps their previous-row states in registers.  The vertical-gap input of
-// offset 2l is the lane's own offset 2l+1; that of 2l+1 comes from the next lane.
-// One warp max-scan per row resolves horizontal gaps for all 64 offsets: each lane
-// contributes the later-wins maximum of its two X values.  Bases are read through
-// per-lane word cursors (one load per 16 rows).
-__device__ __forceinline__ void sw_rows_pair(int64_t I0, int64_t I1, int64_t J0, int64_t J1, int64_t dlo, int64_t B,
-                                             uint64_t qb, uint64_t sb, const uint32_t *__restrict__ qpk,
-                                             const uint32_t *__restrict__ qnb, const uint32_t *__restrict__ bpk,
-                                             const uint32_t *__restrict__ bnb, int32_t match, int32_t mismatch,
-                                             int32_t goe, int32_t ge, int lane, int32_t &best, int64_t &bi,
-                                             int64_t &bj, uint32_t &bs) {
-    int32_t pH0 = 0, pE0 = SW_NEG, pH1 = 0, pE1 = SW_NEG;
-    uint32_t pSH0 = 0, pSE0 = 0, pSH1 = 0, pSE1 = 0;
-    const int32_t b0 = 2 * lane, b1 = 2 * lane + 1;
-    BaseCursor cq(qpk, qnb), cd(bpk, bnb);
-    const int32_t irows = (int32_t)(I1 - I0);
-    const uint32_t Bu = (uint32_t)B;  // start cells: row * B + band offset
-    const int32_t jlo = (int32_t)(J0 - I0 - dlo), jhi = (int32_t)(J1 - 1 - I0 - dlo);  // band offset limits at row I0
-    for (int32_t r = 0; r < irows; ++r) {
-        // row i = I0 + r: band offsets with J0 <= i + dlo + b <= J1 - 1
-        const int32_t blo = max(0, jlo - r), bhi = min((int32_t)B - 1, jhi - r);
-        if (blo > bhi) continue;
-        const bool prow = r > 0;
-        const int32_t pblo = max(0, jlo - r + 1), pbhi = min((int32_t)B - 1, jhi - r + 1);
-        const uint64_t i = (uint64_t)(I0 + r);
-        const uint32_t qc = cq.at(qb + i);
-        // previous-row state at offset b1 + 1 = next lane's b0
-        const int32_t uH = __shfl_down_sync(0xffffffffu, pH0, 1), uE = __shfl_down_sync(0xffffffffu, pE0, 1);
-        const uint32_t uSH = __shfl_down_sync(0xffffffffu, pSH0, 1), uSE = __shfl_down_sync(0xffffffffu, pSE0, 1);
-        const bool act0 = b0 >= blo && b0 <= bhi, act1 = b1 >= blo && b1 <= bhi;
-        const uint64_t j0g = sb + (uint64_t)((int64_t)i + dlo + b0);
-        uint32_t d0 = 4u, d1 = 4u;
-        if (act0) d0 = cd.at(j0g);
-        if (act1) d1 = cd.at(j0g + 1);
-        // cell b0
-        int32_t E0 = SW_NEG;
-        uint32_t SE0 = 0;
-        if (act0 && prow && b1 >= pblo && b1 <= pbhi) {
-            const int32_t eo = pH1 + goe, ee = pE1 + ge;
-            if (eo >= ee) { E0 = eo; SE0 = pSH1; } else { E0 = ee; SE0 = pSE1; }
-        }
-        const bool okd0 = act0 && prow && b0 >= pblo && b0 <= pbhi;
-        const int32_t Hd0 = okd0 ? pH0 : 0;
-        const uint32_t SD0 = (Hd0 > 0) ? pSH0 : (uint32_t)r * Bu + (uint32_t)b0;
-        const int32_t Dg0 = Hd0 + dev_pair(qc, d0, match, mismatch);
-        int32_t c0v; uint32_t c0s;
-        if (Dg0 >= E0) { c0v = Dg0; c0s = SD0; } else { c0v = E0; c0s = SE0; }
-        const int32_t H00 = c0v > 0 ? c0v : 0;
-        // cell b1
-        int32_t E1 = SW_NEG;
-        uint32_t SE1 = 0;
-        if (act1 && prow && b1 + 1 >= pblo && b1 + 1 <= pbhi) {
-            const int32_t eo = uH + goe, ee = uE + ge;
-            if (eo >= ee) { E1 = eo; SE1 = uSH; } else { E1 = ee; SE1 = uSE; }
-        }
-        const bool okd1 = act1 && prow && b1 >= pblo && b1 <= pbhi;
-        const int32_t Hd1 = okd1 ? pH1 : 0;
-        const uint32_t SD1 = (Hd1 > 0) ? pSH1 : (uint32_t)r * Bu + (uint32_t)b1;
-        const int32_t Dg1 = Hd1 + dev_pair(qc, d1, match, mismatch);
-        int32_t c1v; uint32_t c1s;
-        if (Dg1 >= E1) { c1v = Dg1; c1s = SD1; } else { c1v = E1; c1s = SE1; }
-        const int32_t H01 = c1v > 0 ? c1v : 0;
-        // horizontal gaps: F(b) = max_{b'<b} X(b') + ge*(b-1), X(b') = H0(b') + go + ge - ge*b'
-        const int32_t x0 = act0 ? H00 + goe - ge * b0 : SW_XNEG;
-        const int32_t x1 = act1 ? H01 + goe - ge * b1 : SW_XNEG;
-        int32_t xv = x1 >= x0 ? x1 : x0;
-        uint32_t xs = x1 >= x0 ? c1s : c0s;
-        scan_pair_max(xv, xs, lane);
-        int32_t ev = __shfl_up_sync(0xffffffffu, xv, 1);
-        uint32_t es = __shfl_up_sync(0xffffffffu, xs, 1);
-        if (lane == 0) { ev = SW_XNEG; es = 0; }
-        const int32_t F0 = (ev > SW_XNEG) ? ev + ge * (b0 - 1) : SW_NEG;
-        const uint32_t SF0 = es;
-        int32_t e1v = ev;
-        uint32_t e1s = es;
-        if (x0 >= e1v) { e1v = x0; e1s = c0s; }
-        const int32_t F1 = (e1v > SW_XNEG) ? e1v + ge * (b1 - 1) : SW_NEG;
-        int32_t H0v, H1v;
-        uint32_t S0, S1;
-        if (H00 >= F0) { H0v = H00; S0 = c0s; } else { H0v = F0; S0 = SF0; }
-        if (H01 >= F1) { H1v = H01; S1 = c1s; } else { H1v = F1; S1 = e1s; }
-        if (act0 && H0v > best) { best = H0v; bi = (int64_t)i; bj = (int64_t)i + dlo + b0; bs = S0; }
-        if (act1 && H1v > best) { best = H1v; bi = (int64_t)i; bj = (int64_t)i + dlo + b1; bs = S1; }
-        pH0 = H0v; pE0 = E0; pSH0 = S0; pSE0 = SE0;
-        pH1 = H1v; pE1 = E1; pSH1 = S1; pSE1 = SE1;
-    }
-}
-
-
 // Band width (diagonals) of an HSP's alignment: the spread of its end diagonals plus 2w + 1.
 __device__ __forceinline__ int64_t dev_band(const DevHsp &h, int32_t w) {
     const int64_t d_s = (int64_t)h.ds - h.qs, d_e = (int64_t)h.de - h.qe;
     return max(d_s, d_e) - min(d_s, d_e) + 2 * (int64_t)w + 1;
 }
 
-// One HSP aligned by a whole warp: the pair path (bands of at most 64 diagonals), or
-// with STRIP the strip path (the band in chunks of 32 offsets, previous row in scratch).
-template <bool STRIP>
-__device__ void sw_task_warp(const DevHsp *__restrict__ sel, uint32_t task, const uint64_t *__restrict__ strip_off,
-                             SwCell *__restrict__ strips, const uint32_t *__restrict__ qpk,
-                             const uint32_t *__restrict__ qnb, const uint64_t *__restrict__ qstart,
-                             const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                             const uint64_t *__restrict__ seq_start, int32_t match, int32_t mismatch, int32_t go,
-                             int32_t ge, int32_t w, DevAln *__restrict__ out, uint32_t *__restrict__ status) {
+// One HSP aligned by a whole warp on the strip path (bands wider than the register paths hold):
+// the band in chunks of 32 offsets, the previous row in scratch.
+__device__ void sw_task_strip(const DevHsp *__restrict__ sel, uint32_t task, const uint64_t *__restrict__ strip_off,
+                              SwCell *__restrict__ strips, const uint32_t *__restrict__ qpk,
+                              const uint32_t *__restrict__ qnb, const uint64_t *__restrict__ qstart,
+                              const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
+                              const uint64_t *__restrict__ seq_start, int32_t match, int32_t mismatch, int32_t go,
+                              int32_t ge, int32_t w, DevAln *__restrict__ out, uint32_t *__restrict__ status) {
     const int lane = threadIdx.x & 31;
     const DevHsp h = sel[task];
     const uint64_t qb = qstart[h.qi], sb = seq_start[h.seq];
@@ -1513,10 +1407,6 @@ __device__ void sw_task_warp(const DevHsp *__restrict__ sel, uint32_t task, cons
     int64_t bi = INT64_MAX, bj = INT64_MAX;
     uint32_t bs = 0;
     const int32_t goe = go + ge;
-    if (!STRIP) {  // bands of at most 64 diagonals (the caller routes wider ones elsewhere)
-        sw_rows_pair(I0, I1, J0, J1, dlo, B, qb, sb, qpk, qnb, bpk, bnb, match, mismatch, goe, ge, lane, best, bi,
-                     bj, bs);
-    } else
     for (int64_t i = I0; i < I1; ++i) {
         const int64_t blo = max((int64_t)0, J0 - i - dlo), bhi = min(B - 1, J1 - 1 - i - dlo);
         if (blo > bhi) continue;
@@ -1599,512 +1489,377 @@ __device__ void sw_task_warp(const DevHsp *__restrict__ sel, uint32_t task, cons
     }
 }
 
-// 32 consecutive bases of a packed sequence starting at a 16-aligned position: 2-bit
-// codes (first base most significant) and non-base flags (bit = offset).
-struct BaseWin {
-    uint64_t p0 = ~0ull, codes = 0;
-    uint32_t bad = 0;
-    __device__ __forceinline__ void load(const uint32_t *__restrict__ pk, const uint32_t *__restrict__ nb, uint64_t p) {
-        p0 = p & ~15ull;
-        const uint64_t w = p0 >> 4;
-        codes = ((uint64_t)pk[w] << 32) | pk[w + 1];
-        const uint64_t v = p0 >> 5;
-        bad = (p0 & 31) ? ((nb[v] >> 16) | (nb[v + 1] << 16)) : nb[v];
-    }
-    // code of base p (p0 <= p < p0 + 32), 4 for a non-base
-    __device__ __forceinline__ uint32_t at(uint64_t p) const {
-        const uint32_t o = (uint32_t)(p - p0);
-        return ((bad >> o) & 1u) ? 4u : (uint32_t)(codes >> (62 - 2 * o)) & 3u;
+// Register path: a segment of G lanes aligns one HSP, lane l of the segment owning K = KA + KB
+// adjacent band offsets with their previous-row states in registers.  Lane l takes row r in
+// iteration r + l, first its KA offsets, then its KB offsets.  The first part needs the same
+// row of the lane to its left (the horizontal gap that runs into it), finished in the iteration
+// before; the last offset of the second part needs the previous row of the lane to its right
+// (the vertical gap), whose first part came earlier in the same iteration.  So every lane works
+// all the time, a row costs two exchanges with neighbours and K cells of the sequential
+// recurrence, and none needs a scan over the lanes.
+//
+// Cells follow the recurrence with its tie rules: E and F open on ties, the diagonal beats E, H0
+// beats F, F extends from the left cell's H0.  A cell outside the DP window is given no match,
+// and that is enough: left of the window and before its first row H stays 0, so gaps out of
+// there are never positive; cells right of it or below feed no cell inside; and a new best
+// always ends in a match (gaps never add, mismatches subtract).
+//
+// Offsets past the band are computed too (G K is rarely the band's width), without matches, and
+// the band's last offset reads E from the first of them.  A path can only leave the band by F,
+// along a row, and come back by E, down a column: j + 1 offsets out and back cost at least
+// goe + (2j + 1) ge more than the way that stays j + 1 rows on its diagonal, which costs at most
+// j + 1 mismatches more.  With mismatch >= 2 ge (the default -3 against -4) that way is at least
+// as good wherever the path comes back, arrives by the diagonal, and so wins ties: nothing
+// from outside is ever chosen.  For other scores (CUT) offsets past the band pass on no E.
+//
+// Bound by instructions: about 27 a cell (each of the four tracked maxima also selects a start
+// cell) on two pipes that take one every other cycle each, and about 20 a row for the exchange
+// and the bases; the window's limits are kept with the bases, as places without a match, and
+// cost instructions only in blocks of 16 rows that meet one.  Measured against the row-by-row
+// path with a scan over the lanes (and its wavefront form for long alignments) that this
+// replaced, band cells of the whole phase: 50,000 alignments (396 M cells) 1.50 -> 0.57 ms,
+// 30,000 (203 M) 1.15 -> 0.31, bands of 257 diagonals (881 M) 2.57 -> 1.04; one alignment of 400
+// rows alone 218 -> 56 us.
+constexpr int SW_SHIFT = 9;  // cells are row << SW_SHIFT | band offset (up to 512 offsets, 2^23 rows)
+constexpr int SW_MAX_BAND = 32 * 9;
+constexpr int64_t SW_MAX_ROWS = 1ll << (32 - SW_SHIFT);
+
+// One HSP's DP window as packed positions: rows [qlo, qhi) of the query, columns [dlo, dhi) of
+// the bank, both inclusive of nothing outside the sequences; offset 0 of row qlo is at diag.
+struct SwGeom {
+    int64_t qlo, qhi, dlo, dhi, diag;
+    int32_t B;
+    __device__ __forceinline__ void set(const DevHsp &h, const uint64_t *__restrict__ qstart,
+                                        const uint64_t *__restrict__ seq_start, int32_t w) {
+        const int64_t qb = (int64_t)qstart[h.qi], sb = (int64_t)seq_start[h.seq];
+        const int64_t m = (int64_t)qstart[h.qi + 1] - qb, L = (int64_t)seq_start[h.seq + 1] - sb;
+        const int64_t d_s = (int64_t)h.ds - h.qs, d_e = (int64_t)h.de - h.qe, d0 = min(d_s, d_e) - w;
+        qlo = qb + max((int64_t)0, (int64_t)h.qs - w);
+        qhi = qb + min(m, (int64_t)h.qe + w);
+        dlo = sb + max((int64_t)0, (int64_t)h.ds - w);
+        dhi = sb + min(L, (int64_t)h.de + w);
+        diag = sb + (qlo - qb) + d0;
+        B = (int32_t)(max(d_s, d_e) + w - d0 + 1);
     }
 };
 
-// 64 consecutive bases [p0, p0 + 64) of a packed sequence (p0 a multiple of 16) that
-// slide forward 16 at a time, with the next 16 bases loaded one slide ahead, so a
-// warp walking rows rarely waits on memory.  All lanes of a segment hold the same
-// window.  Words at or past `end` (the sequence's end) are never read.
-struct SegWin {
-    uint64_t p0 = 0, hi = 0, lo = 0, bad = 0;  // codes of p0..p0+31 (hi) and p0+32..p0+63 (lo); non-base bits
-    uint32_t nxt_pk = 0, nxt_nb = 0;            // the 16 bases after the window (code word, non-base word)
-    __device__ __forceinline__ static uint32_t pk_at(const uint32_t *__restrict__ pk, uint64_t x, uint64_t end) {
-        return x < end ? pk[x >> 4] : 0u;
+// 32 bases from position p (any sign), first one on top, and their non-base bits from bit 0;
+// words outside the array are clamped (their positions lie outside the DP window).
+__device__ __forceinline__ uint64_t window32(const uint32_t *__restrict__ pk, const uint32_t *__restrict__ nb, int64_t p,
+                                             int64_t last_pk, int64_t last_nb, uint32_t &bad) {
+    const int64_t a = p >> 4, b = p >> 5;
+    const uint32_t w0 = pk[max((int64_t)0, min(a, last_pk))], w1 = pk[max((int64_t)0, min(a + 1, last_pk))];
+    const uint32_t w2 = pk[max((int64_t)0, min(a + 2, last_pk))];
+    const uint32_t n0 = nb[max((int64_t)0, min(b, last_nb))], n1 = nb[max((int64_t)0, min(b + 1, last_nb))];
+    const uint32_t s = 2u * (uint32_t)(p & 15);
+    bad = __funnelshift_r(n0, n1, (uint32_t)(p & 31));
+    return (uint64_t)__funnelshift_l(w1, w0, s) << 32 | __funnelshift_l(w2, w1, s);
+}
+
+// Bit i of the low 16 bits of x to bits 31 - 2 i and 30 - 2 i.
+__device__ __forceinline__ uint32_t spread16_down(uint32_t x) {
+    x &= 0xFFFFu;
+    x = (x | x << 8) & 0x00FF00FFu;
+    x = (x | x << 4) & 0x0F0F0F0Fu;
+    x = (x | x << 2) & 0x33333333u;
+    x = (x | x << 1) & 0x55555555u;  // bit 2 i
+    return __brev(x * 3u);
+}
+// Bits [from, to) of 32 positions (any values).
+__device__ __forceinline__ uint32_t positions(int64_t from, int64_t to) {
+    const uint32_t a = (uint32_t)min(max(from, (int64_t)0), (int64_t)32), b = (uint32_t)min(max(to, (int64_t)0), (int64_t)32);
+    const uint32_t lo = __funnelshift_lc(0u, 0xFFFFFFFFu, a), hi = __funnelshift_lc(0u, 0xFFFFFFFFu, b);
+    return lo & ~hi;
+}
+
+// Packed sequences of a search, as the register paths read them.
+struct SwSeqs {
+    const uint32_t *qpk, *qnb, *bpk, *bnb;
+    int64_t last_qpk, last_qnb, last_bpk, last_bnb;  // last words
+};
+
+template <int K>
+struct SwSet {
+    int32_t H[K], E[K];     // previous row: H of each offset, E that it passes to the offset before it
+    uint32_t SH[K], SE[K];  // their start cells
+    int32_t best;           // best cell so far: score, cell of the row after it, start cell
+    uint32_t bcell, bstart;
+    uint32_t cell;          // the row to come's first offset of the lane, as a cell
+    int64_t q, d;           // the row to come: packed position of its query base, of the lane's first bank base
+    uint32_t dw_hi, dw_lo;  // bank bases from d on, first one on top (loaded for 16 rows)
+    uint32_t qw;            // query bases from q on
+    uint32_t dno_hi, dno_lo;  // in the places of dw: no match there (a non-base, or outside the DP window)
+    uint32_t qno;           // the same of q on, a bit each, q's on top
+    uint32_t in_band;       // bit 30 - 2 k: offset inside the band
+    int64_t qlo, qhi, dlo, dhi;
+
+    __device__ __forceinline__ void start(const SwGeom &g, bool on, int b0, int lag) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) { H[k] = 0; E[k] = SW_NEG; SH[k] = SE[k] = 0; }
+        best = 0; bcell = 0xFFFFFFFFu; bstart = 0;
+        cell = (uint32_t)(-lag * (1 << SW_SHIFT) + b0);
+        if (lag == 0) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) SH[k] = cell + (uint32_t)k;
+        }
+        qlo = g.qlo; qhi = on ? g.qhi : g.qlo; dlo = g.dlo; dhi = g.dhi;
+        q = g.qlo - lag;
+        d = g.diag + b0 - lag;
+        const int32_t B = g.B - b0;
+        in_band = !on || B <= 0 ? 0u : B >= K ? 0x55555555u : 0x55555555u & ~(0xFFFFFFFFu >> (2 * B));
     }
-    __device__ __forceinline__ static uint32_t nb_at(const uint32_t *__restrict__ nb, uint64_t x, uint64_t end) {
-        return x < end ? nb[x >> 5] : 0u;
+    // the bases of the 16 rows to come; returns whether dno or qno has a bit that they meet
+    __device__ __forceinline__ bool load(const SwSeqs &s) {
+        uint32_t db, qb;
+        const uint64_t w = window32(s.bpk, s.bnb, d, s.last_bpk, s.last_bnb, db);
+        dw_hi = (uint32_t)(w >> 32);
+        dw_lo = (uint32_t)w;
+        qw = (uint32_t)(window32(s.qpk, s.qnb, q, s.last_qpk, s.last_qnb, qb) >> 32);
+        db |= ~positions(dlo - d, dhi - d);
+        qb = (qb | ~positions(qlo - q, qhi - q)) & 0xFFFFu;
+        db &= (1u << (15 + K)) - 1u;
+        dno_hi = dno_lo = qno = 0;
+        if (db | qb) {
+            dno_hi = spread16_down(db);
+            dno_lo = spread16_down(db >> 16);
+            qno = __brev(qb);
+        }
+        return (db | qb) != 0;
     }
-    __device__ __forceinline__ void prefetch(const uint32_t *__restrict__ pk, const uint32_t *__restrict__ nb,
-                                             uint64_t end) {
-        nxt_pk = pk_at(pk, p0 + 64, end);
-        nxt_nb = nb_at(nb, p0 + 64, end);
+};
+
+// Compares, selects, maxima and logic all issue to one pipe at half rate, and a maximum that
+// also selects a start cell takes three of them.  The multiply-add pipe, as wide, would idle, so
+// additions and the moves of a taken branch are written as multiply-adds by `one` (1, a value
+// the compiler cannot see through): 12 and 15 instructions a cell instead of 27 on one pipe.
+__device__ __forceinline__ int32_t fma_add(int32_t a, int32_t b, int32_t one) {
+    int32_t r;
+    asm("mad.lo.s32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(one), "r"(b));
+    return r;
+}
+// if (x > v) { v = x; s = t; }
+__device__ __forceinline__ void fma_take_gt(int32_t &v, uint32_t &s, int32_t x, uint32_t t, int32_t one) {
+    asm("{ .reg .pred q; setp.gt.s32 q, %2, %0; @q mul.lo.s32 %0, %2, %4; @q mul.lo.s32 %1, %3, %4; }"
+        : "+r"(v), "+r"(s) : "r"(x), "r"(t), "r"(one));
+}
+// if (x >= v) { v = x; s = t; }
+__device__ __forceinline__ void fma_take_ge(int32_t &v, uint32_t &s, int32_t x, uint32_t t, int32_t one) {
+    asm("{ .reg .pred q; setp.ge.s32 q, %2, %0; @q mul.lo.s32 %0, %2, %4; @q mul.lo.s32 %1, %3, %4; }"
+        : "+r"(v), "+r"(s) : "r"(x), "r"(t), "r"(one));
+}
+// if (v <= 0) s = t;
+__device__ __forceinline__ void fma_if_not_pos(uint32_t &s, int32_t v, uint32_t t, int32_t one) {
+    asm("{ .reg .pred q; setp.le.s32 q, %1, 0; @q mul.lo.s32 %0, %2, %3; }" : "+r"(s) : "r"(v), "r"(t), "r"(one));
+}
+// h + (bit ? match : mismatch)
+__device__ __forceinline__ int32_t fma_score(int32_t h, uint32_t bit, int32_t match, int32_t mismatch, int32_t one) {
+    int32_t r;
+    asm("{ .reg .pred q; setp.ne.u32 q, %2, 0; mad.lo.s32 %0, %1, %5, %4; @q mad.lo.s32 %0, %1, %5, %3; }"
+        : "=&r"(r) : "r"(h), "r"(bit), "r"(match), "r"(mismatch), "r"(one));
+    return r;
+}
+// if (h > best) { best = h; cell = c; start = t; }
+__device__ __forceinline__ void fma_best(int32_t &best, uint32_t &cell, uint32_t &start, int32_t h, uint32_t c, uint32_t t,
+                                         int32_t one) {
+    asm("{ .reg .pred q; setp.gt.s32 q, %3, %0; @q mul.lo.s32 %0, %3, %6; @q mul.lo.s32 %1, %4, %6;"
+        " @q mul.lo.s32 %2, %5, %6; }"
+        : "+r"(best), "+r"(cell), "+r"(start) : "r"(h), "r"(c), "r"(t), "r"(one));
+}
+
+struct SwScore {
+    int32_t match, mismatch, goe, ge, one;
+};
+
+// Cell k of the row: E and F run into it (SE, SF: their start cells); leaves the cell's H, the E
+// that it passes to the offset before it and, in F, the one for the offset after it.
+// bit 30 - 2 k of eq: two equal bases.
+template <int K, bool CUT>
+__device__ __forceinline__ void sw_cell(SwSet<K> &x, int k, uint32_t eq, int32_t E, uint32_t SE, int32_t &F, uint32_t &SF,
+                                        const SwScore &c) {
+    const uint32_t below = x.cell + (uint32_t)k;  // the cell a row on: the start after H = 0
+    int32_t cv = fma_score(x.H[k], eq & (1u << (30 - 2 * k)), c.match, c.mismatch, c.one);  // the diagonal beats E
+    uint32_t C = x.SH[k];
+    fma_take_gt(cv, C, E, SE, c.one);
+    fma_if_not_pos(C, cv, below, c.one);
+    const int32_t H0 = max(cv, 0);
+    const bool ph = H0 >= F;  // H0 beats F
+    const int32_t H = max(H0, F);
+    const uint32_t S = ph ? C : SF;
+    fma_best(x.best, x.bcell, x.bstart, H, below, S, c.one);
+    x.H[k] = H;
+    x.SH[k] = S;
+    // open beats extend
+    const int32_t eo = fma_add(H, c.goe, c.one), ee = fma_add(E, c.ge, c.one);
+    x.E[k] = max(eo, ee);
+    x.SE[k] = eo >= ee ? S : SE;
+    if (CUT && !(x.in_band & (1u << (30 - 2 * k)))) x.E[k] = SW_NEG;
+    const int32_t fo = fma_add(H0, c.goe, c.one);
+    F = fma_add(F, c.ge, c.one);
+    fma_take_ge(F, SF, fo, C, c.one);
+}
+
+// The row's equal bases (bit 30 - 2 k: offset k, inside the band and the DP window) and the step
+// to the next row.  NO: dno and qno have bits.
+template <int K, bool NO>
+__device__ __forceinline__ uint32_t sw_next_row(SwSet<K> &x) {
+    const uint32_t y = ~(x.dw_hi ^ ((x.qw >> 30) * 0x55555555u));
+    uint32_t eq = y & (y >> 1) & x.in_band;
+    if (NO) {
+        eq &= ~(x.dno_hi | (uint32_t)((int32_t)x.qno >> 31));
+        x.dno_hi = __funnelshift_l(x.dno_lo, x.dno_hi, 2);
+        x.dno_lo <<= 2;
+        x.qno <<= 1;
     }
-    __device__ __forceinline__ void init(const uint32_t *__restrict__ pk, const uint32_t *__restrict__ nb, uint64_t p,
-                                         uint64_t end) {
-        p0 = p & ~15ull;
-        hi = ((uint64_t)pk_at(pk, p0, end) << 32) | pk_at(pk, p0 + 16, end);
-        lo = ((uint64_t)pk_at(pk, p0 + 32, end) << 32) | pk_at(pk, p0 + 48, end);
-        // bit o = base p0 + o; words of 32 bases hold p0 at bit 0 or at bit 16
-        if (p0 & 16) {
-            bad = ((uint64_t)nb_at(nb, p0, end) >> 16) | ((uint64_t)nb_at(nb, p0 + 16, end) << 16) |
-                  ((uint64_t)nb_at(nb, p0 + 48, end) << 48);
+    x.dw_hi = __funnelshift_l(x.dw_lo, x.dw_hi, 2);
+    x.dw_lo *= 4u;
+    x.qw *= 4u;
+    x.cell += 1u << SW_SHIFT;
+    return eq;
+}
+
+// One iteration: the lane's next row.  F1, SF1: the F that its last row passes to the right.
+// CUT: offsets past the band must not reach back into it (else the scores see to that).
+template <int G, int KA, int KB, bool NO, bool CUT>
+__device__ __forceinline__ void sw_row(SwSet<KA + KB> &x, int32_t &F1, uint32_t &SF1, int sl, const SwScore &c) {
+    constexpr int K = KA + KB;
+    int32_t F = __shfl_up_sync(0xffffffffu, F1, 1);
+    uint32_t SF = __shfl_up_sync(0xffffffffu, SF1, 1);
+    if (sl == 0) F = SW_NEG;
+    const uint32_t eq = sw_next_row<K, NO>(x);
+#pragma unroll
+    for (int k = 0; k < KA; ++k) sw_cell<K, CUT>(x, k, eq, x.E[k + 1], x.SE[k + 1], F, SF, c);
+    int32_t uE = __shfl_down_sync(0xffffffffu, x.E[0], 1);
+    const uint32_t uSE = __shfl_down_sync(0xffffffffu, x.SE[0], 1);
+    if (sl == G - 1) uE = SW_NEG;
+#pragma unroll
+    for (int k = KA; k < K; ++k)
+        sw_cell<K, CUT>(x, k, eq, k + 1 < K ? x.E[k + 1] : uE, k + 1 < K ? x.SE[k + 1] : uSE, F, SF, c);
+    F1 = F;
+    SF1 = SF;
+}
+
+// Highest score, then first cell, over the G lanes of a segment; the alignment it stands for.
+template <int G>
+__device__ __forceinline__ void sw_finish(int32_t best, uint32_t cell, uint32_t start, const DevHsp &h, bool on, int32_t w,
+                                          DevAln &res) {
+#pragma unroll
+    for (int d = G / 2; d > 0; d >>= 1) {
+        const int32_t ob = __shfl_xor_sync(0xffffffffu, best, d);
+        const uint32_t oc = __shfl_xor_sync(0xffffffffu, cell, d), os = __shfl_xor_sync(0xffffffffu, start, d);
+        if (ob > best || (ob == best && oc < cell)) { best = ob; cell = oc; start = os; }
+    }
+    res.qi = h.qi; res.seq = h.seq; res.qs = res.qe = res.ds = res.de = 0; res.score = 0; res.pad = 0;
+    if (on && best > 0) {
+        const uint32_t bm = (1u << SW_SHIFT) - 1u;
+        const int64_t d_s = (int64_t)h.ds - h.qs, d_e = (int64_t)h.de - h.qe, dlo = min(d_s, d_e) - w;
+        const int64_t I0 = max((int64_t)0, (int64_t)h.qs - w);
+        const int64_t i1 = I0 + (cell >> SW_SHIFT) - 1, i0 = I0 + (start >> SW_SHIFT);  // cell: a row on
+        res.qs = (uint32_t)i0; res.qe = (uint32_t)(i1 + 1);
+        res.ds = (uint32_t)(i0 + dlo + (start & bm)); res.de = (uint32_t)(i1 + dlo + (cell & bm) + 1);
+        res.score = best;
+    }
+}
+
+// Aligns each segment's HSP h (where on; a band of at most G K offsets, at most SW_MAX_ROWS
+// rows); every lane of the segment gets the alignment.
+template <int G, int KA, int KB, bool CUT>
+__device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const SwSeqs &q, const uint64_t *__restrict__ qstart,
+                                        const uint64_t *__restrict__ seq_start, const SwScore &c, int32_t w, DevAln &res) {
+    const int sl = (threadIdx.x & 31) % G;
+    constexpr int K = KA + KB;
+    SwSet<K> x;
+    int32_t T = 0;
+    {
+        SwGeom g{};
+        if (on) {
+            g.set(h, qstart, seq_start, w);
+            T = (int32_t)max(g.qhi - g.qlo, (int64_t)0) + (g.B - 1) / K;
+        }
+        x.start(g, on, K * sl, sl);
+    }
+    if (G < 32) T = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)T);
+    int32_t F1 = SW_NEG;
+    uint32_t SF1 = 0;
+    for (int32_t t0 = 0; t0 < T; t0 += 16) {
+        const bool no = __any_sync(0xffffffffu, x.load(q));
+        x.q += 16; x.d += 16;
+        const int32_t t1 = min(t0 + 16, T);
+        if (no) {
+#pragma unroll 1
+            for (int32_t t = t0; t < t1; ++t) sw_row<G, KA, KB, true, CUT>(x, F1, SF1, sl, c);
         } else {
-            bad = (uint64_t)nb_at(nb, p0, end) | ((uint64_t)nb_at(nb, p0 + 32, end) << 32);
+#pragma unroll 1
+            for (int32_t t = t0; t < t1; ++t) sw_row<G, KA, KB, false, CUT>(x, F1, SF1, sl, c);
         }
-        prefetch(pk, nb, end);
     }
-    __device__ __forceinline__ void advance(const uint32_t *__restrict__ pk, const uint32_t *__restrict__ nb,
-                                            uint64_t end) {
-        const uint64_t q = p0 + 64;
-        hi = (hi << 32) | (lo >> 32);
-        lo = (lo << 32) | nxt_pk;
-        bad = (bad >> 16) | ((uint64_t)((nxt_nb >> (q & 16)) & 0xFFFFu) << 48);
-        p0 += 16;
-        prefetch(pk, nb, end);
-    }
-    // code of base p (p0 <= p < p0 + 64), 4 for a non-base
-    __device__ __forceinline__ uint32_t at(uint64_t p) const {
-        const uint32_t o = (uint32_t)(p - p0);
-        const uint32_t c = (uint32_t)((o < 32 ? hi : lo) >> (62 - 2 * (o & 31))) & 3u;
-        return ((bad >> o) & 1ull) ? 4u : c;
-    }
-};
-
-// Codes of the bases at offsets o, o + 1, ... of a window from the top of a 64-bit
-// word (2 bits each; -31 <= o < 64, offsets outside the window read as 0), and their
-// non-base bits from bit 0.
-__device__ __forceinline__ uint64_t segwin_codes(const SegWin &wn, int32_t o) {
-    if (o < 0) return wn.hi >> (2 * -o);
-    if (o == 0) return wn.hi;
-    if (o < 32) return (wn.hi << (2 * o)) | (wn.lo >> (64 - 2 * o));
-    return wn.lo << (2 * (o - 32));
-}
-__device__ __forceinline__ uint32_t segwin_bad(const SegWin &wn, int32_t o) {
-    return o < 0 ? (uint32_t)(wn.bad << -o) : (uint32_t)(wn.bad >> o);
+    sw_finish<G>(x.best, x.bcell, x.bstart, h, on, w, res);
 }
 
-// Code of the base at offset o (0 <= o < 64) of a window, 4 for a non-base.
-__device__ __forceinline__ uint32_t segwin_code(const SegWin &wn, uint32_t o) {
-    const uint32_t word = o < 32 ? (o < 16 ? (uint32_t)(wn.hi >> 32) : (uint32_t)wn.hi)
-                                 : (o < 48 ? (uint32_t)(wn.lo >> 32) : (uint32_t)wn.lo);
-    const uint32_t c = (word >> (30 - 2 * (o & 15))) & 3u;
-    const uint32_t badw = o < 32 ? (uint32_t)wn.bad : (uint32_t)(wn.bad >> 32);
-    return ((badw >> (o & 31)) & 1u) ? 4u : c;
-}
-
-// 32 / G HSPs per warp: segment s (lanes sG .. sG + G - 1) aligns its own HSP, lane l of
-// the segment owns band offsets K l .. K l + K - 1 and keeps their previous-row states
-// in registers.  All segments step through rows together.  The vertical-gap input of
-// offset b is offset b + 1 of the previous row (own state, or the next lane's first
-// offset); horizontal gaps come from a segmented warp max-scan as in the pair path.
-// A cell outside the DP region keeps H = 0 and E = -inf as its state, so the next row
-// reads its neighbours without range checks: a neutral neighbour yields only E <= 0 and
-// a diagonal from H = 0, neither of which can raise a score (an alignment may begin at
-// any cell); a per-row bit mask of the lane's cells in the region masks the stored
-// state and the best cell.  Every tracked maximum is a DPX max with its predicate
-// (__vibmax_s32: the first operand wins ties), which also selects the start cell.
-// Returns with handled = false (and computes nothing) for an HSP whose band exceeds G K
-// offsets.
-template <int G, int K>
-__device__ __forceinline__ void sw_group(bool valid, const DevHsp &h, const uint32_t *__restrict__ qpk,
-                                         const uint32_t *__restrict__ qnb, const uint64_t *__restrict__ qstart,
-                                         const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                                         const uint64_t *__restrict__ seq_start, int32_t match, int32_t mismatch,
-                                         int32_t goe, int32_t ge, int32_t w, bool &handled, DevAln &res) {
-    const int lane = threadIdx.x & 31, sl = lane % G;
-    int64_t I0 = 0, I1 = 0, J0 = 0, J1 = 0, dlo = 0, B = 0;
-    uint64_t qb = 0, sb = 0, qend = 0, send = 0;
-    if (valid) {
-        qb = qstart[h.qi];
-        sb = seq_start[h.seq];
-        qend = qstart[h.qi + 1];
-        send = seq_start[h.seq + 1];
-        const int64_t m = (int64_t)(qend - qb), L = (int64_t)(send - sb);
-        const int64_t d_s = (int64_t)h.ds - h.qs, d_e = (int64_t)h.de - h.qe;
-        dlo = min(d_s, d_e) - w;
-        B = max(d_s, d_e) + w - dlo + 1;
-        I0 = max((int64_t)0, (int64_t)h.qs - w);
-        I1 = min(m, (int64_t)h.qe + w);
-        J0 = max((int64_t)0, (int64_t)h.ds - w);
-        J1 = min(L, (int64_t)h.de + w);
-    }
-    handled = valid && B <= G * K && I1 - I0 <= 65535;
-    const int32_t rows = handled ? (int32_t)(I1 - I0) : 0;
-    const int32_t max_rows = __reduce_max_sync(0xffffffffu, (uint32_t)rows);
-    const int32_t jlo = (int32_t)(J0 - I0 - dlo), jhi = (int32_t)(J1 - 1 - I0 - dlo);
-    const int32_t Bm1 = (int32_t)B - 1;
-    const int32_t b0 = K * sl;
-    // per-offset constants: X(b) = H0(b) + cX[k], F(b) = max_{b' < b} X(b') + cF[k]
-    int32_t cX[K], cF[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        cX[k] = goe - ge * (b0 + k);
-        cF[k] = ge * (b0 + k - 1);
-    }
-    int32_t pH[K], pE[K];
-    uint32_t pSH[K], pSE[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) { pH[k] = 0; pE[k] = SW_NEG; pSH[k] = 0; pSE[k] = 0; }
-    int32_t best = 0;
-    uint32_t bpos = 0xFFFFFFFFu, bs = 0;  // best cell: row << 16 | band offset, and its start cell
-    // bases: one 64-base window per segment (bands of up to 49 diagonals), else a
-    // 32-base window per lane
-    constexpr bool SEG = G * K <= 49;
-    BaseWin wq, wd;
-    SegWin sq, sd;
-    if (SEG && handled) {
-        sq.init(qpk, qnb, qb + (uint64_t)I0, qend);
-        sd.init(bpk, bnb, sb + (uint64_t)max(I0 + dlo, J0), send);
-    }
-    for (int32_t r = 0; r < max_rows; ++r) {
-        const bool seg_on = r < rows;
-        const int32_t blo = max(0, jlo - r), bhi = min(Bm1, jhi - r);
-        // the lane's offsets b0 + k inside [blo, bhi]
-        const int32_t klo = max(blo - b0, 0), khi = min(bhi - b0, K - 1);
-        const uint32_t amask = (seg_on && klo <= khi) ? ((2u << khi) - 1u) & ~((1u << klo) - 1u) : 0u;
-        const bool lane_on = amask != 0u;
-        // previous-row state of offset K (sl + 1) (the next lane's first offset); the last lane's
-        // is beyond the band
-        int32_t uH = __shfl_down_sync(0xffffffffu, pH[0], 1, G), uE = __shfl_down_sync(0xffffffffu, pE[0], 1, G);
-        const uint32_t uSH = __shfl_down_sync(0xffffffffu, pSH[0], 1, G);
-        const uint32_t uSE = __shfl_down_sync(0xffffffffu, pSE[0], 1, G);
-        if (sl == G - 1) { uH = 0; uE = SW_NEG; }
-        uint32_t qc = 4u;
-        const uint64_t i = (uint64_t)(I0 + r);
-        const uint64_t jb = sb + (uint64_t)((int64_t)i + dlo + b0);  // bank position of offset b0
-        if (SEG) {
-            if (seg_on) {  // the same in every lane of the segment
-                if (qb + i >= sq.p0 + 64) sq.advance(qpk, qnb, qend);
-                const uint64_t jhi_pos = sb + (uint64_t)min((int64_t)i + dlo + B - 1, J1 - 1);
-                if (jhi_pos >= sd.p0 + 64) sd.advance(bpk, bnb, send);
-                if (lane_on) qc = sq.at(qb + i);
-            }
-        } else if (lane_on) {
-            if (i + qb < wq.p0 || i + qb >= wq.p0 + 32) wq.load(qpk, qnb, qb + i);
-            qc = wq.at(qb + i);
-            const uint64_t jfirst = jb + (uint64_t)max(0, blo - b0), jlast = jb + (uint64_t)min(K - 1, bhi - b0);
-            if (jfirst < wd.p0 || jlast >= wd.p0 + 32) wd.load(bpk, bnb, jfirst);
-        }
-        // the lane's K bank bases (window offsets o0 .. o0 + K - 1; o0 >= -(K - 1))
-        uint64_t dcodes = 0;
-        uint32_t dbad = 0;
-        if (SEG && lane_on) {
-            const int32_t o0 = (int32_t)((int64_t)jb - (int64_t)sd.p0);
-            dcodes = segwin_codes(sd, o0);
-            dbad = segwin_bad(sd, o0);
-        }
-        // bit k: offset b0 + k pairs two equal bases (the row's query base against the K codes)
-        uint32_t dm = 0;
-        if (SEG && lane_on && qc < 4u) {
-            const uint32_t x = ~((uint32_t)(dcodes >> 32) ^ (qc * 0x55555555u)), eq = x & (x >> 1);
-#pragma unroll
-            for (int k = 0; k < K; ++k) dm |= ((eq >> (30 - 2 * k)) & 1u) << k;
-            dm &= ~dbad;
-        }
-        const uint32_t rowbase = (uint32_t)r << 16;
-        int32_t H0[K], E[K], X[K];
-        uint32_t C[K], SE[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            // vertical gap from offset b + 1 of the previous row: open wins ties
-            const int32_t vH = k + 1 < K ? pH[k + 1] : uH, vE = k + 1 < K ? pE[k + 1] : uE;
-            const uint32_t vSH = k + 1 < K ? pSH[k + 1] : uSH, vSE = k + 1 < K ? pSE[k + 1] : uSE;
-            bool po;
-            E[k] = __vibmax_s32(vH + goe, vE + ge, &po);
-            SE[k] = po ? vSH : vSE;
-            // diagonal: from the previous row's H, or a start here
-            const int32_t Hd = pH[k];
-            const uint32_t SD = Hd > 0 ? pSH[k] : rowbase | (uint32_t)(b0 + k);
-            bool same;
-            if (SEG) {
-                same = (dm >> k) & 1u;
-            } else {
-                const uint32_t d = ((amask >> k) & 1u) ? wd.at(jb + k) : 4u;  // the window covers the active cells only
-                same = qc < 4u && d == qc;
-            }
-            const int32_t Dg = Hd + (same ? match : mismatch);
-            // diagonal over E on ties
-            bool pd;
-            const int32_t cv = __vibmax_s32(Dg, E[k], &pd);
-            C[k] = pd ? SD : SE[k];
-            H0[k] = max(cv, 0);
-            X[k] = H0[k] + cX[k];
-        }
-        // lane aggregate of X (later offsets win ties), then the segmented scan over lanes
-        int32_t xv = X[0];
-        uint32_t xs = C[0];
-#pragma unroll
-        for (int k = 1; k < K; ++k) {
-            bool p;
-            xv = __vibmax_s32(X[k], xv, &p);
-            xs = p ? C[k] : xs;
-        }
-#pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-            const int32_t ov = __shfl_up_sync(0xffffffffu, xv, o, G);
-            const uint32_t os = __shfl_up_sync(0xffffffffu, xs, o, G);
-            bool p;
-            xv = __vibmax_s32(xv, sl >= o ? ov : SW_XNEG, &p);
-            xs = p ? xs : os;
-        }
-        int32_t ev = __shfl_up_sync(0xffffffffu, xv, 1, G);
-        uint32_t es = __shfl_up_sync(0xffffffffu, xs, 1, G);
-        if (sl == 0) { ev = SW_XNEG; es = 0; }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            // H0 over F on ties
-            bool ph;
-            const int32_t Hv = __vibmax_s32(H0[k], ev + cF[k], &ph);
-            const uint32_t S = ph ? C[k] : es;
-            bool px;
-            ev = __vibmax_s32(X[k], ev, &px);
-            es = px ? C[k] : es;
-            const bool act = (amask >> k) & 1u;
-            const int32_t Hm = act ? Hv : 0;
-            if (Hm > best) { best = Hm; bpos = rowbase | (uint32_t)(b0 + k); bs = S; }
-            pH[k] = Hm; pE[k] = act ? E[k] : SW_NEG; pSH[k] = S; pSE[k] = SE[k];
-        }
-    }
-    // segment reduction: highest score, then smallest row, then smallest offset (smallest j)
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        const int32_t ob = __shfl_down_sync(0xffffffffu, best, o, G);
-        const uint32_t op = __shfl_down_sync(0xffffffffu, bpos, o, G);
-        const uint32_t os = __shfl_down_sync(0xffffffffu, bs, o, G);
-        if (ob > best || (ob == best && op < bpos)) { best = ob; bpos = op; bs = os; }
-    }
-    res.qi = h.qi; res.seq = h.seq; res.qs = res.qe = res.ds = res.de = 0; res.score = 0; res.pad = 0;
-    if (handled && best > 0) {
-        const int64_t bi = I0 + (int64_t)(bpos >> 16), bj = bi + dlo + (int64_t)(bpos & 0xFFFFu);
-        const int64_t i0 = I0 + (int64_t)(bs >> 16), j0 = i0 + dlo + (int64_t)(bs & 0xFFFFu);
-        res.qs = (uint32_t)i0; res.qe = (uint32_t)(bi + 1);
-        res.ds = (uint32_t)j0; res.de = (uint32_t)(bj + 1);
-        res.score = best;
-    }
-}
-
-// One HSP with a band of at most 64 diagonals on anti-diagonal wavefronts, for the
-// longest alignments, whose row-by-row chains would otherwise bound the kernel's time.
-// Cell (r, b) (row I0 + r, band offset b) lies on wavefront t = 2r + b; its diagonal
-// input (r - 1, b) is on t - 2, its vertical input (r - 1, b + 1) and horizontal input
-// (r, b - 1) on t - 1.  Lane l owns offsets 2l and 2l + 1 and computes one of them per
-// wavefront (offset 2l on even t, 2l + 1 on odd t), so each wavefront takes one
-// shuffle step and a short chain of operations instead of a row's scan.  Each cell
-// follows the sequential recurrence with its tie rules: E and F open on ties, the
-// diagonal beats E, H0 beats F; F extends from the left cell's H0 (as the row scan
-// does).  The best cell is the highest score, then the smallest row, then the
-// smallest offset.  Start cells are (row - I0) * B + offset.
-struct WaveCell {
-    int32_t H, E, H0, F;
-    uint32_t SH, SE, C, SF;
-};
-
-__device__ __forceinline__ void sw_wave(const DevHsp &h, const uint32_t *__restrict__ qpk,
-                                        const uint32_t *__restrict__ qnb, const uint64_t *__restrict__ qstart,
-                                        const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                                        const uint64_t *__restrict__ seq_start, int32_t match, int32_t mismatch,
-                                        int32_t goe, int32_t ge, int32_t w, DevAln &res) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t qb = qstart[h.qi], sb = seq_start[h.seq], qend = qstart[h.qi + 1], send = seq_start[h.seq + 1];
-    const int64_t m = (int64_t)(qend - qb), L = (int64_t)(send - sb);
-    const int64_t d_s = (int64_t)h.ds - h.qs, d_e = (int64_t)h.de - h.qe;
-    const int64_t dlo = min(d_s, d_e) - w;
-    const int32_t B = (int32_t)(max(d_s, d_e) + w - dlo + 1);
-    const int64_t I0 = max((int64_t)0, (int64_t)h.qs - w), I1 = min(m, (int64_t)h.qe + w);
-    const int64_t J0 = max((int64_t)0, (int64_t)h.ds - w), J1 = min(L, (int64_t)h.de + w);
-    const int32_t rows = (int32_t)max(I1 - I0, (int64_t)0);
-    const int32_t jlo = (int32_t)(J0 - I0 - dlo), jhi = (int32_t)(J1 - 1 - I0 - dlo);
-    // rows r where offset e is a cell of the window: max(0, jlo - e) <= r <= min(rows - 1, jhi - e)
-    const int32_t b0 = 2 * lane, b1 = 2 * lane + 1;
-    auto lo_of = [&](int32_t e) { return (e >= 0 && e < B) ? max(0, jlo - e) : INT32_MAX; };
-    auto hi_of = [&](int32_t e) { return (e >= 0 && e < B) ? min(rows - 1, jhi - e) : -1; };
-    const int32_t lo_m = lo_of(b0 - 1), hi_m = hi_of(b0 - 1), lo_0 = lo_of(b0), hi_0 = hi_of(b0);
-    const int32_t lo_1 = lo_of(b1), hi_1 = hi_of(b1), lo_2 = lo_of(b1 + 1), hi_2 = hi_of(b1 + 1);
-    WaveCell c0, c1;  // the lane's last cells at offsets 2l and 2l + 1
-    c0.H = c1.H = 0; c0.E = c1.E = SW_NEG; c0.H0 = c1.H0 = 0; c0.F = c1.F = SW_NEG;
-    c0.SH = c1.SH = c0.SE = c1.SE = c0.C = c1.C = c0.SF = c1.SF = 0;
-    bool v0 = false, v1 = false;  // cells (r - 1, 2l) and (r - 1, 2l + 1) were in the window
-    int32_t best = 0, br = INT32_MAX, bb = INT32_MAX;
-    uint32_t bs = 0;
-    SegWin sq, sd;
-    sq.init(qpk, qnb, qb + (uint64_t)I0, qend);
-    sd.init(bpk, bnb, sb + (uint64_t)max(I0 + dlo, J0), send);
-    // window offsets of this lane's bases at iteration k = t / 2 (row r = k - l): query
-    // base I0 + r, bank base I0 + dlo + r + 2l (offset 2l; 2l + 1 is the next one)
-    int32_t oq = (int32_t)((int64_t)(qb + (uint64_t)I0) - (int64_t)sq.p0) - lane;
-    int32_t od = (int32_t)((int64_t)sb + I0 + dlo - (int64_t)sd.p0) + lane;
-    int32_t qmax = (int32_t)((int64_t)(qb + (uint64_t)I0) - (int64_t)sq.p0);  // lane 0's query offset
-    // last bank offset the wavefront pair t, t + 1 reads: I0 + dlo + (t + B) / 2, at most J1 - 1
-    const int64_t dmax0 = (int64_t)sb + I0 + dlo - (int64_t)sd.p0;
-    const int64_t dcap = (int64_t)sb + J1 - 1 - (int64_t)sd.p0;
-    int32_t dshift = 0;  // 16 x the bank window's advances
-    uint32_t rB = (uint32_t)(-lane) * (uint32_t)B;  // r * B (start cells)
-    const int32_t T = rows > 0 ? 2 * rows + B - 2 : 0;  // wavefronts 0 .. T - 1
-    for (int32_t t = 0, r = -lane; t < T; t += 2, ++r, ++oq, ++od, ++qmax, rB += (uint32_t)B) {
-        if (qmax >= 64) { sq.advance(qpk, qnb, qend); oq -= 16; qmax -= 16; }
-        if (min(dmax0 + (t + B) / 2, dcap) - dshift >= 64) { sd.advance(bpk, bnb, send); od -= 16; dshift += 16; }
-        const uint32_t qc = (r >= 0 && r < rows) ? segwin_code(sq, (uint32_t)oq) : 4u;
-        // even wavefront t: cell (r, 2l); left (r, 2l - 1) is lane l - 1's, from wavefront t - 1
-        {
-            const int32_t lH0 = __shfl_up_sync(0xffffffffu, c1.H0, 1), lF = __shfl_up_sync(0xffffffffu, c1.F, 1);
-            const uint32_t lC = __shfl_up_sync(0xffffffffu, c1.C, 1), lSF = __shfl_up_sync(0xffffffffu, c1.SF, 1);
-            const bool cv = r >= lo_0 && r <= hi_0;
-            int32_t E = SW_NEG;
-            uint32_t SE = 0;
-            if (cv && v1) {  // up-right (r - 1, 2l + 1): own, from wavefront t - 1
-                const int32_t eo = c1.H + goe, ee = c1.E + ge;
-                if (eo >= ee) { E = eo; SE = c1.SH; } else { E = ee; SE = c1.SE; }
-            }
-            const int32_t Hd = (cv && v0) ? c0.H : 0;
-            const uint32_t SD = Hd > 0 ? c0.SH : rB + (uint32_t)b0;
-            const int32_t sc = cv ? dev_pair(qc, segwin_code(sd, (uint32_t)od), match, mismatch) : mismatch;
-            const int32_t Dg = Hd + sc;
-            int32_t cand;
-            uint32_t C;
-            if (Dg >= E) { cand = Dg; C = SD; } else { cand = E; C = SE; }
-            const int32_t H0 = cand > 0 ? cand : 0;
-            int32_t F = SW_NEG;
-            uint32_t SF = 0;
-            if (cv && r >= lo_m && r <= hi_m) {
-                const int32_t fo = lH0 + goe, fe = lF + ge;
-                if (fo >= fe) { F = fo; SF = lC; } else { F = fe; SF = lSF; }
-            }
-            int32_t H;
-            uint32_t SH;
-            if (H0 >= F) { H = H0; SH = C; } else { H = F; SH = SF; }
-            // cells of one lane come in row-major order: the first maximum wins
-            if (cv && H > best) { best = H; br = r; bb = b0; bs = SH; }
-            c0.H = H; c0.E = E; c0.H0 = H0; c0.F = F; c0.SH = SH; c0.SE = SE; c0.C = C; c0.SF = SF;
-            v0 = cv;
-        }
-        // odd wavefront t + 1: cell (r, 2l + 1); up-right (r - 1, 2l + 2) is lane l + 1's, from wavefront t
-        {
-            const int32_t uH = __shfl_down_sync(0xffffffffu, c0.H, 1), uE = __shfl_down_sync(0xffffffffu, c0.E, 1);
-            const uint32_t uSH = __shfl_down_sync(0xffffffffu, c0.SH, 1), uSE = __shfl_down_sync(0xffffffffu, c0.SE, 1);
-            const bool cv = r >= lo_1 && r <= hi_1;
-            int32_t E = SW_NEG;
-            uint32_t SE = 0;
-            if (cv && r - 1 >= lo_2 && r - 1 <= hi_2) {
-                const int32_t eo = uH + goe, ee = uE + ge;
-                if (eo >= ee) { E = eo; SE = uSH; } else { E = ee; SE = uSE; }
-            }
-            const int32_t Hd = (cv && v1) ? c1.H : 0;
-            const uint32_t SD = Hd > 0 ? c1.SH : rB + (uint32_t)b1;
-            const int32_t sc = cv ? dev_pair(qc, segwin_code(sd, (uint32_t)od + 1u), match, mismatch) : mismatch;
-            const int32_t Dg = Hd + sc;
-            int32_t cand;
-            uint32_t C;
-            if (Dg >= E) { cand = Dg; C = SD; } else { cand = E; C = SE; }
-            const int32_t H0 = cand > 0 ? cand : 0;
-            int32_t F = SW_NEG;
-            uint32_t SF = 0;
-            if (cv && v0) {  // left (r, 2l): own, just computed
-                const int32_t fo = c0.H0 + goe, fe = c0.F + ge;
-                if (fo >= fe) { F = fo; SF = c0.C; } else { F = fe; SF = c0.SF; }
-            }
-            int32_t H;
-            uint32_t SH;
-            if (H0 >= F) { H = H0; SH = C; } else { H = F; SH = SF; }
-            if (cv && H > best) { best = H; br = r; bb = b1; bs = SH; }
-            c1.H = H; c1.E = E; c1.H0 = H0; c1.F = F; c1.SH = SH; c1.SE = SE; c1.C = C; c1.SF = SF;
-            v1 = cv;
-        }
-    }
-    // highest score, then smallest row, then smallest offset
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int32_t ob = __shfl_down_sync(0xffffffffu, best, o);
-        const int32_t orr = __shfl_down_sync(0xffffffffu, br, o), obb = __shfl_down_sync(0xffffffffu, bb, o);
-        const uint32_t os = __shfl_down_sync(0xffffffffu, bs, o);
-        if (ob > best || (ob == best && (orr < br || (orr == br && obb < bb)))) { best = ob; br = orr; bb = obb; bs = os; }
-    }
-    res.qi = h.qi; res.seq = h.seq; res.qs = res.qe = res.ds = res.de = 0; res.score = 0; res.pad = 0;
-    if (best > 0) {
-        const int64_t bi = I0 + br, bj = bi + dlo + bb;
-        const int64_t i0 = I0 + (int64_t)(bs / (uint32_t)B), j0 = i0 + dlo + (int64_t)(bs % (uint32_t)B);
-        res.qs = (uint32_t)i0; res.qe = (uint32_t)(bi + 1);
-        res.ds = (uint32_t)j0; res.de = (uint32_t)(bj + 1);
-        res.score = best;
-    }
-}
-
-// Warps take 32 / SWG_G selected HSPs at a time; each segment of SWG_G lanes aligns one
-// whose band fits SWG_G x SWG_K offsets, and the whole warp then aligns the others one by
-// one (pair or strip path).
-// SWG_G lanes per HSP (32 / SWG_G HSPs per warp), SWG_K band offsets per lane: <8, 5>
-// (bands of up to 40 diagonals, the default), <16, 3> (48) or <32, 2> (64).
-template <int SWG_G, int SWG_K>
-__global__ void __launch_bounds__(128, 1) k_banded_sw(const DevHsp *__restrict__ sel, uint32_t n,
-                                                   const uint64_t *__restrict__ strip_off, SwCell *__restrict__ strips,
-                                                   const uint32_t *__restrict__ qpk, const uint32_t *__restrict__ qnb,
+// Alignments of the selected HSPs, longest first (order): the first n_long tasks a warp each
+// (32 lanes with two offsets: the shortest rows, for the alignments that would bound the
+// kernel's time), the others 32 / G to a warp.  Bands over 64 diagonals (and windows of
+// SW_MAX_ROWS rows) go to the list that k_banded_sw_wide takes.  <8, 3, 2> covers bands of up to
+// 40 diagonals (33 and up at the default width), <16, 2, 1> 48; k_sw_prepare counts tasks with
+// wider bands, up to 64, among the long ones.
+template <int G, int KA, int KB, bool CUT>
+__global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ sel, uint32_t n, SwSeqs q,
                                                    const uint64_t *__restrict__ qstart,
-                                                   const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                                                   const uint64_t *__restrict__ seq_start, int32_t match,
-                                                   int32_t mismatch, int32_t go, int32_t ge, int32_t w,
+                                                   const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
                                                    uint32_t *__restrict__ next_task, const uint64_t *__restrict__ order,
                                                    uint32_t *__restrict__ wide, uint32_t *__restrict__ wide_count,
                                                    const uint32_t *__restrict__ n_long, uint32_t *__restrict__ next_long,
-                                                   DevAln *__restrict__ out, uint32_t *__restrict__ status) {
-    const int lane = threadIdx.x & 31, seg = lane / SWG_G;
-    constexpr int NG = 32 / SWG_G;
-    // the first n_long tasks of the order (the longest alignments): one warp each on wavefronts
+                                                   DevAln *__restrict__ out) {
+    const int lane = threadIdx.x & 31, seg = lane / G;
     const uint32_t nl = *n_long;
+    // the task at place j of the order, if a register path of `cap` offsets takes it; wider ones
+    // are listed by the lane `lists`
+    auto take = [&](uint32_t j, uint32_t end, int cap, bool lists, uint32_t &task, DevHsp &h) {
+        if (j >= end) return false;
+        task = (uint32_t)order[j];
+        h = sel[task];
+        const int64_t rows = (int64_t)h.qe - h.qs + 2 * (int64_t)w;
+        if (dev_band(h, w) <= cap && rows <= SW_MAX_ROWS) return true;
+        if (lists) wide[atomicAdd(wide_count, 1u)] = task;
+        return false;
+    };
     for (;;) {
         uint32_t j = 0;
         if (lane == 0) j = atomicAdd(next_long, 1u);
         j = __shfl_sync(0xffffffffu, j, 0);
         if (j >= nl) break;
-        const uint32_t task = (uint32_t)order[j];
-        const DevHsp h = sel[task];
-        if (dev_band(h, w) > 64) {
-            if (lane == 0) wide[atomicAdd(wide_count, 1u)] = task;
-            continue;
-        }
+        uint32_t task = 0;
+        DevHsp h{};
+        if (!take(j, nl, 64, lane == 0, task, h)) continue;
         DevAln res;
-        sw_wave(h, qpk, qnb, qstart, bpk, bnb, seq_start, match, mismatch, go + ge, ge, w, res);
+        sw_band<32, 1, 1, CUT>(h, true, q, qstart, seq_start, c, w, res);
         if (lane == 0) out[task] = res;
     }
+    constexpr uint32_t NT = 32 / G;
     for (;;) {
         uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(next_task, (uint32_t)NG);
+        if (lane == 0) base = atomicAdd(next_task, NT);
         base = __shfl_sync(0xffffffffu, base, 0) + nl;
         if (base >= n) return;
-        const bool valid = base + seg < n;
-        const uint32_t task = valid ? (uint32_t)order[base + seg] : 0u;  // longest alignments first
+        uint32_t task = 0;
         DevHsp h{};
-        if (valid) h = sel[task];
-        bool handled = false;
+        const bool first = lane % G == 0, on = take(base + seg, n, G * (KA + KB), first, task, h);
+        if (!__any_sync(0xffffffffu, on)) continue;
         DevAln res;
-        sw_group<SWG_G, SWG_K>(valid, h, qpk, qnb, qstart, bpk, bnb, seq_start, match, mismatch, go + ge, ge, w,
-                               handled, res);
-        if (handled && lane % SWG_G == 0) out[task] = res;
-        // wider bands: one HSP at a time with the whole warp
-        uint32_t rest = __ballot_sync(0xffffffffu, valid && !handled && lane % SWG_G == 0);
-        while (rest) {
-            const int src = __ffs(rest) - 1;
-            rest &= rest - 1;
-            const uint32_t t2 = (uint32_t)order[base + (uint32_t)(src / SWG_G)];
-            if (dev_band(sel[t2], w) > 64) {  // wide bands: k_banded_sw_wide
-                if (lane == 0) wide[atomicAdd(wide_count, 1u)] = t2;
-                continue;
-            }
-            sw_task_warp<false>(sel, t2, strip_off, strips, qpk, qnb, qstart, bpk, bnb, seq_start, match, mismatch, go,
-                                ge, w, out, status);
-            __syncwarp();
-        }
+        sw_band<G, KA, KB, CUT>(h, on, q, qstart, seq_start, c, w, res);
+        if (on && first) out[task] = res;
     }
 }
 
-// Bands wider than 64 diagonals, one HSP per warp: up to 32 x SWW_K offsets with the
-// row states in registers (the grouped path over the whole warp), wider ones on the
-// strip path.  A kernel of its own, so that its registers do not limit the main
+// Bands wider than 64 diagonals, a warp each: up to SW_MAX_BAND offsets in registers, wider ones
+// on the strip path.  A kernel of its own, so that its registers do not limit the main
 // alignment kernel.
-constexpr int SWW_K = 9;
+template <bool CUT>
 __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict__ sel, const uint32_t *__restrict__ wide,
                                                         const uint32_t *__restrict__ wide_count,
                                                         uint32_t *__restrict__ next, const uint64_t *__restrict__ strip_off,
-                                                        SwCell *__restrict__ strips, const uint32_t *__restrict__ qpk,
-                                                        const uint32_t *__restrict__ qnb, const uint64_t *__restrict__ qstart,
-                                                        const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                                                        const uint64_t *__restrict__ seq_start, int32_t match,
-                                                        int32_t mismatch, int32_t go, int32_t ge, int32_t w,
+                                                        SwCell *__restrict__ strips, SwSeqs q,
+                                                        const uint64_t *__restrict__ qstart,
+                                                        const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
                                                         DevAln *__restrict__ out, uint32_t *__restrict__ status) {
     const int lane = threadIdx.x & 31;
     const uint32_t n = *wide_count;
@@ -2115,15 +1870,13 @@ __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict
         if (j >= n) return;
         const uint32_t task = wide[j];
         const DevHsp h = sel[task];
-        bool handled = false;
-        DevAln res;
-        sw_group<32, SWW_K>(true, h, qpk, qnb, qstart, bpk, bnb, seq_start, match, mismatch, go + ge, ge, w, handled,
-                            res);
-        if (handled) {
+        if (dev_band(h, w) <= SW_MAX_BAND && (int64_t)h.qe - h.qs + 2 * (int64_t)w <= SW_MAX_ROWS) {
+            DevAln res;
+            sw_band<32, 5, 4, CUT>(h, true, q, qstart, seq_start, c, w, res);
             if (lane == 0) out[task] = res;
         } else {
-            sw_task_warp<true>(sel, task, strip_off, strips, qpk, qnb, qstart, bpk, bnb, seq_start, match, mismatch,
-                               go, ge, w, out, status);
+            sw_task_strip(sel, task, strip_off, strips, q.qpk, q.qnb, qstart, q.bpk, q.bnb, seq_start, c.match, c.mismatch,
+                          c.goe - c.ge, c.ge, w, out, status);
         }
         __syncwarp();
     }
@@ -2135,10 +1888,11 @@ __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict
 //   cells[1] (wider bands);
 // - its alignment-order key (65535 - DP-window rows) << 32 | task, so that an ascending sort
 //   on bits 32..47 hands out the longest alignments first (they bound the kernel's time) and
-//   groups alignments of similar length; alignments of at least long_rows rows are counted
-//   in *n_long (they sort first).
-__global__ void k_sw_prepare(const DevHsp *__restrict__ h, uint32_t n, int32_t w, const uint64_t *__restrict__ qstart,
-                             uint32_t *__restrict__ B, unsigned long long *__restrict__ cells, uint32_t long_rows,
+//   groups alignments of similar length; alignments of at least long_rows rows, and those
+//   whose bands are wider than the grouped path's `cap` offsets, are counted in *n_long (they
+//   sort first).
+__global__ void k_sw_prepare(const DevHsp *__restrict__ h, uint32_t n, int32_t w, int cap,
+                             const uint64_t *__restrict__ qstart, uint32_t *__restrict__ B, unsigned long long *__restrict__ cells, uint32_t long_rows,
                              uint64_t *__restrict__ keys, uint32_t *__restrict__ n_long) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = i < n;
@@ -2151,6 +1905,7 @@ __global__ void k_sw_prepare(const DevHsp *__restrict__ h, uint32_t n, int32_t w
         const int64_t m = (int64_t)(qstart[x.qi + 1] - qstart[x.qi]);
         rows = min(m, (int64_t)x.qe + w) - max((int64_t)0, (int64_t)x.qs - w);
         if (rows > 0) atomicAdd(cells + (b > 64 ? 1 : 0), (unsigned long long)(rows * b));
+        if (b > cap && b <= 64) rows = 65535;
         const int64_t r = rows < 0 ? 0 : (rows > 65535 ? 65535 : rows);
         keys[i] = ((uint64_t)(65535 - (uint32_t)r) << 32) | i;
     }
@@ -3114,14 +2869,25 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         unsigned long long *dp_cells = reinterpret_cast<unsigned long long *>(arena.alloc_n<uint64_t>(2));
         GN_CUDA(cudaMemsetAsync(dp_cells, 0, 16, s));
         uint64_t *okeys = arena.alloc_n<uint64_t>(n_sel), *okeys_alt = arena.alloc_n<uint64_t>(n_sel);
-        // alignments of at least sw_long rows go to the wavefront path (their rows would
-        // bound the kernel's time on the grouped path)
-        uint32_t sw_long = ix->tuning.sw_wave_rows ? ix->tuning.sw_wave_rows : 512;
+        // lanes per HSP of the grouped path (the index's tuning; GN_SW_LANES overrides)
+        uint32_t sw_lanes = ix->tuning.sw_lanes ? ix->tuning.sw_lanes : 8;
+        if (const char *e = getenv("GN_SW_LANES")) sw_lanes = (uint32_t)atoi(e);
+        if (sw_lanes != 16 && sw_lanes != 32) sw_lanes = 8;
+        // Alignments of at least sw_long rows get a warp each, and warps are few, one or two a
+        // scheduler: a warp alone issues at nearly half the pipes' rate, and the longest alignments,
+        // which bound the phase, slow down with every warp that shares theirs.  us at 4 | 8 | 16
+        // warps an SM, rows from 512 | 1,024 (default band): 4,900 alignments 165 165 | 182 212 |
+        // 223 257; 30,000 alignments 534 375 | 374 307 | 436 449; 50,000 1036 768 | 716 567 | 672
+        // 613.  With no more alignments than warps each gets its own (sw_lanes = 32 asks for that).
+        const bool many = n_sel > (uint32_t)num_sms() * 64;
+        uint32_t sw_long = ix->tuning.sw_wave_rows ? ix->tuning.sw_wave_rows : many ? 1024 : 512;
+        if (n_sel <= (uint32_t)num_sms() * 4 || sw_lanes == 32) sw_long = 1;
         if (const char *e = getenv("GN_SW_LONG_ROWS")) sw_long = (uint32_t)std::max(1l, strtol(e, nullptr, 10));
         uint32_t *n_long = arena.alloc_n<uint32_t>(2);
         GN_CUDA(cudaMemsetAsync(n_long, 0, 8, s));
         GN_LAUNCH("k_sw_prepare", n_sel, s,
-                  k_sw_prepare<<<blocks_for(n_sel), 256, 0, s>>>(sel, n_sel, (int32_t)p.band_w, qstart_d, B, dp_cells,
+                  k_sw_prepare<<<blocks_for(n_sel), 256, 0, s>>>(sel, n_sel, (int32_t)p.band_w,
+                                                                  sw_lanes == 16 ? 48 : 40, qstart_d, B, dp_cells,
                                                                   sw_long, okeys, n_long));
         void *scr = arena.alloc(scan_scratch_bytes(n_sel));
         exclusive_scan_u32(B, soff, n_sel, scr, s);
@@ -3135,24 +2901,22 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
                                     ? okeys_alt : okeys;
         GN_CUDA(cudaMemsetAsync(counter, 0, 12, s));
         uint32_t *wide = arena.alloc_n<uint32_t>(n_sel);
-        // lanes per HSP of the grouped path (the index's tuning; GN_SW_LANES overrides)
-        uint32_t sw_lanes = ix->tuning.sw_lanes ? ix->tuning.sw_lanes : 8;
-        if (const char *e = getenv("GN_SW_LANES")) sw_lanes = (uint32_t)atoi(e);
-        if (sw_lanes != 16 && sw_lanes != 32) sw_lanes = 8;
-        auto sw_kernel = sw_lanes == 32 ? k_banded_sw<32, 2> : sw_lanes == 16 ? k_banded_sw<16, 3> : k_banded_sw<8, 5>;
-        const uint32_t per_warp = 32 / sw_lanes;
-        unsigned warps = (unsigned)std::min<uint64_t>((n_sel + per_warp - 1) / per_warp, (uint64_t)num_sms() * 32);
+        const bool cut = sc.mismatch < 2 * sc.gap_extend;
+        auto sw_kernel = sw_lanes == 16 ? (cut ? k_banded_sw<16, 2, 1, true> : k_banded_sw<16, 2, 1, false>)
+                                        : (cut ? k_banded_sw<8, 3, 2, true> : k_banded_sw<8, 3, 2, false>);
+        auto wide_kernel = cut ? k_banded_sw_wide<true> : k_banded_sw_wide<false>;
+        const SwScore score{sc.match, sc.mismatch, sc.gap_open + sc.gap_extend, sc.gap_extend, 1};
+        const SwSeqs seqs{qp.pk, qp.nb, ix->bank.pk, ix->bank.nb,
+                          (int64_t)Packed::pk_words(M) - 1, (int64_t)Packed::nb_words(M) - 1,
+                          (int64_t)Packed::pk_words(ix->n_bases) - 1, (int64_t)Packed::nb_words(ix->n_bases) - 1};
+        const unsigned warps = (unsigned)std::min<uint64_t>(n_sel, (uint64_t)num_sms() * (many ? 8 : 4));
         GN_LAUNCH("k_banded_sw", area[0], s,
-                  sw_kernel<<<(warps * 32 + 127) / 128, 128, 0, s>>>(sel, n_sel, soff, strips, qp.pk, qp.nb, qstart_d,
-                                                          ix->bank.pk, ix->bank.nb, ix->seq_start_d, sc.match,
-                                                          sc.mismatch, sc.gap_open, sc.gap_extend,
+                  sw_kernel<<<(warps * 32 + 127) / 128, 128, 0, s>>>(sel, n_sel, seqs, qstart_d, ix->seq_start_d, score,
                                                           (int32_t)p.band_w, counter, order, wide, counter + 1,
-                                                          n_long, n_long + 1, aln, status));
+                                                          n_long, n_long + 1, aln));
         GN_LAUNCH("k_banded_sw_wide", area[1], s,
-                  k_banded_sw_wide<<<num_sms() * 4, 128, 0, s>>>(sel, wide, counter + 1, counter + 2, soff, strips, qp.pk,
-                                                                qp.nb, qstart_d, ix->bank.pk, ix->bank.nb,
-                                                                ix->seq_start_d, sc.match, sc.mismatch, sc.gap_open,
-                                                                sc.gap_extend, (int32_t)p.band_w, aln, status));
+                  wide_kernel<<<num_sms() * 4, 128, 0, s>>>(sel, wide, counter + 1, counter + 2, soff, strips, seqs, qstart_d,
+                                                            ix->seq_start_d, score, (int32_t)p.band_w, aln, status));
     }
     timer.mark("banded_sw");
     if (keep) {
