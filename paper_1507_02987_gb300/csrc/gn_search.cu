@@ -889,60 +889,6 @@ __device__ __forceinline__ int32_t dev_pair(uint32_t a, uint32_t b, int32_t matc
     return (a < 4u && a == b) ? match : mismatch;
 }
 
-// One direction of the X-drop walk, 32 steps per round for a whole warp.  Step e
-// (1-based) compares query base qg(e) with bank base dg(e).  The sequential rule
-// (score += s; if score > best: best = score, ext = e; else if best - score > X:
-// stop) stops at the first e where max(best so far, score_e) - score_e > X, and
-// ext is the first step that reached the final best.  Returns ext.
-// The walk continues a lane's walk: steps e_first.. with the score, best and ext that the
-// steps before e_first left (0, 0, 0 and e_first = 1 for a fresh walk).
-template <int DIR>
-__device__ __forceinline__ uint32_t xdrop_walk_warp(const uint32_t *__restrict__ qpk, const uint32_t *__restrict__ qnb,
-                                                    const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                                                    uint64_t qg0, uint64_t dg0, uint32_t emax, int32_t match,
-                                                    int32_t mismatch, int32_t X, int lane, uint32_t e_first,
-                                                    int32_t score0, int32_t best0, uint32_t ext0) {
-    int32_t carry_score = score0, carry_best = best0;
-    uint32_t carry_ext = ext0;
-    for (uint32_t e0 = e_first; e0 <= emax; e0 += 32) {
-        const uint32_t e = e0 + lane;
-        const bool in = e <= emax;
-        int32_t sc = 0;
-        if (in) {
-            const uint64_t qg = DIR > 0 ? qg0 + (e - 1) : qg0 - e;
-            const uint64_t dg = DIR > 0 ? dg0 + (e - 1) : dg0 - e;
-            sc = dev_pair(dev_base(qpk, qnb, qg), dev_base(bpk, bnb, dg), match, mismatch);
-        }
-        // running score (inclusive prefix sum) and running best (inclusive prefix max)
-        int32_t S = sc;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t t = __shfl_up_sync(0xffffffffu, S, o);
-            if (lane >= o) S += t;
-        }
-        S += carry_score;
-        int32_t M = in ? S : INT32_MIN;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t t = __shfl_up_sync(0xffffffffu, M, o);
-            if (lane >= o) M = max(M, t);
-        }
-        M = max(M, carry_best);
-        const uint32_t stop = __ballot_sync(0xffffffffu, in && M - S > X);
-        const uint32_t last = stop ? (uint32_t)(__ffs(stop) - 1) : 31u;  // last lane that counts this round
-        const int32_t Mlast = __shfl_sync(0xffffffffu, M, last);
-        if (Mlast > carry_best) {
-            // first step of this round that reached the new best
-            const uint32_t hit = __ballot_sync(0xffffffffu, in && (uint32_t)lane <= last && S == Mlast);
-            carry_ext = e0 + (uint32_t)(__ffs(hit) - 1);
-            carry_best = Mlast;
-        }
-        if (stop) break;
-        carry_score = __shfl_sync(0xffffffffu, S, 31);
-    }
-    return carry_ext;
-}
-
 // 16 bases from position p (p >= -16; bases before 0 read as code 0, non-base): 2-bit
 // codes with base p in bits 31-30, and a mask with bit i set when base p + i is a non-base.
 // The packed arrays carry two words past the last base, so p + 15 may pass the end.
@@ -956,122 +902,162 @@ __device__ __forceinline__ void base_window16(const uint32_t *__restrict__ pk, c
     bad = (uint32_t)(((((uint64_t)n1) << 32) | n0) >> (uint32_t)(p & 31)) & 0xFFFFu;
 }
 
-// One direction of the walk on one lane, by the sequential rule, for at most lim steps,
-// 16 steps per window of bases: returns whether the walk ended (the drop passed X, or the
-// sequence ended); score, best, ext and the steps taken are left for a continuation.
-template <int DIR>
-__device__ __forceinline__ bool xdrop_walk_lane(const uint32_t *__restrict__ qpk, const uint32_t *__restrict__ qnb,
-                                                const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                                                uint64_t qg0, uint64_t dg0, uint32_t emax, int32_t match,
-                                                int32_t mismatch, int32_t X, uint32_t lim, int32_t &score,
-                                                int32_t &best, uint32_t &ext, uint32_t &steps) {
-    score = 0;
-    best = 0;
-    ext = 0;
-    const uint32_t until = min(emax, lim);
-    for (uint32_t e0 = 0; e0 < until; e0 += 16) {
-        // steps e0 + 1 .. e0 + 16: positions qg0 + e0 .. + 15 (right), qg0 - e0 - 16 .. - 1 (left)
-        const int64_t qp = DIR > 0 ? (int64_t)(qg0 + e0) : (int64_t)qg0 - (int64_t)e0 - 16;
-        const int64_t dp = DIR > 0 ? (int64_t)(dg0 + e0) : (int64_t)dg0 - (int64_t)e0 - 16;
-        uint32_t wq, bq, wd, bd;
-        base_window16(qpk, qnb, qp, wq, bq);
-        base_window16(bpk, bnb, dp, wd, bd);
-        const uint32_t x = ~(wq ^ wd), eq = x & (x >> 1);  // bit 30 - 2k: codes equal at window base k
-        const uint32_t bad = bq | bd;
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            const uint32_t e = e0 + (uint32_t)t + 1;
-            if (e > until) {
-                steps = until;
-                return until == emax;
-            }
-            const int k = DIR > 0 ? t : 15 - t;
-            const bool same = ((eq >> (30 - 2 * k)) & 1u) && !((bad >> k) & 1u);
-            score += same ? match : mismatch;
-            if (score > best) {
-                best = score;
-                ext = e;
-            } else if (best - score > X) {
-                steps = e;
-                return true;
-            }
-        }
-    }
-    steps = until;
-    return until == emax;
+// 32 bases from position p (any sign), first one on top, and their non-base bits from bit 0;
+// words outside the array are clamped (the caller takes nothing from their positions).
+__device__ __forceinline__ uint64_t window32(const uint32_t *__restrict__ pk, const uint32_t *__restrict__ nb, int64_t p,
+                                             int64_t last_pk, int64_t last_nb, uint32_t &bad) {
+    const int64_t a = p >> 4, b = p >> 5;
+    const uint32_t w0 = pk[max((int64_t)0, min(a, last_pk))], w1 = pk[max((int64_t)0, min(a + 1, last_pk))];
+    const uint32_t w2 = pk[max((int64_t)0, min(a + 2, last_pk))];
+    const uint32_t n0 = nb[max((int64_t)0, min(b, last_nb))], n1 = nb[max((int64_t)0, min(b + 1, last_nb))];
+    const uint32_t s = 2u * (uint32_t)(p & 15);
+    bad = __funnelshift_r(n0, n1, (uint32_t)(p & 31));
+    return (uint64_t)__funnelshift_l(w1, w0, s) << 32 | __funnelshift_l(w2, w1, s);
 }
 
-// X-drop extension of both ends of every HSP.  Each lane walks one HSP's ends on its own
-// (most walks end within a few dozen steps) for at most lim steps each; the warp then
-// continues the walks that did not end, one after the other, 32 steps per round.
-__global__ void k_xdrop(DevHsp *__restrict__ h, uint32_t n, const uint32_t *__restrict__ qpk,
-                        const uint32_t *__restrict__ qnb, const uint64_t *__restrict__ qstart,
-                        const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
-                        const uint64_t *__restrict__ seq_start, int32_t match, int32_t mismatch, int32_t X,
-                        uint32_t nq, uint32_t n_seqs, uint32_t lim, uint32_t *__restrict__ next_group) {
+// Bit i of the low 16 bits of x to bits 31 - 2 i and 30 - 2 i.
+__device__ __forceinline__ uint32_t spread16_down(uint32_t x) {
+    x &= 0xFFFFu;
+    x = (x | x << 8) & 0x00FF00FFu;
+    x = (x | x << 4) & 0x0F0F0F0Fu;
+    x = (x | x << 2) & 0x33333333u;
+    x = (x | x << 1) & 0x55555555u;  // bit 2 i
+    return __brev(x * 3u);
+}
+// Packed sequences of a search.
+struct PackedPair {
+    const uint32_t *qpk, *qnb, *bpk, *bnb;
+    int64_t last_qpk, last_qnb, last_bpk, last_bnb;  // last words
+};
+
+// Bits 31 - 2 i and 30 - 2 i of w[j]: bases 16 j + i of the windows at q and d are equal bases
+// (codes agree, no non-base); both windows start inside their arrays or, at the front, before
+// them (base positions below 0 come out as anything).
+__device__ __forceinline__ void equal32(const PackedPair &s, int64_t q, int64_t d, uint32_t w[2]) {
+    uint32_t qb, db;
+    uint64_t y;
+    if (q >= 0 && d >= 0) {  // two words past the last base are there, so nothing needs a limit
+        const uint32_t *a = s.qpk + (q >> 4), *b = s.bpk + (d >> 4), *m = s.qnb + (q >> 5), *n = s.bnb + (d >> 5);
+        const uint32_t a0 = a[0], a1 = a[1], a2 = a[2], b0 = b[0], b1 = b[1], b2 = b[2];
+        const uint32_t m0 = m[0], m1 = m[1], n0 = n[0], n1 = n[1];
+        const uint32_t sq = 2u * (uint32_t)(q & 15), sd = 2u * (uint32_t)(d & 15);
+        w[0] = __funnelshift_l(a1, a0, sq) ^ __funnelshift_l(b1, b0, sd);
+        w[1] = __funnelshift_l(a2, a1, sq) ^ __funnelshift_l(b2, b1, sd);
+        qb = __funnelshift_r(m0, m1, (uint32_t)(q & 31));
+        db = __funnelshift_r(n0, n1, (uint32_t)(d & 31));
+    } else {
+        y = window32(s.qpk, s.qnb, q, s.last_qpk, s.last_qnb, qb) ^ window32(s.bpk, s.bnb, d, s.last_bpk, s.last_bnb, db);
+        w[0] = (uint32_t)(y >> 32);
+        w[1] = (uint32_t)y;
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const uint32_t e = ~(w[j] | w[j] >> 1) & 0x55555555u;
+        w[j] = e | e << 1;
+    }
+    if (qb | db) {
+        w[0] &= ~spread16_down(qb | db);
+        w[1] &= ~spread16_down((qb | db) >> 16);
+    }
+}
+
+// X-drop extension.  The rule, step e = 1, 2, .. out from an HSP's end: score += s; if score >
+// best: best = score, ext = e; else if best - score > X: stop.  Within a run of matches the
+// best is at its end, and within a run of mismatches only the drop after the last one matters,
+// so a walk takes one step per run, from 32 bases' equality bits at a time (left windows are
+// mirrored).  A lane takes one end of an HSP.  Walks are mostly one window long and sometimes,
+// inside a repeat, hundreds, so a lane whose walk has ended waits only until XD_REFILL lanes of its
+// warp have, and then gets a new one from the counter.  Writes the end's two words; len is left
+// to whoever needs it.  Bound by the latency of each end's first window, whose place is random.
+// Measured against a step per base with 32 HSPs a warp, whose walks over 64 steps the warp
+// continued one by one: 2.1 M HSPs on 4 Gbp 1.07 -> 0.35 ms, 103,000 on 400 Mbp 0.43 -> 0.08,
+// 177,000 of chromosome-scale queries 0.49 -> 0.12.  Refill at 8, 16, 24 lanes: 0.43, 0.40, 0.35.
+constexpr int XD_REFILL = 24;
+
+__global__ void __launch_bounds__(256) k_xdrop(DevHsp *__restrict__ h, uint32_t n, PackedPair seq,
+                                               const uint64_t *__restrict__ qstart,
+                                               const uint64_t *__restrict__ seq_start, int32_t match, int32_t mismatch,
+                                               int32_t X, uint32_t nq, uint32_t n_seqs,
+                                               unsigned long long *__restrict__ next_end) {
     const int lane = threadIdx.x & 31;
+    const uint64_t ends = 2ull * n;
+    bool more = true;    // the counter has not run out
+    bool open = false;   // the lane's walk goes on
+    uint64_t item = 0;   // HSP << 1 | right end
+    uint32_t e = 0, emax = 0, ext = 0;
+    int64_t q = 0, d = 0;
+    int32_t score = 0, best = 0;
     for (;;) {
-        // groups of 32 HSPs from a counter: a warp whose group held long walks takes fewer
-        uint32_t g = 0;
-        if (lane == 0) g = atomicAdd(next_group, 1u);
-        const uint32_t b0 = __shfl_sync(0xffffffffu, g, 0) * 32u;
-        if (b0 >= n) break;
-        const uint32_t i = b0 + lane;
-        bool valid = i < n;
-        DevHsp r;
-        uint64_t qb = 0, sb = 0;
-        uint32_t emax_l = 0, emax_r = 0;
-        if (valid) {
-            r = h[i];
-            valid = GN_CHECK(r.qi < nq && r.seq < n_seqs);
-        }
-        if (valid) {
-            qb = qstart[r.qi];
-            sb = seq_start[r.seq];
-            const uint32_t m = (uint32_t)(qstart[r.qi + 1] - qb), L = (uint32_t)(seq_start[r.seq + 1] - sb);
-            emax_l = min(r.qs, r.ds);
-            emax_r = min(m - r.qe, L - r.de);
-        }
-        int32_t sl = 0, bl = 0, sr = 0, br = 0;
-        uint32_t el = 0, er = 0, nl = 0, nr = 0;
-        bool done_l = true, done_r = true;
-        if (valid) {
-            done_l = xdrop_walk_lane<-1>(qpk, qnb, bpk, bnb, qb + r.qs, sb + r.ds, emax_l, match, mismatch, X, lim, sl,
-                                         bl, el, nl);
-            done_r = xdrop_walk_lane<1>(qpk, qnb, bpk, bnb, qb + r.qe, sb + r.de, emax_r, match, mismatch, X, lim, sr,
-                                        br, er, nr);
-        }
-        // walks that did not end: the whole warp continues them
-        uint32_t todo = __ballot_sync(0xffffffffu, !done_l || !done_r);
-        while (todo) {
-            const int src = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const uint64_t q0 = __shfl_sync(0xffffffffu, qb, src), s0 = __shfl_sync(0xffffffffu, sb, src);
-            const bool cl = __shfl_sync(0xffffffffu, !done_l, src), cr = __shfl_sync(0xffffffffu, !done_r, src);
-            if (cl) {
-                const uint32_t qs = __shfl_sync(0xffffffffu, valid ? r.qs : 0u, src);
-                const uint32_t ds = __shfl_sync(0xffffffffu, valid ? r.ds : 0u, src);
-                const uint32_t x = xdrop_walk_warp<-1>(
-                    qpk, qnb, bpk, bnb, q0 + qs, s0 + ds, __shfl_sync(0xffffffffu, emax_l, src), match, mismatch, X,
-                    lane, __shfl_sync(0xffffffffu, nl, src) + 1, __shfl_sync(0xffffffffu, sl, src),
-                    __shfl_sync(0xffffffffu, bl, src), __shfl_sync(0xffffffffu, el, src));
-                if (lane == src) el = x;
-            }
-            if (cr) {
-                const uint32_t qe = __shfl_sync(0xffffffffu, valid ? r.qe : 0u, src);
-                const uint32_t de = __shfl_sync(0xffffffffu, valid ? r.de : 0u, src);
-                const uint32_t x = xdrop_walk_warp<1>(
-                    qpk, qnb, bpk, bnb, q0 + qe, s0 + de, __shfl_sync(0xffffffffu, emax_r, src), match, mismatch, X,
-                    lane, __shfl_sync(0xffffffffu, nr, src) + 1, __shfl_sync(0xffffffffu, sr, src),
-                    __shfl_sync(0xffffffffu, br, src), __shfl_sync(0xffffffffu, er, src));
-                if (lane == src) er = x;
+        const uint32_t idle = __ballot_sync(0xffffffffu, !open);
+        if (more && __popc(idle) >= XD_REFILL) {
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(next_end, (unsigned long long)__popc(idle));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            more = at + __popc(idle) < ends;
+            if (!open) {
+                item = at + __popc(idle & ((1u << lane) - 1u));
+                if (item < ends) {
+                    const DevHsp &r = h[item >> 1];
+                    const uint32_t qi = r.qi, sq = r.seq;
+                    if (GN_CHECK(qi < nq && sq < n_seqs)) {
+                        const int64_t qb = (int64_t)qstart[qi], sb = (int64_t)seq_start[sq];
+                        if (item & 1) {
+                            const uint32_t qe = r.qe, de = r.de;
+                            emax = (uint32_t)min((int64_t)qstart[qi + 1] - qb - qe, (int64_t)seq_start[sq + 1] - sb - de);
+                            q = qb + qe;
+                            d = sb + de;
+                        } else {
+                            const uint32_t qs = r.qs, ds = r.ds;
+                            emax = min(qs, ds);
+                            q = qb + qs;
+                            d = sb + ds;
+                        }
+                        e = ext = 0;
+                        score = best = 0;
+                        open = emax > 0;
+                    }
+                }
             }
         }
-        if (valid) {
-            r.qs -= el; r.ds -= el;
-            r.qe += er; r.de += er;
-            r.len = min(r.qe - r.qs, r.de - r.ds);
-            h[i] = r;
+        if (!__any_sync(0xffffffffu, open)) {
+            if (!more) break;
+            continue;
+        }
+        if (open) {
+            const bool right = item & 1;
+            uint32_t w[2];
+            equal32(seq, right ? q : q - 32, right ? d : d - 32, w);
+            if (!right) {
+                const uint32_t t = __brev(w[0]);
+                w[0] = __brev(w[1]);
+                w[1] = t;
+            }
+            q += right ? 32 : -32;
+            d += right ? 32 : -32;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                uint32_t eq = w[j], left = open ? min(16u, emax - e) : 0u;
+                while (left) {
+                    const uint32_t m = min((uint32_t)__clz(~eq) >> 1, left);  // matches
+                    score += (int32_t)m * match;
+                    e += m;
+                    left -= m;
+                    if (m && score > best) { best = score; ext = e; }
+                    eq = __funnelshift_lc(0u, eq, 2 * m);
+                    const uint32_t x = min((uint32_t)__clz(eq) >> 1, left);  // mismatches
+                    if ((int64_t)best - score - (int64_t)x * mismatch > X) { open = false; break; }
+                    score += (int32_t)x * mismatch;
+                    e += x;
+                    left -= x;
+                    eq = __funnelshift_lc(0u, eq, 2 * x);
+                }
+            }
+            if (e >= emax) open = false;
+            if (!open && ext) {
+                uint32_t *r = reinterpret_cast<uint32_t *>(h + (item >> 1));
+                if (right) { r[W_QE] += ext; r[W_DE] += ext; }
+                else { r[W_QS] -= ext; r[W_DS] -= ext; }
+            }
         }
     }
 }
@@ -1543,40 +1529,12 @@ struct SwGeom {
     }
 };
 
-// 32 bases from position p (any sign), first one on top, and their non-base bits from bit 0;
-// words outside the array are clamped (their positions lie outside the DP window).
-__device__ __forceinline__ uint64_t window32(const uint32_t *__restrict__ pk, const uint32_t *__restrict__ nb, int64_t p,
-                                             int64_t last_pk, int64_t last_nb, uint32_t &bad) {
-    const int64_t a = p >> 4, b = p >> 5;
-    const uint32_t w0 = pk[max((int64_t)0, min(a, last_pk))], w1 = pk[max((int64_t)0, min(a + 1, last_pk))];
-    const uint32_t w2 = pk[max((int64_t)0, min(a + 2, last_pk))];
-    const uint32_t n0 = nb[max((int64_t)0, min(b, last_nb))], n1 = nb[max((int64_t)0, min(b + 1, last_nb))];
-    const uint32_t s = 2u * (uint32_t)(p & 15);
-    bad = __funnelshift_r(n0, n1, (uint32_t)(p & 31));
-    return (uint64_t)__funnelshift_l(w1, w0, s) << 32 | __funnelshift_l(w2, w1, s);
-}
-
-// Bit i of the low 16 bits of x to bits 31 - 2 i and 30 - 2 i.
-__device__ __forceinline__ uint32_t spread16_down(uint32_t x) {
-    x &= 0xFFFFu;
-    x = (x | x << 8) & 0x00FF00FFu;
-    x = (x | x << 4) & 0x0F0F0F0Fu;
-    x = (x | x << 2) & 0x33333333u;
-    x = (x | x << 1) & 0x55555555u;  // bit 2 i
-    return __brev(x * 3u);
-}
 // Bits [from, to) of 32 positions (any values).
 __device__ __forceinline__ uint32_t positions(int64_t from, int64_t to) {
     const uint32_t a = (uint32_t)min(max(from, (int64_t)0), (int64_t)32), b = (uint32_t)min(max(to, (int64_t)0), (int64_t)32);
     const uint32_t lo = __funnelshift_lc(0u, 0xFFFFFFFFu, a), hi = __funnelshift_lc(0u, 0xFFFFFFFFu, b);
     return lo & ~hi;
 }
-
-// Packed sequences of a search, as the register paths read them.
-struct SwSeqs {
-    const uint32_t *qpk, *qnb, *bpk, *bnb;
-    int64_t last_qpk, last_qnb, last_bpk, last_bnb;  // last words
-};
 
 template <int K>
 struct SwSet {
@@ -1609,7 +1567,7 @@ struct SwSet {
         in_band = !on || B <= 0 ? 0u : B >= K ? 0x55555555u : 0x55555555u & ~(0xFFFFFFFFu >> (2 * B));
     }
     // the bases of the 16 rows to come; returns whether dno or qno has a bit that they meet
-    __device__ __forceinline__ bool load(const SwSeqs &s) {
+    __device__ __forceinline__ bool load(const PackedPair &s) {
         uint32_t db, qb;
         const uint64_t w = window32(s.bpk, s.bnb, d, s.last_bpk, s.last_bnb, db);
         dw_hi = (uint32_t)(w >> 32);
@@ -1763,7 +1721,7 @@ __device__ __forceinline__ void sw_finish(int32_t best, uint32_t cell, uint32_t 
 // Aligns each segment's HSP h (where on; a band of at most G K offsets, at most SW_MAX_ROWS
 // rows); every lane of the segment gets the alignment.
 template <int G, int KA, int KB, bool CUT>
-__device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const SwSeqs &q, const uint64_t *__restrict__ qstart,
+__device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const PackedPair &q, const uint64_t *__restrict__ qstart,
                                         const uint64_t *__restrict__ seq_start, const SwScore &c, int32_t w, DevAln &res) {
     const int sl = (threadIdx.x & 31) % G;
     constexpr int K = KA + KB;
@@ -1802,7 +1760,7 @@ __device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const SwSeqs &
 // 40 diagonals (33 and up at the default width), <16, 2, 1> 48; k_sw_prepare counts tasks with
 // wider bands, up to 64, among the long ones.
 template <int G, int KA, int KB, bool CUT>
-__global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ sel, uint32_t n, SwSeqs q,
+__global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ sel, uint32_t n, PackedPair q,
                                                    const uint64_t *__restrict__ qstart,
                                                    const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
                                                    uint32_t *__restrict__ next_task, const uint64_t *__restrict__ order,
@@ -1857,7 +1815,7 @@ template <bool CUT>
 __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict__ sel, const uint32_t *__restrict__ wide,
                                                         const uint32_t *__restrict__ wide_count,
                                                         uint32_t *__restrict__ next, const uint64_t *__restrict__ strip_off,
-                                                        SwCell *__restrict__ strips, SwSeqs q,
+                                                        SwCell *__restrict__ strips, PackedPair q,
                                                         const uint64_t *__restrict__ qstart,
                                                         const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
                                                         DevAln *__restrict__ out, uint32_t *__restrict__ status) {
@@ -2766,28 +2724,27 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         if (n_hsp) memcpy(res->st_hsp.data(), v.data(), sizeof(DevHsp) * n_hsp);
     }
 
+    const PackedPair seqs{qp.pk, qp.nb, ix->bank.pk, ix->bank.nb, (int64_t)Packed::pk_words(M) - 1,
+                          (int64_t)Packed::nb_words(M) - 1, (int64_t)Packed::pk_words(ix->n_bases) - 1,
+                          (int64_t)Packed::nb_words(ix->n_bases) - 1};
     // a9: extension
     if (n_hsp) {
-        // resident warps only, taking 32-HSP groups from a counter
-        uint32_t *next_group = arena.alloc_n<uint32_t>(1);
-        GN_CUDA(cudaMemsetAsync(next_group, 0, 4, s));
+        // resident warps only, taking HSP ends from a counter
+        unsigned long long *next_end = reinterpret_cast<unsigned long long *>(arena.alloc_n<uint64_t>(1));
+        GN_CUDA(cudaMemsetAsync(next_end, 0, 8, s));
         int xocc = 0;
         GN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&xocc, k_xdrop, 256, 0));
         const uint64_t xwarps =
-            std::min<uint64_t>((n_hsp + 31) / 32, (uint64_t)num_sms() * std::max(xocc, 1) * 8);
-        // steps a lane walks alone before the warp takes the walk over (GN_XDROP_LANE_STEPS overrides)
-        uint32_t lim = 64;
-        if (const char *e = getenv("GN_XDROP_LANE_STEPS")) lim = (uint32_t)std::max(0l, strtol(e, nullptr, 10));
+            std::min<uint64_t>((2ull * n_hsp + 31) / 32, (uint64_t)num_sms() * std::max(xocc, 1) * 8);
         GN_LAUNCH("k_xdrop", n_hsp, s,
-                  k_xdrop<<<blocks_for(xwarps * 32, 256), 256, 0, s>>>(hsp, n_hsp, qp.pk, qp.nb, qstart_d,
-                                                                      ix->bank.pk, ix->bank.nb, ix->seq_start_d,
-                                                                      sc.match, sc.mismatch, p.xdrop, nq, ix->n_seqs,
-                                                                      lim, next_group));
+                  k_xdrop<<<blocks_for(xwarps * 32, 256), 256, 0, s>>>(hsp, n_hsp, seqs, qstart_d, ix->seq_start_d, sc.match,
+                                                                      sc.mismatch, p.xdrop, nq, ix->n_seqs, next_end));
     }
     timer.mark("xdrop_extend");
     if (keep) {
         std::vector<DevHsp> v = to_host(hsp, n_hsp, s);
         res->st_ext.resize(n_hsp);
+        for (DevHsp &x : v) x.len = std::min(x.qe - x.qs, x.de - x.ds);  // the extension leaves len to its readers
         if (n_hsp) memcpy(res->st_ext.data(), v.data(), sizeof(DevHsp) * n_hsp);
     }
 
@@ -2906,9 +2863,6 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
                                         : (cut ? k_banded_sw<8, 3, 2, true> : k_banded_sw<8, 3, 2, false>);
         auto wide_kernel = cut ? k_banded_sw_wide<true> : k_banded_sw_wide<false>;
         const SwScore score{sc.match, sc.mismatch, sc.gap_open + sc.gap_extend, sc.gap_extend, 1};
-        const SwSeqs seqs{qp.pk, qp.nb, ix->bank.pk, ix->bank.nb,
-                          (int64_t)Packed::pk_words(M) - 1, (int64_t)Packed::nb_words(M) - 1,
-                          (int64_t)Packed::pk_words(ix->n_bases) - 1, (int64_t)Packed::nb_words(ix->n_bases) - 1};
         const unsigned warps = (unsigned)std::min<uint64_t>(n_sel, (uint64_t)num_sms() * (many ? 8 : 4));
         GN_LAUNCH("k_banded_sw", area[0], s,
                   sw_kernel<<<(warps * 32 + 127) / 128, 128, 0, s>>>(sel, n_sel, seqs, qstart_d, ix->seq_start_d, score,
