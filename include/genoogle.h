@@ -249,6 +249,10 @@ GN_API void gn_results_free(gn_results *results);
  * of range). */
 GN_API gn_status gn_results_get(const gn_results *results, uint32_t query, const gn_hit **hits, uint32_t *n);
 GN_API gn_status gn_results_count(const gn_results *results, uint32_t *n_queries, uint64_t *n_hits);
+/* All of them at once: the hits of query q are (*hits)[(*start)[q]] .. (*hits)[(*start)[q + 1] - 1]
+ * (start has n_queries + 1 entries).  Both stay valid until gn_results_free.  Errors: GN_EINVAL
+ * (missing pointer). */
+GN_API gn_status gn_results_all(const gn_results *results, const gn_hit **hits, const uint64_t **start);
 
 /* Phase outputs kept with GN_FLAG_KEEP_STAGES (GN_EINVAL otherwise).
  * Stage ids: GN_STAGE_HSP (HSPs from merged hits), GN_STAGE_EXT (after

@@ -600,6 +600,13 @@ gn_status gn_results_count(const gn_results *r, uint32_t *nq, uint64_t *nh) {
     return GN_OK;
 }
 
+gn_status gn_results_all(const gn_results *r, const gn_hit **hits, const uint64_t **start) {
+    if (!r || !hits || !start) { g_last_error = "results, hits and start are required"; return GN_EINVAL; }
+    *hits = r->hits.data();
+    *start = r->qoff.data();
+    return GN_OK;
+}
+
 gn_status gn_results_stage(const gn_results *r, gn_stage stage, const void **data, uint64_t *n) {
     if (!r || !data || !n) { g_last_error = "results, data and n are required"; return GN_EINVAL; }
     if (!r->has_stages && stage != GN_STAGE_HITS) { g_last_error = "search ran without GN_FLAG_KEEP_STAGES"; return GN_EINVAL; }
