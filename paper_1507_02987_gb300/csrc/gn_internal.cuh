@@ -93,7 +93,10 @@ constexpr uint32_t MAX_QUERIES = 65536;
 constexpr uint64_t HIT_BYTES = 24;  // device bytes budgeted per raw hit of a query chunk
 
 // --------------------------------------------------------- device memory --
-// Stream-ordered allocations from the device's default memory pool.
+// Stream-ordered allocations from the device's default memory pool.  Small requests share
+// blocks of ARENA_BLOCK bytes (a search makes some forty, most of them of a few KB); each
+// request counts as one for the counters and for fault injection.
+constexpr size_t ARENA_BLOCK = 1 << 20, ARENA_SMALL = 1 << 17;
 class DeviceArena {
 public:
     explicit DeviceArena(cudaStream_t s) : stream_(s) {}
@@ -104,8 +107,54 @@ public:
     cudaStream_t stream() const { return stream_; }
 
 private:
+    void *raw(size_t bytes);
     cudaStream_t stream_;
     std::vector<void *> ptrs_;
+    unsigned char *block_ = nullptr;  // the current block, block_left_ bytes of it unused
+    size_t block_left_ = 0;
+    int64_t requests_ = 0;
+};
+
+// Pinned host blocks and timing events that a handle's searches reuse: at most KEEP of each are
+// kept, the others are freed when they are given back.  For any thread.
+class HostPool {
+public:
+    ~HostPool() { clear(); }
+    void *take_pinned(size_t bytes, size_t *got);
+    void give_pinned(void *p, size_t bytes);
+    cudaEvent_t take_event();  // nullptr if none can be made
+    void give_event(cudaEvent_t e);
+    void clear();
+
+private:
+    static constexpr size_t KEEP_PINNED = 8, KEEP_EVENTS = 128, KEEP_BYTES = 1 << 20;
+    std::mutex mu_;
+    std::vector<std::pair<void *, size_t>> pinned_;
+    std::vector<cudaEvent_t> events_;
+};
+struct PinnedBlock {  // stream: the one that copies into it; it is given back with no copy in flight
+    HostPool &pool;
+    cudaStream_t stream;
+    size_t bytes = 0;
+    unsigned char *p;
+    bool in_flight = false;
+    PinnedBlock(HostPool &pl, size_t n, cudaStream_t s) : pool(pl), stream(s) {
+        p = static_cast<unsigned char *>(pl.take_pinned(n, &bytes));
+    }
+    void fetch(size_t at, const void *dev, size_t n) {
+        in_flight = true;
+        GN_CUDA(cudaMemcpyAsync(p + at, dev, n, cudaMemcpyDeviceToHost, stream));
+    }
+    void wait() {
+        GN_CUDA(cudaStreamSynchronize(stream));
+        in_flight = false;
+    }
+    ~PinnedBlock() {
+        if (in_flight) cudaStreamSynchronize(stream);
+        pool.give_pinned(p, bytes);
+    }
+    PinnedBlock(const PinnedBlock &) = delete;
+    PinnedBlock &operator=(const PinnedBlock &) = delete;
 };
 
 void configure_mempool(int device);
@@ -181,8 +230,11 @@ int bits_for(uint64_t max_value);  // bits needed to hold values in [0, max_valu
 
 int num_sms();
 
-// Compacts records whose flag is non-zero, keeping their order; returns the count
-// (synchronizes the stream to read it).
+// Compacts records whose flag is non-zero, keeping their order; returns where the device finds
+// the count.
+const uint64_t *compact_records_async(const uint32_t *in, int rec_words, const uint32_t *flags, uint32_t n, uint32_t *out,
+                                      DeviceArena &arena, cudaStream_t s);
+// The same, and reads the count (synchronizes the stream).
 uint32_t compact_records(const uint32_t *in, int rec_words, const uint32_t *flags, uint32_t n, uint32_t *out,
                          DeviceArena &arena, cudaStream_t s);
 
@@ -338,6 +390,7 @@ struct gn_index {
     };
     std::vector<KernelStat> last_kernels;
     std::mutex phase_mu;
+    gn::HostPool host_pool;
 };
 
 struct gn_results {

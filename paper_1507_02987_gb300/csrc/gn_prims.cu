@@ -51,11 +51,7 @@ void debug_fail_alloc(uint64_t nth) { g_fail_alloc_in.store(nth); }
 uint64_t debug_alloc_count() { return g_alloc_count.load(); }
 int64_t debug_live_allocs() { return g_live_allocs.load(); }
 
-void *DeviceArena::alloc(size_t bytes) {
-    uint64_t v = g_fail_alloc_in.load();
-    while (v && !g_fail_alloc_in.compare_exchange_weak(v, v - 1)) {
-    }
-    if (v == 1) throw Error{GN_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed (injected)"};
+void *DeviceArena::raw(size_t bytes) {
     void *p = nullptr;
     cudaError_t e = cudaMallocAsync(&p, bytes ? bytes : 1, stream_);
     if (e != cudaSuccess) {
@@ -64,6 +60,28 @@ void *DeviceArena::alloc(size_t bytes) {
                                    cudaGetErrorString(e)};
     }
     ptrs_.push_back(p);
+    return p;
+}
+
+void *DeviceArena::alloc(size_t bytes) {
+    uint64_t v = g_fail_alloc_in.load();
+    while (v && !g_fail_alloc_in.compare_exchange_weak(v, v - 1)) {
+    }
+    if (v == 1) throw Error{GN_ENOMEM, "device allocation of " + std::to_string(bytes) + " bytes failed (injected)"};
+    void *p;
+    const size_t want = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
+    if (want <= ARENA_SMALL) {
+        if (want > block_left_) {
+            block_ = static_cast<unsigned char *>(raw(ARENA_BLOCK));
+            block_left_ = ARENA_BLOCK;
+        }
+        p = block_;
+        block_ += want;
+        block_left_ -= want;
+    } else {
+        p = raw(bytes);
+    }
+    ++requests_;
     g_alloc_count.fetch_add(1);
     g_live_allocs.fetch_add(1);
     return p;
@@ -71,8 +89,72 @@ void *DeviceArena::alloc(size_t bytes) {
 
 void DeviceArena::release() {
     for (void *p : ptrs_) cudaFreeAsync(p, stream_);
-    g_live_allocs.fetch_sub((int64_t)ptrs_.size());
+    g_live_allocs.fetch_sub(requests_);
     ptrs_.clear();
+    requests_ = 0;
+    block_ = nullptr;
+    block_left_ = 0;
+}
+
+void *HostPool::take_pinned(size_t bytes, size_t *got) {
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        for (size_t i = 0; i < pinned_.size(); ++i)
+            if (pinned_[i].second >= bytes) {
+                void *p = pinned_[i].first;
+                *got = pinned_[i].second;
+                pinned_.erase(pinned_.begin() + (long)i);
+                return p;
+            }
+    }
+    void *p = nullptr;
+    *got = std::max<size_t>(bytes, 1 << 16);
+    GN_CUDA(cudaHostAlloc(&p, *got, cudaHostAllocDefault));
+    return p;
+}
+
+void HostPool::give_pinned(void *p, size_t bytes) {
+    if (!p) return;
+    if (bytes <= KEEP_BYTES) {
+        std::lock_guard<std::mutex> lk(mu_);
+        if (pinned_.size() < KEEP_PINNED) {
+            pinned_.emplace_back(p, bytes);
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
+cudaEvent_t HostPool::take_event() {
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        if (!events_.empty()) {
+            cudaEvent_t e = events_.back();
+            events_.pop_back();
+            return e;
+        }
+    }
+    cudaEvent_t e = nullptr;
+    return cudaEventCreate(&e) == cudaSuccess ? e : nullptr;
+}
+
+void HostPool::give_event(cudaEvent_t e) {
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        if (events_.size() < KEEP_EVENTS) {
+            events_.push_back(e);
+            return;
+        }
+    }
+    cudaEventDestroy(e);
+}
+
+void HostPool::clear() {
+    std::lock_guard<std::mutex> lk(mu_);
+    for (auto &b : pinned_) cudaFreeHost(b.first);
+    for (cudaEvent_t e : events_) cudaEventDestroy(e);
+    pinned_.clear();
+    events_.clear();
 }
 
 // --------------------------------------------------------------- packing --

@@ -12,7 +12,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <cstddef>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
 
@@ -1131,15 +1133,32 @@ __global__ void k_stitch_sweep(const DevHsp *__restrict__ in, uint32_t n, uint32
 // other indices are flagged 0.
 __device__ __forceinline__ uint64_t ov_key(const DevHsp &h) { return ((uint64_t)h.ds << 32) | h.qe; }
 
-__global__ void k_overlap_sweep(const DevHsp *__restrict__ in, uint32_t n, DevHsp *__restrict__ out,
-                                uint32_t *__restrict__ flag) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t qi = in[i].qi, seq = in[i].seq;
-    if (i > 0 && in[i - 1].qi == qi && in[i - 1].seq == seq) return;  // not the head of a run
+// The sweep of the run that starts at record i (rec(j): record j of n); boxes go to out and flag
+// from i on.  With in_order, boxes of one run that begin at the same qs are put in (ds, qe, de)
+// order (a later box can reach further back in the bank than an earlier one), the order by
+// which equally long ones are selected.  Returns the index after the run.
+template <class Rec, class Flag>
+__device__ __forceinline__ uint32_t overlap_run(Rec rec, uint32_t i, uint32_t n, DevHsp *__restrict__ out, Flag set_flag,
+                                                bool in_order) {
+    DevHsp first = rec(i);
+    const uint32_t qi = first.qi, seq = first.seq;
     uint32_t o = i;  // next box slot
     bool open = false;
     DevHsp box{};  // set by the run's first record
+    auto put = [&]() {
+        box.len = min(box.qe - box.qs, box.de - box.ds);
+        uint32_t at = o++;
+        set_flag(at, 1u);
+        if (in_order) {
+            while (at > i) {
+                const DevHsp p = out[at - 1];
+                const uint64_t kp = ((uint64_t)p.ds << 32) | p.qe, kb = ((uint64_t)box.ds << 32) | box.qe;
+                if (p.qs != box.qs || kp < kb || (kp == kb && p.de <= box.de)) break;
+                out[at--] = p;
+            }
+        }
+        out[at] = box;
+    };
     auto visit = [&](const DevHsp &h) {
         if (open && h.qs < box.qe && box.qs < h.qe && h.ds < box.de && box.ds < h.de) {
             box.qs = min(box.qs, h.qs);
@@ -1148,21 +1167,26 @@ __global__ void k_overlap_sweep(const DevHsp *__restrict__ in, uint32_t n, DevHs
             box.de = max(box.de, h.de);
             return;
         }
-        if (open) {
-            box.len = min(box.qe - box.qs, box.de - box.ds);
-            out[o] = box;
-            flag[o++] = 1;
-        }
+        if (open) put();
         box = h;
         open = true;
     };
     uint32_t g0 = i;
-    while (g0 < n && in[g0].qi == qi && in[g0].seq == seq) {
-        const uint32_t qs = in[g0].qs;
+    DevHsp cur = first;
+    for (;;) {
+        // the group of records at cur's qs: [g0, g1); next: the record after it, if in the run
         uint32_t g1 = g0 + 1;
-        while (g1 < n && in[g1].qi == qi && in[g1].seq == seq && in[g1].qs == qs) ++g1;
+        DevHsp next{};
+        bool more = false;
+        while (g1 < n) {
+            next = rec(g1);
+            more = next.qi == qi && next.seq == seq;
+            if (!more || next.qs != cur.qs) break;
+            ++g1;
+            more = false;
+        }
         if (g1 - g0 == 1) {
-            visit(in[g0]);
+            visit(cur);
         } else {
             // the group's records by increasing (ds, qe), then index: each step takes the
             // smallest (key, index) above the last one taken
@@ -1172,38 +1196,48 @@ __global__ void k_overlap_sweep(const DevHsp *__restrict__ in, uint32_t n, DevHs
                 uint64_t best_k = ~0ull;
                 uint32_t best_j = g1;
                 for (uint32_t j = g0; j < g1; ++j) {
-                    const uint64_t kj = ov_key(in[j]);
+                    const uint64_t kj = ov_key(rec(j));
                     const bool after = t == g0 || kj > last_k || (kj == last_k && j > last_j);
                     if (after && (kj < best_k || (kj == best_k && j < best_j))) {
                         best_k = kj;
                         best_j = j;
                     }
                 }
-                visit(in[best_j]);
+                visit(rec(best_j));
                 last_k = best_k;
                 last_j = best_j;
             }
         }
         g0 = g1;
+        if (!more) break;
+        cur = next;
     }
-    box.len = min(box.qe - box.qs, box.de - box.ds);
-    out[o] = box;
-    flag[o++] = 1;
-    for (uint32_t j = o; j < g0; ++j) flag[j] = 0;
+    put();
+    for (uint32_t j = o; j < g0; ++j) set_flag(j, 0u);
+    return g0;
+}
+
+__global__ void k_overlap_sweep(const DevHsp *__restrict__ in, uint32_t n, DevHsp *__restrict__ out,
+                                uint32_t *__restrict__ flag, int in_order) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    if (i > 0 && in[i - 1].qi == in[i].qi && in[i - 1].seq == in[i].seq) return;  // not the head of a run
+    overlap_run([&](uint32_t j) { return in[j]; }, i, n, out, [&](uint32_t j, uint32_t v) { flag[j] = v; }, in_order != 0);
 }
 
 // ----------------------------------------------------- a11: selection --
 // Per-query selection on records sorted by (qi, seq, qs, ds, qe, de): a block per
 // query keeps its N longest records, ties broken by that order (a stable choice by
 // length), and writes them by (length desc, seq, qs, ds, qe, de).  The N-th largest
-// length T comes from two 256-bin histograms (high and low byte of the length); the
-// selected records are those longer than T and the first ones of length T.
+// length T comes from a 256-bin histogram per byte of the length (two, or three where a
+// query is longer than 65,535 bases), high byte first; the selected records are those
+// longer than T and the first ones of length T.
 constexpr int SQ_CAP = 1024;  // largest N this kernel handles
 constexpr int SQ_THREADS = 512;
 
 __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__restrict__ rec,
                                                              const uint32_t *__restrict__ qfirst,
-                                                             const uint64_t *__restrict__ qout, uint32_t N,
+                                                             const uint64_t *__restrict__ qout, uint32_t N, int bytes,
                                                              DevHsp *__restrict__ sel) {
     __shared__ uint32_t hist[256];
     __shared__ uint32_t warp_tot[SQ_THREADS / 32];
@@ -1214,10 +1248,11 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
     const uint64_t out0 = qout[q];
     const uint32_t nsel = (uint32_t)(qout[q + 1] - out0);
     if (nsel == 0) return;
+    const uint32_t max_len = (1u << (8 * bytes)) - 1u;
     uint32_t T = 0, r_eq = n;  // n <= N: every record is selected
     if (n > N) {
-        uint32_t above = 0, hb = 0;
-        for (int level = 0; level < 2; ++level) {
+        uint32_t above = 0;
+        for (int shift = 8 * (bytes - 1); shift >= 0; shift -= 8) {  // T: its bytes so far
             for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
             __syncthreads();
             // one shared-memory atomic per distinct bin of a warp's 32 records (lengths are
@@ -1226,9 +1261,8 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
                 const uint32_t i = i0 + (threadIdx.x & 31u);
                 uint32_t bin = 256u;
                 if (i < b) {
-                    const uint32_t len = min(rec[i].len, 65535u);
-                    if (level == 0) bin = len >> 8;
-                    else if ((len >> 8) == hb) bin = len & 0xFFu;
+                    const uint32_t len = min(rec[i].len, max_len);
+                    if (((uint64_t)len >> (shift + 8)) == T) bin = (len >> shift) & 0xFFu;
                 }
                 const uint32_t peers = __match_any_sync(0xffffffffu, bin);
                 if (bin < 256u && (threadIdx.x & 31u) == (uint32_t)(__ffs(peers) - 1))
@@ -1239,12 +1273,12 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
                 uint32_t acc = above;
                 int x = 255;
                 while (acc + hist[x] < N) acc += hist[x--];
-                T_s = level == 0 ? (uint32_t)x : ((hb << 8) | (uint32_t)x);
+                T_s = (T << 8) | (uint32_t)x;
                 gt_s = acc;
             }
             __syncthreads();
-            if (level == 0) { hb = T_s; above = gt_s; }
-            else { T = T_s; above = gt_s; }
+            T = T_s;
+            above = gt_s;
             __syncthreads();
         }
         r_eq = N - above;  // records of length T to take, in array order
@@ -1257,7 +1291,7 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
     const uint32_t lo = min(n, threadIdx.x * per), hi = min(n, lo + per);
     uint32_t n_gt = 0, n_eq = 0;
     for (uint32_t i = lo; i < hi; ++i) {
-        const uint32_t len = min(rec[a + i].len, 65535u);
+        const uint32_t len = min(rec[a + i].len, max_len);
         const bool gt = n <= N || len > T;
         n_gt += gt ? 1u : 0u;
         n_eq += (!gt && len == T) ? 1u : 0u;
@@ -1267,12 +1301,12 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
     const uint32_t n_take = n_gt + min(n_eq, r_eq > eq_rank ? r_eq - eq_rank : 0u);
     uint32_t pos = block_excl_scan(n_take, warp_tot, tot);
     for (uint32_t i = lo; i < hi; ++i) {
-        const uint32_t len = min(rec[a + i].len, 65535u);
+        const uint32_t len = min(rec[a + i].len, max_len);
         const bool gt = n <= N || len > T;
         const bool eq = !gt && len == T;
         const bool take = gt || (eq && eq_rank < r_eq);
         eq_rank += eq ? 1u : 0u;
-        if (take) keys[pos++] = ((uint64_t)(65535u - len) << 32) | i;
+        if (take) keys[pos++] = ((uint64_t)(max_len - len) << 32) | i;
     }
     __syncthreads();
     // bitonic sort of the nsel keys (unique: they carry the position)
@@ -1307,13 +1341,93 @@ __device__ __forceinline__ uint32_t first_of_query(const DevHsp *__restrict__ re
     return lo;
 }
 
-__global__ void k_query_bounds(const DevHsp *__restrict__ rec, uint32_t n, uint32_t nq, uint32_t *__restrict__ first,
-                               uint32_t N, uint32_t *__restrict__ cnt) {
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+// n_dev: the number of records.  first64: the same as first, as a prefix sum of all records.
+__global__ void k_query_bounds(const DevHsp *__restrict__ rec, const uint64_t *__restrict__ n_dev, uint32_t nq,
+                               uint32_t *__restrict__ first, uint64_t *__restrict__ first64, uint32_t N,
+                               uint32_t *__restrict__ cnt) {
+    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x, n = (uint32_t)*n_dev;
     if (q > nq) return;
     const uint32_t f = first_of_query(rec, n, q);
     first[q] = f;
+    if (first64) first64[q] = f;
     if (cnt && q < nq) cnt[q] = min(N, first_of_query(rec, n, q + 1) - f);
+}
+
+// Overlap merging and query bounds of a small search in one block: sorts the records of up to
+// MB_CAP HSPs by (qi, seq, qs) (a key of at most 64 bits; ties keep their order, which the sweep
+// does not depend on), sweeps the runs, compacts the boxes and finds each query's first box,
+// and the prefix sums of min(N, boxes) (N = 0: of all boxes) as k_query_bounds and a scan do.
+// Replaces eight launches: a search of a handful of HSPs is a chain of launches of 2 to 5 us each.
+constexpr uint32_t MB_CAP = 2048, MB_QUERIES = 4096;
+constexpr int MB_THREADS = 512;
+
+__global__ void __launch_bounds__(MB_THREADS) k_merge_block(const DevHsp *__restrict__ in, uint32_t n, uint32_t seq_bits,
+                                                            uint32_t qs_bits, uint32_t nq, uint32_t N, int in_order,
+                                                            DevHsp *__restrict__ boxes, DevHsp *__restrict__ out,
+                                                            uint32_t *__restrict__ first, uint64_t *__restrict__ qo,
+                                                            uint64_t *__restrict__ n_out) {
+    __shared__ uint64_t key[MB_CAP];
+    __shared__ uint16_t idx[MB_CAP];
+    __shared__ uint8_t flag[MB_CAP];
+    __shared__ uint32_t warp_tot[MB_THREADS / 32];
+    uint32_t P = 32;
+    while (P < n) P <<= 1;
+    for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
+        uint64_t k = ~0ull;
+        if (i < n) k = ((((uint64_t)in[i].qi << seq_bits) | in[i].seq) << qs_bits) | in[i].qs;
+        key[i] = k;
+        idx[i] = i < n ? (uint16_t)i : (uint16_t)0xFFFFu;
+    }
+    __syncthreads();
+    for (uint32_t k2 = 2; k2 <= P; k2 <<= 1) {
+        for (uint32_t j = k2 >> 1; j > 0; j >>= 1) {
+            for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
+                const uint32_t x = i ^ j;
+                if (x > i) {
+                    const uint64_t a = key[i], b = key[x];
+                    const uint16_t ia = idx[i], ib = idx[x];
+                    if ((a > b || (a == b && ia > ib)) == ((i & k2) == 0)) {
+                        key[i] = b; key[x] = a;
+                        idx[i] = ib; idx[x] = ia;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        if (i > 0 && key[i - 1] >> qs_bits == key[i] >> qs_bits) continue;
+        overlap_run([&](uint32_t j) { return in[idx[j]]; }, i, n, boxes,
+                    [&](uint32_t j, uint32_t v) { flag[j] = (uint8_t)v; }, in_order != 0);
+    }
+    __syncthreads();
+    uint32_t n_mg = 0;
+    for (uint32_t i0 = 0; i0 < n; i0 += blockDim.x) {
+        const uint32_t i = i0 + threadIdx.x, f = i < n ? flag[i] : 0u;
+        uint32_t tot = 0;
+        const uint32_t at = n_mg + block_excl_scan(f, warp_tot, tot);
+        if (f) out[at] = boxes[i];
+        n_mg += tot;
+    }
+    __syncthreads();
+    uint64_t sum = 0;
+    for (uint32_t q0 = 0; q0 <= nq; q0 += blockDim.x) {
+        const uint32_t q = q0 + threadIdx.x;
+        uint32_t c = 0;
+        if (q <= nq) {
+            const uint32_t f = first_of_query(out, n_mg, q);
+            first[q] = f;
+            if (q < nq) {
+                c = first_of_query(out, n_mg, q + 1) - f;
+                if (N) c = min(N, c);
+            }
+        }
+        uint32_t tot = 0;
+        const uint32_t at = block_excl_scan(c, warp_tot, tot);
+        if (q <= nq) qo[q] = sum + at;
+        sum += tot;
+    }
+    if (threadIdx.x == 0) *n_out = n_mg;
 }
 
 __global__ void k_first_of_query(const uint32_t *__restrict__ recs, int W, uint32_t n, uint32_t *__restrict__ first) {
@@ -1366,8 +1480,8 @@ __device__ __forceinline__ int64_t dev_band(const DevHsp &h, int32_t w) {
 
 // One HSP aligned by a whole warp on the strip path (bands wider than the register paths hold):
 // the band in chunks of 32 offsets, the previous row in scratch.
-__device__ void sw_task_strip(const DevHsp *__restrict__ sel, uint32_t task, const uint64_t *__restrict__ strip_off,
-                              SwCell *__restrict__ strips, const uint32_t *__restrict__ qpk,
+__device__ void sw_task_strip(const DevHsp *__restrict__ sel, uint32_t task, SwCell *__restrict__ row,
+                              const uint32_t *__restrict__ qpk,
                               const uint32_t *__restrict__ qnb, const uint64_t *__restrict__ qstart,
                               const uint32_t *__restrict__ bpk, const uint32_t *__restrict__ bnb,
                               const uint64_t *__restrict__ seq_start, int32_t match, int32_t mismatch, int32_t go,
@@ -1388,7 +1502,6 @@ __device__ void sw_task_strip(const DevHsp *__restrict__ sel, uint32_t task, con
         if (lane == 0) { atomicOr(status, DEV_ERR_BAND_TOO_WIDE); out[task] = res; }
         return;
     }
-    SwCell *row = strips + strip_off[task];
     int32_t best = 0;
     int64_t bi = INT64_MAX, bj = INT64_MAX;
     uint32_t bs = 0;
@@ -1753,6 +1866,13 @@ __device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const PackedPa
     sw_finish<G>(x.best, x.bcell, x.bstart, h, on, w, res);
 }
 
+// What the number of alignments, known on the device only, decides: see the alignment kernels'
+// launch in search().
+__device__ __forceinline__ bool sw_many(uint32_t n, uint32_t sms) { return n > sms * 64u; }
+__device__ __forceinline__ uint32_t sw_long_rows(uint32_t n, uint32_t sms) {
+    return n <= sms * 4u ? 1u : sw_many(n, sms) ? 1024u : 512u;
+}
+
 // Alignments of the selected HSPs, longest first (order): the first n_long tasks a warp each
 // (32 lanes with two offsets: the shortest rows, for the alignments that would bound the
 // kernel's time), the others 32 / G to a warp.  Bands over 64 diagonals (and windows of
@@ -1760,20 +1880,22 @@ __device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const PackedPa
 // 40 diagonals (33 and up at the default width), <16, 2, 1> 48; k_sw_prepare counts tasks with
 // wider bands, up to 64, among the long ones.
 template <int G, int KA, int KB, bool CUT>
-__global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ sel, uint32_t n, PackedPair q,
+__global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ sel, const uint64_t *__restrict__ n_dev,
+                                                   uint32_t sms, PackedPair q,
                                                    const uint64_t *__restrict__ qstart,
                                                    const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
-                                                   uint32_t *__restrict__ next_task, const uint64_t *__restrict__ order,
+                                                   uint32_t *__restrict__ next_task, const uint32_t *__restrict__ order,
                                                    uint32_t *__restrict__ wide, uint32_t *__restrict__ wide_count,
                                                    const uint32_t *__restrict__ n_long, uint32_t *__restrict__ next_long,
                                                    DevAln *__restrict__ out) {
     const int lane = threadIdx.x & 31, seg = lane / G;
-    const uint32_t nl = *n_long;
+    const uint32_t n = (uint32_t)*n_dev, nl = order ? *n_long : n;  // no order: a warp each
+    if (!sw_many(n, sms) && blockIdx.x >= sms) return;  // four warps an SM (see the launch)
     // the task at place j of the order, if a register path of `cap` offsets takes it; wider ones
     // are listed by the lane `lists`
     auto take = [&](uint32_t j, uint32_t end, int cap, bool lists, uint32_t &task, DevHsp &h) {
         if (j >= end) return false;
-        task = (uint32_t)order[j];
+        task = order ? order[j] : j;
         h = sel[task];
         const int64_t rows = (int64_t)h.qe - h.qs + 2 * (int64_t)w;
         if (dev_band(h, w) <= cap && rows <= SW_MAX_ROWS) return true;
@@ -1808,17 +1930,17 @@ __global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ se
     }
 }
 
-// Bands wider than 64 diagonals, a warp each: up to SW_MAX_BAND offsets in registers, wider ones
-// on the strip path.  A kernel of its own, so that its registers do not limit the main
-// alignment kernel.
+// Bands wider than 64 diagonals, a warp each: up to SW_MAX_BAND offsets in registers; still
+// wider ones are listed, with the widest band, for k_banded_sw_strip.  A kernel of its own, so
+// that its registers do not limit the main alignment kernel.
 template <bool CUT>
 __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict__ sel, const uint32_t *__restrict__ wide,
                                                         const uint32_t *__restrict__ wide_count,
-                                                        uint32_t *__restrict__ next, const uint64_t *__restrict__ strip_off,
-                                                        SwCell *__restrict__ strips, PackedPair q,
+                                                        uint32_t *__restrict__ next, PackedPair q,
                                                         const uint64_t *__restrict__ qstart,
                                                         const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
-                                                        DevAln *__restrict__ out, uint32_t *__restrict__ status) {
+                                                        uint32_t *__restrict__ strip, uint32_t *__restrict__ strip_count,
+                                                        uint32_t *__restrict__ strip_band, DevAln *__restrict__ out) {
     const int lane = threadIdx.x & 31;
     const uint32_t n = *wide_count;
     for (;;) {
@@ -1828,47 +1950,111 @@ __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict
         if (j >= n) return;
         const uint32_t task = wide[j];
         const DevHsp h = sel[task];
-        if (dev_band(h, w) <= SW_MAX_BAND && (int64_t)h.qe - h.qs + 2 * (int64_t)w <= SW_MAX_ROWS) {
+        const int64_t B = dev_band(h, w);
+        if (B <= SW_MAX_BAND && (int64_t)h.qe - h.qs + 2 * (int64_t)w <= SW_MAX_ROWS) {
             DevAln res;
             sw_band<32, 5, 4, CUT>(h, true, q, qstart, seq_start, c, w, res);
             if (lane == 0) out[task] = res;
-        } else {
-            sw_task_strip(sel, task, strip_off, strips, q.qpk, q.qnb, qstart, q.bpk, q.bnb, seq_start, c.match, c.mismatch,
-                          c.goe - c.ge, c.ge, w, out, status);
+        } else if (lane == 0) {
+            strip[atomicAdd(strip_count, 1u)] = task;
+            atomicMax(strip_band, (uint32_t)min(B, (int64_t)65536));
         }
         __syncwarp();
     }
 }
 
-// Preparation of the alignment phase, per selected HSP:
-// - the strip length of its band (B + 1), and the band area (DP-window rows x B, the cells
-//   the alignment kernels evaluate) summed into cells[0] (bands of at most 64 diagonals) or
-//   cells[1] (wider bands);
-// - its alignment-order key (65535 - DP-window rows) << 32 | task, so that an ascending sort
-//   on bits 32..47 hands out the longest alignments first (they bound the kernel's time) and
-//   groups alignments of similar length; alignments of at least long_rows rows, and those
-//   whose bands are wider than the grouped path's `cap` offsets, are counted in *n_long (they
-//   sort first).
-__global__ void k_sw_prepare(const DevHsp *__restrict__ h, uint32_t n, int32_t w, int cap,
-                             const uint64_t *__restrict__ qstart, uint32_t *__restrict__ B, unsigned long long *__restrict__ cells, uint32_t long_rows,
-                             uint64_t *__restrict__ keys, uint32_t *__restrict__ n_long) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in = i < n;
-    int64_t rows = 0;
-    if (in) {
-        const DevHsp x = h[i];
-        const int64_t d_s = (int64_t)x.ds - x.qs, d_e = (int64_t)x.de - x.qe;
-        const int64_t b = (max(d_s, d_e) + w) - (min(d_s, d_e) - w) + 1;
-        B[i] = (uint32_t)min(b + 1, (int64_t)65537);  // +1: the strip is read at b + 1
-        const int64_t m = (int64_t)(qstart[x.qi + 1] - qstart[x.qi]);
-        rows = min(m, (int64_t)x.qe + w) - max((int64_t)0, (int64_t)x.qs - w);
-        if (rows > 0) atomicAdd(cells + (b > 64 ? 1 : 0), (unsigned long long)(rows * b));
-        if (b > cap && b <= 64) rows = 65535;
-        const int64_t r = rows < 0 ? 0 : (rows > 65535 ? 65535 : rows);
-        keys[i] = ((uint64_t)(65535 - (uint32_t)r) << 32) | i;
+// The listed alignments on the strip path, each warp with a strip of strip_cells cells.
+__global__ void __launch_bounds__(128) k_banded_sw_strip(const DevHsp *__restrict__ sel, const uint32_t *__restrict__ strip,
+                                                         uint32_t n, uint32_t *__restrict__ next,
+                                                         SwCell *__restrict__ strips, uint64_t strip_cells, PackedPair q,
+                                                         const uint64_t *__restrict__ qstart,
+                                                         const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
+                                                         DevAln *__restrict__ out, uint32_t *__restrict__ status) {
+    const int lane = threadIdx.x & 31;
+    SwCell *row = strips + (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * strip_cells;
+    for (;;) {
+        uint32_t j = 0;
+        if (lane == 0) j = atomicAdd(next, 1u);
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= n) return;
+        sw_task_strip(sel, strip[j], row, q.qpk, q.qnb, qstart, q.bpk, q.bnb, seq_start, c.match, c.mismatch, c.goe - c.ge,
+                      c.ge, w, out, status);
+        __syncwarp();
     }
-    const uint32_t lng = __ballot_sync(0xffffffffu, in && rows >= (int64_t)min(long_rows, 65535u));
-    if ((threadIdx.x & 31) == 0 && lng) atomicAdd(n_long, (uint32_t)__popc(lng));
+}
+
+// Alignment order: the longest first (they bound the phase's time), alignments of similar
+// length together.  Each task falls in one of SWO_BINS bins by its DP-window rows, four a
+// factor of two, falling; the first half of the bins takes the tasks that get a warp each: those
+// of at least long_rows rows, and those whose bands are wider than the grouped path's `cap`
+// offsets, up to 64.  k_sw_prepare counts the bins (hist) and, for the kernel times, the band
+// area (rows x band, the cells the alignment kernels evaluate) of bands of at most 64 diagonals
+// and of wider ones; k_sw_order places each task after the bins before its own.
+constexpr int SWO_BINS = 128;
+
+__device__ __forceinline__ uint32_t sw_bin(const DevHsp &x, int32_t w, int cap, const uint64_t *__restrict__ qstart,
+                                           uint32_t long_rows, int64_t &rows) {
+    const int64_t m = (int64_t)(qstart[x.qi + 1] - qstart[x.qi]), b = dev_band(x, w);
+    rows = max(min(m, (int64_t)x.qe + w) - max((int64_t)0, (int64_t)x.qs - w), (int64_t)0);
+    const uint32_t r = (uint32_t)min(rows, (int64_t)65535);
+    const int e = 31 - __clz(r | 1u);  // 0 .. 15
+    const uint32_t quarter = e >= 2 ? (r >> (e - 2)) & 3u : (r << (2 - e)) & 3u;
+    const uint32_t bin = 63u - (uint32_t)(4 * e) - quarter;
+    return (r >= long_rows || (b > cap && b <= 64)) ? bin : bin + 64u;
+}
+
+__global__ void __launch_bounds__(256) k_sw_prepare(const DevHsp *__restrict__ h, const uint64_t *__restrict__ n_dev,
+                                                    int32_t w, int cap, const uint64_t *__restrict__ qstart,
+                                                    uint32_t long_rows, uint32_t sms, uint32_t *__restrict__ hist,
+                                                    unsigned long long *__restrict__ cells) {
+    __shared__ uint32_t s_hist[SWO_BINS];
+    const uint32_t n = (uint32_t)*n_dev, i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x * blockDim.x >= n) return;
+    if (!long_rows) long_rows = sw_long_rows(n, sms);
+    for (int j = threadIdx.x; j < SWO_BINS; j += blockDim.x) s_hist[j] = 0u;
+    __syncthreads();
+    if (i < n) {
+        const DevHsp x = h[i];
+        int64_t rows;
+        atomicAdd(&s_hist[sw_bin(x, w, cap, qstart, long_rows, rows)], 1u);
+        if (cells && rows) {
+            const int64_t b = dev_band(x, w);
+            atomicAdd(cells + (b > 64 ? 1 : 0), (unsigned long long)(rows * b));
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < SWO_BINS; j += blockDim.x)
+        if (s_hist[j]) atomicAdd(&hist[j], s_hist[j]);
+}
+
+__global__ void __launch_bounds__(256) k_sw_order(const DevHsp *__restrict__ h, const uint64_t *__restrict__ n_dev,
+                                                  int32_t w, int cap, const uint64_t *__restrict__ qstart,
+                                                  uint32_t long_rows, uint32_t sms, const uint32_t *__restrict__ hist,
+                                                  uint32_t *__restrict__ placed, uint32_t *__restrict__ order,
+                                                  uint32_t *__restrict__ n_long) {
+    __shared__ uint32_t base[SWO_BINS], count[SWO_BINS], warp_tot[8];
+    const uint32_t n = (uint32_t)*n_dev, i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x * blockDim.x >= n) return;
+    if (!long_rows) long_rows = sw_long_rows(n, sms);
+    uint32_t tot = 0;
+    const uint32_t before = block_excl_scan(threadIdx.x < SWO_BINS ? hist[threadIdx.x] : 0u, warp_tot, tot);
+    if (threadIdx.x < SWO_BINS) {
+        base[threadIdx.x] = before;
+        count[threadIdx.x] = 0u;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == SWO_BINS / 2) *n_long = before;
+    __syncthreads();
+    uint32_t bin = 0, rank = 0;
+    if (i < n) {
+        int64_t rows;
+        bin = sw_bin(h[i], w, cap, qstart, long_rows, rows);
+        rank = atomicAdd(&count[bin], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < SWO_BINS && count[threadIdx.x])
+        base[threadIdx.x] += atomicAdd(&placed[threadIdx.x], count[threadIdx.x]);
+    __syncthreads();
+    if (i < n) order[base[bin] + rank] = i;
 }
 
 // ------------------------------------------------------ a13: ranking --
@@ -1951,18 +2137,24 @@ __device__ void rq_bitonic(uint16_t *idx, const DevAln *rec, const uint8_t *keep
     }
 }
 
-__global__ void __launch_bounds__(256) k_rank_query(const DevAln *__restrict__ aln, const uint32_t *__restrict__ qrange,
+// qo: first alignment of each query, as a prefix sum.  A query of more than RQ_CAP alignments is
+// left out and *too_many set: the caller then ranks the call by sorting.
+__global__ void __launch_bounds__(256) k_rank_query(const DevAln *__restrict__ aln, const uint64_t *__restrict__ qo,
                                                     uint32_t nq, const uint64_t *__restrict__ qstart, double n_bank,
                                                     double lambda, double K, double max_e, gn_hit *__restrict__ out,
-                                                    uint32_t *__restrict__ qcount) {
+                                                    uint32_t *__restrict__ qcount, uint32_t *__restrict__ too_many) {
     __shared__ DevAln rec[RQ_CAP];
     __shared__ uint16_t idx[RQ_CAP];
     __shared__ uint8_t keep[RQ_CAP];
     __shared__ uint32_t nk_s, ne_s;
     for (uint32_t q = blockIdx.x; q < nq; q += gridDim.x) {
-        const uint32_t start = qrange[2 * q], n = qrange[2 * q + 1] - start;
-        if (n == 0) {
-            if (threadIdx.x == 0) qcount[q] = 0;
+        const uint64_t start = qo[q];
+        const uint32_t n = (uint32_t)(qo[q + 1] - start);
+        if (n == 0 || n > RQ_CAP) {
+            if (threadIdx.x == 0) {
+                qcount[q] = 0;
+                if (n) *too_many = 1u;
+            }
             continue;
         }
         uint32_t P = 1;
@@ -2008,19 +2200,10 @@ __global__ void __launch_bounds__(256) k_rank_query(const DevAln *__restrict__ a
     }
 }
 
-__global__ void k_query_ranges(const DevAln *__restrict__ a, uint32_t n, uint32_t *__restrict__ qrange) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t q = a[i].qi;
-    if (i == 0 || a[i - 1].qi != q) qrange[2 * q] = i;
-    if (i == n - 1 || a[i + 1].qi != q) qrange[2 * q + 1] = i + 1;
-}
-
-__global__ void k_gather_ranked(const gn_hit *__restrict__ in, const uint32_t *__restrict__ qrange,
+__global__ void k_gather_ranked(const gn_hit *__restrict__ in, const uint64_t *__restrict__ from,
                                 const uint64_t *__restrict__ qoff, uint32_t nq, gn_hit *__restrict__ out) {
     for (uint32_t q = blockIdx.x; q < nq; q += gridDim.x) {
-        const uint32_t start = qrange[2 * q];
-        const uint64_t o = qoff[q], c = qoff[q + 1] - o;
+        const uint64_t start = from[q], o = qoff[q], c = qoff[q + 1] - o;
         for (uint32_t k = threadIdx.x; k < c; k += blockDim.x) out[o + k] = in[start + k];
     }
 }
@@ -2034,17 +2217,24 @@ __global__ void k_scatter_flagged(const uint32_t *__restrict__ in, int W, const 
     if (flags[i]) out[pos[i] * W + w] = in[t];
 }
 
+const uint64_t *compact_records_async(const uint32_t *in, int W, const uint32_t *flags, uint32_t n, uint32_t *out,
+                                      DeviceArena &arena, cudaStream_t s) {
+    uint64_t *pos = arena.alloc_n<uint64_t>(n + 1ull);
+    void *scr = arena.alloc(scan_scratch_bytes(n));
+    exclusive_scan_u32(flags, pos, n, scr, s);
+    const uint64_t tot = (uint64_t)n * W;
+    if (n)
+        GN_LAUNCH("k_scatter_flagged", n, s,
+                  k_scatter_flagged<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(in, W, flags, pos, n, out));
+    return pos + n;
+}
+
 uint32_t compact_records(const uint32_t *in, int W, const uint32_t *flags, uint32_t n, uint32_t *out,
                          DeviceArena &arena, cudaStream_t s) {
     if (n == 0) return 0;
-    uint64_t *pos = arena.alloc_n<uint64_t>(n + 1);
-    void *scr = arena.alloc(scan_scratch_bytes(n));
-    exclusive_scan_u32(flags, pos, n, scr, s);
-    uint64_t tot = (uint64_t)n * W;
-    GN_LAUNCH("k_scatter_flagged", n, s,
-              k_scatter_flagged<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(in, W, flags, pos, n, out));
+    const uint64_t *count = compact_records_async(in, W, flags, n, out, arena, s);
     uint64_t cnt = 0;
-    GN_CUDA(cudaMemcpyAsync(&cnt, pos + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    GN_CUDA(cudaMemcpyAsync(&cnt, count, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     GN_CUDA(cudaStreamSynchronize(s));
     return (uint32_t)cnt;
 }
@@ -2053,11 +2243,12 @@ uint32_t compact_records(const uint32_t *in, int W, const uint32_t *flags, uint3
 namespace {
 struct PhaseTimer {
     cudaStream_t s;
+    HostPool &pool;
     std::vector<std::pair<const char *, cudaEvent_t>> marks;
-    explicit PhaseTimer(cudaStream_t st) : s(st) {}
+    PhaseTimer(cudaStream_t st, HostPool &pl) : s(st), pool(pl) {}
     void mark(const char *name) {
-        cudaEvent_t e;
-        if (cudaEventCreate(&e) != cudaSuccess) return;
+        cudaEvent_t e = pool.take_event();
+        if (!e) return;
         cudaEventRecord(e, s);
         marks.emplace_back(name, e);
     }
@@ -2070,7 +2261,7 @@ struct PhaseTimer {
         }
     }
     ~PhaseTimer() {
-        for (auto &m : marks) cudaEventDestroy(m.second);
+        for (auto &m : marks) pool.give_event(m.second);
     }
 };
 
@@ -2082,6 +2273,23 @@ std::vector<T> to_host(const T *d, size_t n, cudaStream_t s) {
         GN_CUDA(cudaStreamSynchronize(s));
     }
     return h;
+}
+
+// Resident blocks of a kernel without dynamic shared memory, asked of the driver once per kernel
+// and device (a search asks for five).
+int blocks_per_sm(const void *fn, int threads) {
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, int> known;
+    int dev = 0;
+    GN_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    int &n = known[{fn, dev}];
+    if (!n) {
+        int occ = 0;
+        GN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, 0));
+        n = std::max(occ, 1);
+    }
+    return n;
 }
 
 unsigned blocks_for(uint64_t n, unsigned t = 256) { return (unsigned)std::max<uint64_t>(1, (n + t - 1) / t); }
@@ -2157,6 +2365,29 @@ void both_strands(const uint8_t *qbases_dev, const std::vector<uint64_t> &qstart
     *out_bases = d;
 }
 
+// Words that a search's kernels write and its host code reads.
+struct SearchWords {
+    uint32_t wait_status, status;
+    uint32_t n_hsp, n_cand;            // HSPs and candidates of the signature scan
+    uint32_t next_tile, next_cand;
+    uint32_t n_wide, next_wide, next_task, n_long, next_long;
+    uint32_t n_strip, strip_band, next_strip;
+    uint32_t too_many, pad;
+    unsigned long long next_end, cells[2];
+    uint32_t bins[SWO_BINS], placed[SWO_BINS];
+};
+static_assert(sizeof(SearchWords) % 8 == 0, "SearchWords is followed by 64-bit words");
+
+// Segments of a query set: one per MAX_QUERY_LEN bases or part, SEG_STEP apart (see search).
+uint64_t count_segments(const std::vector<uint64_t> &qstart) {
+    uint64_t n = 0;
+    for (size_t i = 0; i + 1 < qstart.size(); ++i) {
+        const uint64_t m = qstart[i + 1] - qstart[i];
+        n += m <= MAX_QUERY_LEN ? 1 : 1 + (m - MAX_QUERY_LEN + SEG_STEP - 1) / SEG_STEP;
+    }
+    return n;
+}
+
 void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t> &qstart_h, const SearchOptions &o,
             cudaStream_t s, gn_results *res) {
     const uint32_t nq = (uint32_t)(qstart_h.size() - 1);
@@ -2168,7 +2399,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     const bool keep_hits = (p.flags & GN_FLAG_KEEP_HITS) != 0;
     res->n_queries = nq;
     res->has_stages = keep;
-    PhaseTimer timer(s);
+    PhaseTimer timer(s, ix->host_pool);
     timer.mark("start");
     KernelTimer ktimer;
     struct TimerScope {
@@ -2178,10 +2409,18 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     };
     TimerScope tscope((p.flags & GN_FLAG_TIME_KERNELS) ? &ktimer : nullptr);
     DeviceArena arena(s);
-    // bounded device-side waits (the scans' look-back) record a timeout here
-    uint32_t *wait_status = arena.alloc_n<uint32_t>(1);
-    GN_CUDA(cudaMemsetAsync(wait_status, 0, 4, s));
-    WaitStatusScope wscope(wait_status);
+    // What the host reads back while a search runs, and the counters its kernels work with, in one
+    // place that one memset clears: the words of SearchWords, the alignment order's bins, then the
+    // hits per query (or segment).
+    const uint64_t n_seg_max = count_segments(qstart_h);
+    GN_REQUIRE(n_seg_max <= MAX_QUERIES, GN_ETOOBIG, "more than 65,536 query segments in one call");
+    const size_t words_bytes = sizeof(SearchWords) + 8 * (n_seg_max + 1);
+    SearchWords *words = static_cast<SearchWords *>(arena.alloc(words_bytes));
+    GN_CUDA(cudaMemsetAsync(words, 0, words_bytes, s));
+    uint64_t *hq_d = reinterpret_cast<uint64_t *>(words + 1);
+    uint32_t *wait_status = &words->wait_status, *status = &words->status;
+    WaitStatusScope wscope(wait_status);  // bounded device-side waits (the scans' look-back) record a timeout there
+    PinnedBlock pin(ix->host_pool, std::max<size_t>(words_bytes, 1 << 16), s);
 #ifdef GN_CHECKS
     uint32_t *check_bits = nullptr;  // the failed device-side checks of this search
     GN_CUDA(cudaGetSymbolAddress(reinterpret_cast<void **>(&check_bits), g_check_bits));
@@ -2221,7 +2460,6 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
             segmented = true;
         }
     }
-    GN_REQUIRE(seg_parent.size() <= MAX_QUERIES, GN_ETOOBIG, "more than 65,536 query segments in one call");
     if (segmented) {
         GN_REQUIRE(p.max_hit_distance + (uint32_t)k <= SEG_OVERLAP, GN_EINVAL,
                    "queries over 65,535 bases need max_hit_distance + seed span <= 8,192");
@@ -2272,10 +2510,8 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     uint64_t *hoff = arena.alloc_n<uint64_t>(HM + 1);
     uint32_t *src = scan ? nullptr : arena.alloc_n<uint32_t>(HM);
     QueryRec *qrec = scan ? arena.alloc_n<QueryRec>(HM) : nullptr;
-    uint64_t *hq_d = arena.alloc_n<uint64_t>(hnq + 1);
     const int flank = (int)std::min<uint32_t>(SIG_FLANK_BASES, p.min_hsp_len > (uint32_t)k ? p.min_hsp_len - (uint32_t)k : 0u);
     if (scan) {
-        GN_CUDA(cudaMemsetAsync(hq_d, 0, 8 * (hnq + 1), s));
         auto kernel = kind == SIG_FLANK ? k_query_recs<SIG_FLANK> : k_query_recs<SIG_AHEAD>;
         if (HM)
             GN_LAUNCH("k_query_recs", HM, s,
@@ -2295,46 +2531,55 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     if (!scan)
         GN_LAUNCH("k_gather_u64", hnq + 1, s,
                   k_gather_u64<<<blocks_for(hnq + 1), 256, 0, s>>>(hoff, hstart_d, hnq + 1, hq_d));
-    std::vector<uint64_t> hq = to_host(hq_d, hnq + 1, s);
-    if (scan) {
-        uint64_t at = 0;
-        for (uint32_t i = 0; i <= hnq; ++i) {
-            const uint64_t h = hq[i];
-            GN_REQUIRE(i == hnq || h < (1ull << 32), GN_ETOOBIG, "a query has 2^32 seed hits or more");
-            hq[i] = at;
-            at += h;
+    // hits per query as prefix sums; the scan route reads them with its HSP count
+    std::vector<uint64_t> hq;
+    auto read_hits = [&](const uint64_t *from) {
+        hq.assign(from, from + hnq + 1);
+        if (scan) {
+            uint64_t at = 0;
+            for (uint32_t i = 0; i <= hnq; ++i) {
+                const uint64_t h = hq[i];
+                GN_REQUIRE(i == hnq || h < (1ull << 32), GN_ETOOBIG, "a query has 2^32 seed hits or more");
+                hq[i] = at;
+                at += h;
+            }
         }
+        GN_REQUIRE(!o.max_hit_bytes || hq[hnq] * HIT_BYTES <= o.max_hit_bytes, GN_ETOOBIG,
+                   "the query alone exceeds the server's memory budget");
+    };
+    if (!scan || g_ktimer) {
+        pin.fetch(0, hq_d, 8 * (hnq + 1));
+        pin.wait();
+        read_hits(reinterpret_cast<const uint64_t *>(pin.p));
     }
-    GN_REQUIRE(!o.max_hit_bytes || hq[hnq] * HIT_BYTES <= o.max_hit_bytes, GN_ETOOBIG,
-               "the query alone exceeds the server's memory budget");
     timer.mark("query_codes");
-    if (keep) {
-        res->st_hit_counts.resize(hnq);
-        for (uint32_t i = 0; i < hnq; ++i) res->st_hit_counts[i] = hq[i + 1] - hq[i];
-    }
 
     // a6-a8 per chunk of queries whose hits fit the budget
-    size_t free_b = 0, total_b = 0;
-    GN_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    // bytes per hit of a chunk: hit keys and their ping-pong buffer on the sort path, or the
-    // fixed-capacity buckets (up to ~22 B per hit without the repeat filter) and spill lists
-    uint64_t mem_for_hits = (uint64_t)(free_b * 0.55);
-    if (o.mem_cap) mem_for_hits = std::min(mem_for_hits, o.mem_cap);
-    // (a query chunk holds < 2^32 hits: the fill kernel indexes a tile's hits in 32 bits)
-    uint64_t hit_budget = std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1ull << 20, mem_for_hits / HIT_BYTES));
-    if (const char *e = getenv("GN_MAX_CHUNK_HITS")) {  // smaller chunks (exercises the multi-chunk path)
-        uint64_t v = strtoull(e, nullptr, 10);
-        if (v) hit_budget = std::min<uint64_t>(v, 0xFFFFFFFFull);
+    uint64_t hit_budget = 0;
+    if (!scan) {
+        size_t free_b = 0, total_b = 0;
+        GN_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        // bytes per hit of a chunk: hit keys and their ping-pong buffer on the sort path, or the
+        // fixed-capacity buckets (up to ~22 B per hit without the repeat filter) and spill lists
+        uint64_t mem_for_hits = (uint64_t)(free_b * 0.55);
+        if (o.mem_cap) mem_for_hits = std::min(mem_for_hits, o.mem_cap);
+        // (a query chunk holds < 2^32 hits: the fill kernel indexes a tile's hits in 32 bits)
+        hit_budget = std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1ull << 20, mem_for_hits / HIT_BYTES));
+        if (const char *e = getenv("GN_MAX_CHUNK_HITS")) {  // smaller chunks (exercises the multi-chunk path)
+            uint64_t v = strtoull(e, nullptr, 10);
+            if (v) hit_budget = std::min<uint64_t>(v, 0xFFFFFFFFull);
+        }
     }
     const uint64_t gbits_max = (uint64_t)bits_for(ix->n_bases + QBIAS);
     const uint32_t max_chunk_q = (uint32_t)std::min<uint64_t>(MAX_QUERIES, 1ull << std::min<uint64_t>(48 - gbits_max, 31));
 
-    uint32_t hsp_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 16, hq[hnq] / 128));
+    // The scan route sizes its lists from the hits that the list lengths' mean promises (repeats
+    // and skewed bases bring more): lists that turn out short are enlarged and their kernel rerun.
+    const uint64_t hits_guess = scan ? (uint64_t)((double)HM * (double)ix->n_postings / std::pow(4.0, ix->k)) : hq[hnq];
+    uint32_t hsp_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 14, hits_guess / 64));
     DevHsp *hsp = arena.alloc_n<DevHsp>(hsp_cap);
     uint32_t n_hsp = 0;
-    uint32_t *counter = arena.alloc_n<uint32_t>(4);
-    uint32_t *status = arena.alloc_n<uint32_t>(1);
-    GN_CUDA(cudaMemsetAsync(status, 0, 4, s));
+    uint32_t *counter = &words->n_hsp;
     std::vector<uint32_t> hits_q;
 
     // appends HSPs through `launch(out, room)`, growing the HSP buffer and relaunching on overflow
@@ -2361,50 +2606,65 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         }
         throw Error{GN_EINTERNAL, "HSP buffer growth did not converge"};
     };
-    if (scan && hq[hnq]) {
+    if (scan && HM) {
         auto kernel = kind == SIG_FLANK ? k_seed_scan<SIG_FLANK> : k_seed_scan<SIG_AHEAD>;
         auto chain = kind == SIG_FLANK ? k_chain<SIG_FLANK> : k_chain<SIG_AHEAD>;
-        int occ = 0, cocc = 0;
-        GN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, SCAN_THREADS, 0));
-        GN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cocc, chain, SCAN_THREADS, 0));
-        // resident blocks; fewer when the hits (at most 4 a unit, plus an offset's own unit) do not fill them
-        const uint64_t tiles = (hq[hnq] / 4 + 2 * HM) / 64 + 1;
+        const int occ = blocks_per_sm(reinterpret_cast<const void *>(kernel), SCAN_THREADS);
+        const int cocc = blocks_per_sm(reinterpret_cast<const void *>(chain), SCAN_THREADS);
+        // resident blocks; fewer when the units (four hits each, at least one an offset) do not fill them
+        const uint64_t tiles = (hits_guess / 4 + 2 * HM) / 64 + 1;
         const unsigned grid = (unsigned)std::max<uint64_t>(
-            1, std::min<uint64_t>((tiles + SCAN_THREADS / 32 - 1) / (SCAN_THREADS / 32), (uint64_t)num_sms() * std::max(occ, 1)));
+            1, std::min<uint64_t>((tiles + SCAN_THREADS / 32 - 1) / (SCAN_THREADS / 32), (uint64_t)num_sms() * occ));
         // room for candidates: about 1 % of the hits at stride 11
-        uint64_t cand_cap = std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 16, hq[hnq] / 32));
+        uint64_t cand_cap = std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 14, hits_guess / 24));
         uint2 *cand = arena.alloc_n<uint2>(cand_cap);
-        uint32_t *sctr = arena.alloc_n<uint32_t>(4);  // candidates, tile counter, candidate counter
+        const uint64_t units = g_ktimer ? hq[hnq] : 0;
         bool scanned = false;
         for (int attempt = 0;; ++attempt) {
-            uint32_t n_cand = 0;
-            emit([&](DevHsp *o, uint32_t room) {
-                if (!scanned) {
-                    GN_CUDA(cudaMemsetAsync(sctr, 0, 16, s));
-                    GN_LAUNCH("k_seed_scan", hq[hnq], s,
-                              kernel<<<grid, SCAN_THREADS, 0, s>>>(qrec, hoff, HM, reinterpret_cast<const uint4 *>(ix->sig_d),
-                                                                   post_alloc_entries(ix->n_postings) / 4, flank, cand,
-                                                                   sctr, (uint32_t)cand_cap, sctr + 1));
-                    scanned = true;
-                }
-                GN_CUDA(cudaMemsetAsync(sctr + 2, 0, 4, s));
-                const ScanCtx c{qinfo, hstart_d, ix->post_d, ix->bank.pk, ix->bank.nb, hqp.pk, hqp.nb, seed_shape(ix),
-                                ix->t, (int)links, flank, hit_min_len, seq_map(ix), o, counter, room, status,
-                                ix->n_postings, ix->n_bases, HM};
-                GN_LAUNCH("k_chain", hq[hnq], s,
-                          chain<<<(unsigned)std::min<uint64_t>((cand_cap + SCAN_THREADS - 1) / SCAN_THREADS,
-                                                               (uint64_t)num_sms() * std::max(cocc, 1)),
-                                  SCAN_THREADS, 0, s>>>(c, cand, sctr, (uint32_t)cand_cap, sctr + 2));
-                GN_CUDA(cudaMemcpyAsync(&n_cand, sctr, 4, cudaMemcpyDeviceToHost, s));
-            });
-            if (n_cand <= cand_cap) break;
-            GN_REQUIRE(attempt < 1, GN_EINTERNAL, "candidate list sizing did not converge");
-            n_hsp = 0;  // the rerun emits everything again
-            cand_cap = n_cand;
-            cand = arena.alloc_n<uint2>(cand_cap);
-            scanned = false;
+            if (attempt) {  // n_hsp and next_cand, and the scan's own counters if it runs again
+                GN_CUDA(cudaMemsetAsync(&words->n_hsp, 0, 4, s));
+                GN_CUDA(cudaMemsetAsync(&words->next_cand, 0, 4, s));
+                if (!scanned) GN_CUDA(cudaMemsetAsync(&words->n_cand, 0, 8, s));
+            }
+            if (!scanned)
+                GN_LAUNCH("k_seed_scan", units, s,
+                          kernel<<<grid, SCAN_THREADS, 0, s>>>(qrec, hoff, HM, reinterpret_cast<const uint4 *>(ix->sig_d),
+                                                               post_alloc_entries(ix->n_postings) / 4, flank, cand,
+                                                               &words->n_cand, (uint32_t)cand_cap, &words->next_tile));
+            const ScanCtx c{qinfo, hstart_d, ix->post_d, ix->bank.pk, ix->bank.nb, hqp.pk, hqp.nb, seed_shape(ix),
+                            ix->t, (int)links, flank, hit_min_len, seq_map(ix), hsp, counter, hsp_cap, status,
+                            ix->n_postings, ix->n_bases, HM};
+            GN_LAUNCH("k_chain", units, s,
+                      chain<<<(unsigned)std::min<uint64_t>((cand_cap + SCAN_THREADS - 1) / SCAN_THREADS, (uint64_t)num_sms() * cocc),
+                              SCAN_THREADS, 0, s>>>(c, cand, &words->n_cand, (uint32_t)cand_cap, &words->next_cand));
+            pin.fetch(0, words, words_bytes);
+            pin.wait();
+            const SearchWords *got = reinterpret_cast<const SearchWords *>(pin.p);
+            if (hq.empty()) read_hits(reinterpret_cast<const uint64_t *>(pin.p + sizeof(SearchWords)));
+            const uint32_t n_cand = got->n_cand, n_new = got->n_hsp;
+            if (n_cand <= cand_cap && n_new <= hsp_cap) {
+                n_hsp = n_new;
+                break;
+            }
+            GN_REQUIRE(attempt < 3, GN_EINTERNAL, "candidate and HSP list sizing did not converge");
+            GN_REQUIRE(n_new < 0xFFFFFFFFu, GN_ETOOBIG, "more than 2^32 HSPs in one call");
+            scanned = n_cand <= cand_cap;
+            if (!scanned) {
+                cand_cap = n_cand;
+                cand = arena.alloc_n<uint2>(cand_cap);
+            }
+            if (n_new > hsp_cap) {
+                hsp_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull, (uint64_t)n_new + n_new / 4);
+                hsp = arena.alloc_n<DevHsp>(hsp_cap);
+            }
+            GN_CUDA(cudaMemsetAsync(status, 0, 4, s));
         }
         timer.mark("seed_scan");
+    }
+    if (hq.empty()) hq.assign(hnq + 1, 0);  // no offsets at all
+    if (keep) {
+        res->st_hit_counts.resize(hnq);
+        for (uint32_t i = 0; i < hnq; ++i) res->st_hit_counts[i] = hq[i + 1] - hq[i];
     }
 
     uint32_t qa = scan ? hnq : 0;
@@ -2643,19 +2903,19 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
                 unsigned long long n_ovf = 0;
                 unsigned long long *ovf_count = spill_count;
                 uint32_t *big = carena.alloc_n<uint32_t>(NB);  // buckets for the block-level grouping
-                uint32_t *big_count = carena.alloc_n<uint32_t>(1);
+                uint32_t *big_count = carena.alloc_n<uint32_t>(1), *next_bucket = carena.alloc_n<uint32_t>(1);
                 uint32_t n_big = 0;
                 for (int attempt = 0;; ++attempt) {
                     const uint32_t hsp_before = n_hsp;
                     emit([&](DevHsp *o, uint32_t room) {
                         GN_CUDA(cudaMemsetAsync(ovf_count, 0, 8, s));
-                        GN_CUDA(cudaMemsetAsync(counter + 1, 0, 4, s));
+                        GN_CUDA(cudaMemsetAsync(next_bucket, 0, 4, s));
                         GN_CUDA(cudaMemsetAsync(big_count, 0, 4, s));
                         GN_LAUNCH("k_bucket_group", n_kept, s,
                                   k_bucket_group_warp<<<ggrid, BGW_WARPS * 32, smem, s>>>(
                                       bkeys, bcount, bcap, NB, bq, qa, qbits, k, p.max_hit_distance, hit_min_len,
                                       singles, seq_map(ix), o, counter, room, gsp + spilled_fill,
-                                      (unsigned long long)group_room, ovf_count, status, counter + 1, big,
+                                      (unsigned long long)group_room, ovf_count, status, next_bucket, big,
                                       big_count));
                         // read back with the HSP count, in emit's one synchronisation
                         GN_CUDA(cudaMemcpyAsync(&n_ovf, ovf_count, 8, cudaMemcpyDeviceToHost, s));
@@ -2730,15 +2990,12 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     // a9: extension
     if (n_hsp) {
         // resident warps only, taking HSP ends from a counter
-        unsigned long long *next_end = reinterpret_cast<unsigned long long *>(arena.alloc_n<uint64_t>(1));
-        GN_CUDA(cudaMemsetAsync(next_end, 0, 8, s));
-        int xocc = 0;
-        GN_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&xocc, k_xdrop, 256, 0));
         const uint64_t xwarps =
-            std::min<uint64_t>((2ull * n_hsp + 31) / 32, (uint64_t)num_sms() * std::max(xocc, 1) * 8);
+            std::min<uint64_t>((2ull * n_hsp + 31) / 32,
+                               (uint64_t)num_sms() * blocks_per_sm(reinterpret_cast<const void *>(k_xdrop), 256) * 8);
         GN_LAUNCH("k_xdrop", n_hsp, s,
                   k_xdrop<<<blocks_for(xwarps * 32, 256), 256, 0, s>>>(hsp, n_hsp, seqs, qstart_d, ix->seq_start_d, sc.match,
-                                                                      sc.mismatch, p.xdrop, nq, ix->n_seqs, next_end));
+                                                                      sc.mismatch, p.xdrop, nq, ix->n_seqs, &words->next_end));
     }
     timer.mark("xdrop_extend");
     if (keep) {
@@ -2748,53 +3005,75 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         if (n_hsp) memcpy(res->st_ext.data(), v.data(), sizeof(DevHsp) * n_hsp);
     }
 
-    // a10: merge overlapped HSPs
-    uint32_t n_mg = 0;
+    // From here on counts stay on the device (merged HSPs, selected ones, alignments kept): the
+    // buffers are sized by what they can be at most, and the kernels read them there, so that the
+    // phases follow each other without the host.  Only stage outputs and the paths that sort
+    // records over the whole call read them in between.
+    const uint32_t N = p.max_alignments;
+    const char *senv = getenv("GN_SELECT_PATH"), *renv = getenv("GN_RANK_PATH");
+    const bool sort_select = (N > (uint32_t)SQ_CAP) || (N == 0 && keep) || (senv && strcmp(senv, "sort") == 0);
+    bool sort_rank = N > (uint32_t)RQ_CAP || sort_select || (renv && strcmp(renv, "sort") == 0);
+    auto read_count = [&](const uint64_t *dev) {
+        pin.fetch(0, dev, 8);
+        pin.wait();
+        return (uint32_t)*reinterpret_cast<const uint64_t *>(pin.p);
+    };
+
+    // a10: merge overlapped HSPs; per query, its first box and the prefix sums of what is selected
+    uint64_t *n_mg_d = arena.alloc_n<uint64_t>(2), *n_sel_own = n_mg_d + 1;
     DevHsp *merged = arena.alloc_n<DevHsp>(n_hsp);
+    uint32_t *qfirst = arena.alloc_n<uint32_t>(nq + 1);
+    uint64_t *qo = arena.alloc_n<uint64_t>(nq + 1);  // selected HSPs of the queries before each
+    uint32_t n_mg = 0;                               // read only where it is needed
     if (n_hsp) {
-        uint32_t *perm = arena.alloc_n<uint32_t>(n_hsp);
-        // (qi, seq, qs) order; the sweep takes the records of one qs by (ds, qe)
-        sort_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, n_hsp,
-                     {{W_QI, qib, false}, {W_SEQ, seqb, false}, {W_QS, qposb, false}}, perm, arena, s);
-        DevHsp *srt = arena.alloc_n<DevHsp>(n_hsp);
-        gather_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, perm, n_hsp,
-                       reinterpret_cast<uint32_t *>(srt), s);
         DevHsp *boxes = arena.alloc_n<DevHsp>(n_hsp);
-        uint32_t *flag = arena.alloc_n<uint32_t>(n_hsp);
-        GN_LAUNCH("k_overlap_sweep", n_hsp, s,
-                  k_overlap_sweep<<<blocks_for(n_hsp), 256, 0, s>>>(srt, n_hsp, boxes, flag));
-        n_mg = compact_records(reinterpret_cast<const uint32_t *>(boxes), HSP_WORDS, flag, n_hsp,
-                               reinterpret_cast<uint32_t *>(merged), arena, s);
+        if (n_hsp <= MB_CAP && nq <= MB_QUERIES && qib + seqb + qposb <= 64) {
+            GN_LAUNCH("k_merge_block", n_hsp, s,
+                      k_merge_block<<<1, MB_THREADS, 0, s>>>(hsp, n_hsp, (uint32_t)seqb, (uint32_t)qposb, nq, N, keep ? 0 : 1,
+                                                             boxes, merged, qfirst, qo, n_mg_d));
+        } else {
+            uint32_t *perm = arena.alloc_n<uint32_t>(n_hsp);
+            // (qi, seq, qs) order; the sweep takes the records of one qs by (ds, qe)
+            sort_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, n_hsp,
+                         {{W_QI, qib, false}, {W_SEQ, seqb, false}, {W_QS, qposb, false}}, perm, arena, s);
+            DevHsp *srt = arena.alloc_n<DevHsp>(n_hsp);
+            gather_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, perm, n_hsp,
+                           reinterpret_cast<uint32_t *>(srt), s);
+            uint32_t *flag = arena.alloc_n<uint32_t>(n_hsp);
+            GN_LAUNCH("k_overlap_sweep", n_hsp, s,
+                      k_overlap_sweep<<<blocks_for(n_hsp), 256, 0, s>>>(srt, n_hsp, boxes, flag, keep ? 0 : 1));
+            const uint64_t *count = compact_records_async(reinterpret_cast<const uint32_t *>(boxes), HSP_WORDS, flag, n_hsp,
+                                                          reinterpret_cast<uint32_t *>(merged), arena, s);
+            GN_CUDA(cudaMemcpyAsync(n_mg_d, count, 8, cudaMemcpyDeviceToDevice, s));
+            uint32_t *cnt_sel = N && !sort_select ? arena.alloc_n<uint32_t>(nq) : nullptr;
+            GN_LAUNCH("k_query_bounds", nq + 1, s,
+                      k_query_bounds<<<blocks_for(nq + 1), 256, 0, s>>>(merged, n_mg_d, nq, qfirst, cnt_sel ? nullptr : qo, N, cnt_sel));
+            if (cnt_sel) {
+                void *scr = arena.alloc(scan_scratch_bytes(nq));
+                exclusive_scan_u32(cnt_sel, qo, nq, scr, s);
+            }
+        }
     }
     timer.mark("overlap_merge");
+    if (n_hsp && (keep || sort_select)) n_mg = read_count(n_mg_d);
     if (keep) {
         std::vector<DevHsp> v = to_host(merged, n_mg, s);
         res->st_merged.resize(n_mg);
         if (n_mg) memcpy(res->st_merged.data(), v.data(), sizeof(DevHsp) * n_mg);
     }
 
-    // a11: longest first, at most max_alignments per query
-    uint32_t n_sel = 0;
-    DevHsp *sel = arena.alloc_n<DevHsp>(n_mg);
-    uint32_t *first = arena.alloc_n<uint32_t>(nq);
-    const char *senv = getenv("GN_SELECT_PATH");
-    const bool per_query_select = p.max_alignments > 0 && p.max_alignments <= (uint32_t)SQ_CAP &&
-                                  max_qlen <= 65535 && !(senv && strcmp(senv, "sort") == 0);
-    if (n_mg && per_query_select) {
-        uint32_t *qb = arena.alloc_n<uint32_t>(nq + 1);
-        uint32_t *cnt = arena.alloc_n<uint32_t>(nq);
-        GN_LAUNCH("k_query_bounds", nq + 1, s,
-                  k_query_bounds<<<blocks_for(nq + 1), 256, 0, s>>>(merged, n_mg, nq, qb, p.max_alignments, cnt));
-        uint64_t *qo = arena.alloc_n<uint64_t>(nq + 1);
-        void *scr = arena.alloc(scan_scratch_bytes(nq));
-        exclusive_scan_u32(cnt, qo, nq, scr, s);
-        uint64_t tot = 0;
-        GN_CUDA(cudaMemcpyAsync(&tot, qo + nq, 8, cudaMemcpyDeviceToHost, s));
-        GN_LAUNCH("k_select_query", n_mg, s,
-                  k_select_query<<<nq, SQ_THREADS, 0, s>>>(merged, qb, qo, p.max_alignments, sel));
-        GN_CUDA(cudaStreamSynchronize(s));
-        n_sel = (uint32_t)tot;
-    } else if (n_mg) {
+    // a11: longest first, at most max_alignments per query (all of them: the boxes as they are)
+    const uint32_t sel_cap = (uint32_t)std::min<uint64_t>(n_hsp, N ? (uint64_t)nq * N : ~0ull);
+    uint32_t n_sel = 0;                      // read only where it is needed
+    const uint64_t *n_sel_d = qo + nq;       // the same on the device
+    DevHsp *sel = merged;
+    if (n_hsp && !sort_select && N) {
+        sel = arena.alloc_n<DevHsp>(sel_cap);
+        GN_LAUNCH("k_select_query", n_hsp, s,
+                  k_select_query<<<nq, SQ_THREADS, 0, s>>>(merged, qfirst, qo, N, max_qlen > 65535 ? 3 : 2, sel));
+    } else if (n_mg && sort_select) {
+        sel = arena.alloc_n<DevHsp>(n_mg);
+        uint32_t *first = arena.alloc_n<uint32_t>(nq);
         uint32_t *perm = arena.alloc_n<uint32_t>(n_mg);
         sort_records(reinterpret_cast<const uint32_t *>(merged), HSP_WORDS, n_mg,
                      {{W_QI, qib, false}, {W_LEN, qposb, true}, {W_SEQ, seqb, false}, {W_QS, qposb, false},
@@ -2807,11 +3086,14 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
                   k_first_of_query<<<blocks_for(n_mg), 256, 0, s>>>(reinterpret_cast<const uint32_t *>(srt), HSP_WORDS, n_mg, first));
         uint32_t *flag = arena.alloc_n<uint32_t>(n_mg);
         GN_LAUNCH("k_select_flags", n_mg, s,
-                  k_select_flags<<<blocks_for(n_mg), 256, 0, s>>>(srt, n_mg, first, p.max_alignments, flag));
-        n_sel = compact_records(reinterpret_cast<const uint32_t *>(srt), HSP_WORDS, flag, n_mg,
-                                reinterpret_cast<uint32_t *>(sel), arena, s);
+                  k_select_flags<<<blocks_for(n_mg), 256, 0, s>>>(srt, n_mg, first, N, flag));
+        const uint64_t *count = compact_records_async(reinterpret_cast<const uint32_t *>(srt), HSP_WORDS, flag, n_mg,
+                                                      reinterpret_cast<uint32_t *>(sel), arena, s);
+        GN_CUDA(cudaMemcpyAsync(n_sel_own, count, 8, cudaMemcpyDeviceToDevice, s));
+        n_sel_d = n_sel_own;
     }
     timer.mark("select");
+    if (n_hsp && (keep || sort_rank)) n_sel = (n_mg || !sort_select) ? read_count(n_sel_d) : 0;
     if (keep) {
         std::vector<DevHsp> v = to_host(sel, n_sel, s);
         res->st_sel.resize(n_sel);
@@ -2819,13 +3101,13 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     }
 
     // a12: banded Smith-Waterman
-    DevAln *aln = arena.alloc_n<DevAln>(n_sel);
-    if (n_sel) {
-        uint32_t *B = arena.alloc_n<uint32_t>(n_sel);
-        uint64_t *soff = arena.alloc_n<uint64_t>(n_sel + 1);
-        unsigned long long *dp_cells = reinterpret_cast<unsigned long long *>(arena.alloc_n<uint64_t>(2));
-        GN_CUDA(cudaMemsetAsync(dp_cells, 0, 16, s));
-        uint64_t *okeys = arena.alloc_n<uint64_t>(n_sel), *okeys_alt = arena.alloc_n<uint64_t>(n_sel);
+    const bool any_sel = n_hsp && (!sort_select || n_mg);
+    DevAln *aln = arena.alloc_n<DevAln>(any_sel ? sel_cap : 0);
+    const SwScore score{sc.match, sc.mismatch, sc.gap_open + sc.gap_extend, sc.gap_extend, 1};
+    const bool cut = sc.mismatch < 2 * sc.gap_extend;
+    uint32_t *strip = nullptr;
+    if (any_sel) {
+        const uint32_t sms = (uint32_t)num_sms();
         // lanes per HSP of the grouped path (the index's tuning; GN_SW_LANES overrides)
         uint32_t sw_lanes = ix->tuning.sw_lanes ? ix->tuning.sw_lanes : 8;
         if (const char *e = getenv("GN_SW_LANES")) sw_lanes = (uint32_t)atoi(e);
@@ -2835,42 +3117,64 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         // which bound the phase, slow down with every warp that shares theirs.  us at 4 | 8 | 16
         // warps an SM, rows from 512 | 1,024 (default band): 4,900 alignments 165 165 | 182 212 |
         // 223 257; 30,000 alignments 534 375 | 374 307 | 436 449; 50,000 1036 768 | 716 567 | 672
-        // 613.  With no more alignments than warps each gets its own (sw_lanes = 32 asks for that).
-        const bool many = n_sel > (uint32_t)num_sms() * 64;
-        uint32_t sw_long = ix->tuning.sw_wave_rows ? ix->tuning.sw_wave_rows : many ? 1024 : 512;
-        if (n_sel <= (uint32_t)num_sms() * 4 || sw_lanes == 32) sw_long = 1;
+        // 613.  So rows from 512 at 4 warps an SM, from 1,024 at 8 with more than 64 alignments an
+        // SM (sw_long_rows, sw_many: the device knows the number), and with no more alignments
+        // than warps each gets its own, in any order (sw_lanes = 32 asks for that).
+        uint32_t sw_long = ix->tuning.sw_wave_rows;
         if (const char *e = getenv("GN_SW_LONG_ROWS")) sw_long = (uint32_t)std::max(1l, strtol(e, nullptr, 10));
-        uint32_t *n_long = arena.alloc_n<uint32_t>(2);
-        GN_CUDA(cudaMemsetAsync(n_long, 0, 8, s));
-        GN_LAUNCH("k_sw_prepare", n_sel, s,
-                  k_sw_prepare<<<blocks_for(n_sel), 256, 0, s>>>(sel, n_sel, (int32_t)p.band_w,
-                                                                  sw_lanes == 16 ? 48 : 40, qstart_d, B, dp_cells,
-                                                                  sw_long, okeys, n_long));
-        void *scr = arena.alloc(scan_scratch_bytes(n_sel));
-        exclusive_scan_u32(B, soff, n_sel, scr, s);
-        uint64_t cells = 0, area[2] = {0, 0};
-        GN_CUDA(cudaMemcpyAsync(&cells, soff + n_sel, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-        GN_CUDA(cudaMemcpyAsync(area, dp_cells, 2 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-        GN_CUDA(cudaStreamSynchronize(s));
-        SwCell *strips = arena.alloc_n<SwCell>(cells);
-        void *rs = arena.alloc(radix_scratch_bytes(n_sel));
-        const uint64_t *order = radix_sort(okeys, okeys_alt, nullptr, nullptr, n_sel, 32, 48, rs, s, TAG_RECORD_SORT)
-                                    ? okeys_alt : okeys;
-        GN_CUDA(cudaMemsetAsync(counter, 0, 12, s));
-        uint32_t *wide = arena.alloc_n<uint32_t>(n_sel);
-        const bool cut = sc.mismatch < 2 * sc.gap_extend;
+        if (sw_lanes == 32) sw_long = 1;
+        const bool ordered = sel_cap > sms * 4 || getenv("GN_SW_LONG_ROWS");
+        uint32_t *order = ordered ? arena.alloc_n<uint32_t>(sel_cap) : nullptr;
+        const int cap = sw_lanes == 16 ? 48 : 40;
+        if (ordered || g_ktimer)
+            GN_LAUNCH("k_sw_prepare", sel_cap, s,
+                      k_sw_prepare<<<blocks_for(sel_cap), 256, 0, s>>>(sel, n_sel_d, (int32_t)p.band_w, cap, qstart_d, sw_long, sms,
+                                                                       words->bins, g_ktimer ? words->cells : nullptr));
+        if (ordered)
+            GN_LAUNCH("k_sw_order", sel_cap, s,
+                      k_sw_order<<<blocks_for(sel_cap), 256, 0, s>>>(sel, n_sel_d, (int32_t)p.band_w, cap, qstart_d, sw_long, sms,
+                                                                     words->bins, words->placed, order, &words->n_long));
+        uint64_t area[2] = {0, 0};
+        if (g_ktimer) {
+            pin.fetch(0, words->cells, 16);
+            pin.wait();
+            memcpy(area, pin.p, 16);
+        }
+        uint32_t *wide = arena.alloc_n<uint32_t>(sel_cap);
+        strip = arena.alloc_n<uint32_t>(sel_cap);
         auto sw_kernel = sw_lanes == 16 ? (cut ? k_banded_sw<16, 2, 1, true> : k_banded_sw<16, 2, 1, false>)
                                         : (cut ? k_banded_sw<8, 3, 2, true> : k_banded_sw<8, 3, 2, false>);
         auto wide_kernel = cut ? k_banded_sw_wide<true> : k_banded_sw_wide<false>;
-        const SwScore score{sc.match, sc.mismatch, sc.gap_open + sc.gap_extend, sc.gap_extend, 1};
-        const unsigned warps = (unsigned)std::min<uint64_t>(n_sel, (uint64_t)num_sms() * (many ? 8 : 4));
         GN_LAUNCH("k_banded_sw", area[0], s,
-                  sw_kernel<<<(warps * 32 + 127) / 128, 128, 0, s>>>(sel, n_sel, seqs, qstart_d, ix->seq_start_d, score,
-                                                          (int32_t)p.band_w, counter, order, wide, counter + 1,
-                                                          n_long, n_long + 1, aln));
+                  sw_kernel<<<std::min<uint32_t>((sel_cap + 3) / 4, sms * 2), 128, 0, s>>>(
+                      sel, n_sel_d, sms, seqs, qstart_d, ix->seq_start_d, score, (int32_t)p.band_w, &words->next_task, order, wide,
+                      &words->n_wide, &words->n_long, &words->next_long, aln));
         GN_LAUNCH("k_banded_sw_wide", area[1], s,
-                  wide_kernel<<<num_sms() * 4, 128, 0, s>>>(sel, wide, counter + 1, counter + 2, soff, strips, seqs, qstart_d,
-                                                            ix->seq_start_d, score, (int32_t)p.band_w, aln, status));
+                  wide_kernel<<<std::min<uint32_t>((sel_cap + 3) / 4, sms * 4), 128, 0, s>>>(
+                      sel, wide, &words->n_wide, &words->next_wide, seqs, qstart_d, ix->seq_start_d, score, (int32_t)p.band_w, strip,
+                      &words->n_strip, &words->strip_band, aln));
+    }
+    // bands that no register path holds, once the host knows of them: they are rare, and the rest of
+    // the search does not wait for the question
+    auto align_strips = [&](const SearchWords &got) {
+        const uint64_t cells = (uint64_t)got.strip_band + 2;
+        const uint64_t warps = std::min<uint64_t>({(uint64_t)got.n_strip, (uint64_t)num_sms() * 16,
+                                                   std::max<uint64_t>(1, (1ull << 30) / (cells * sizeof(SwCell)))});
+        const uint64_t blocks = (warps + 3) / 4;
+        SwCell *strips = arena.alloc_n<SwCell>(blocks * 4 * cells);
+        GN_LAUNCH("k_banded_sw_strip", got.n_strip, s,
+                  k_banded_sw_strip<<<(unsigned)blocks, 128, 0, s>>>(sel, strip, got.n_strip, &words->next_strip, strips, cells, seqs,
+                                                                     qstart_d, ix->seq_start_d, score, (int32_t)p.band_w, aln,
+                                                                     status));
+    };
+    SearchWords got{};
+    bool strips_done = false;
+    if (any_sel && (keep || sort_rank)) {
+        pin.fetch(0, words, sizeof(SearchWords));
+        pin.wait();
+        memcpy(&got, pin.p, sizeof(SearchWords));
+        if (got.n_strip) align_strips(got);
+        strips_done = true;
     }
     timer.mark("banded_sw");
     if (keep) {
@@ -2885,32 +3189,65 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
 
     // a13: duplicates (same query, sequence and ranges: keep the best score), rank by score, statistics
     uint32_t n_out = 0;
-    gn_hit *fin = arena.alloc_n<gn_hit>(n_sel);
-    const uint64_t *qoff_dev = nullptr;  // per-query offsets of fin, when a phase computed them
-    const char *renv = getenv("GN_RANK_PATH");
-    const bool per_query_rank = p.max_alignments != 0 && p.max_alignments <= (uint32_t)RQ_CAP &&
-                                !(renv && strcmp(renv, "sort") == 0);
-    if (n_sel && per_query_rank) {
-        uint32_t *qrange = arena.alloc_n<uint32_t>(2ull * nq);
-        GN_CUDA(cudaMemsetAsync(qrange, 0, 8ull * nq, s));
-        GN_LAUNCH("k_query_ranges", n_sel, s, k_query_ranges<<<blocks_for(n_sel), 256, 0, s>>>(aln, n_sel, qrange));
-        gn_hit *hits = arena.alloc_n<gn_hit>(n_sel);
+    gn_hit *fin = arena.alloc_n<gn_hit>(any_sel ? sel_cap : 0);
+    bool hits_read = false;  // res->hits and res->qoff are filled
+    if (any_sel && !sort_rank) {
+        // a small call's hits come back as they lie (each query's at its selected HSPs' place)
+        // with the counts, in one read; a larger one's are put together first
+        const size_t hits_bytes = sizeof(gn_hit) * (size_t)sel_cap, qo_bytes = 8 * (nq + 1ull);
+        const bool small = hits_bytes + qo_bytes + 4ull * nq <= (1u << 17);
+        gn_hit *hits = arena.alloc_n<gn_hit>(sel_cap);
         uint32_t *qcount = arena.alloc_n<uint32_t>(nq);
         const unsigned rgrid = (unsigned)std::min<uint64_t>(nq, (uint64_t)num_sms() * 8);
-        GN_LAUNCH("k_rank_query", n_sel, s,
-                  k_rank_query<<<rgrid, 256, 0, s>>>(aln, qrange, nq, qstart_d, (double)ix->n_bases, sc.lambda, sc.K,
-                                                     p.max_evalue, hits, qcount));
         uint64_t *qoff = arena.alloc_n<uint64_t>(nq + 1);
         void *scr = arena.alloc(scan_scratch_bytes(nq));
-        exclusive_scan_u32(qcount, qoff, nq, scr, s);
-        qoff_dev = qoff;  // the results' per-query offsets
-        uint64_t tot = 0;
-        GN_CUDA(cudaMemcpyAsync(&tot, qoff + nq, 8, cudaMemcpyDeviceToHost, s));
-        GN_CUDA(cudaStreamSynchronize(s));
-        n_out = (uint32_t)tot;
-        GN_LAUNCH("k_gather_ranked", n_out, s,
-                  k_gather_ranked<<<rgrid, 256, 0, s>>>(hits, qrange, qoff, nq, fin));
-    } else if (n_sel) {
+        PinnedBlock back(ix->host_pool, sizeof(SearchWords) + qo_bytes + (small ? hits_bytes + 4ull * nq : 0), s);
+        for (;;) {
+            GN_LAUNCH("k_rank_query", sel_cap, s,
+                      k_rank_query<<<rgrid, 256, 0, s>>>(aln, qo, nq, qstart_d, (double)ix->n_bases, sc.lambda, sc.K,
+                                                         p.max_evalue, hits, qcount, &words->too_many));
+            size_t at = sizeof(SearchWords);
+            if (small) {
+                back.fetch(at, qo, qo_bytes);
+                at += qo_bytes;
+                back.fetch(at, hits, hits_bytes);
+                at += hits_bytes;
+                back.fetch(at, qcount, 4ull * nq);
+            } else {
+                exclusive_scan_u32(qcount, qoff, nq, scr, s);
+                GN_LAUNCH("k_gather_ranked", sel_cap, s,
+                          k_gather_ranked<<<rgrid, 256, 0, s>>>(hits, qo, qoff, nq, fin));
+                back.fetch(at, qoff, qo_bytes);
+            }
+            back.fetch(0, words, sizeof(SearchWords));
+            back.wait();
+            memcpy(&got, back.p, sizeof(SearchWords));
+            if (strips_done || !got.n_strip) break;
+            align_strips(got);
+            strips_done = true;
+        }
+        if (got.too_many) {
+            sort_rank = true;
+            n_sel = read_count(n_sel_d);
+        } else {
+            res->qoff.resize(nq + 1);
+            const uint64_t *q_at = reinterpret_cast<const uint64_t *>(back.p + sizeof(SearchWords));
+            if (small) {
+                const gn_hit *h = reinterpret_cast<const gn_hit *>(back.p + sizeof(SearchWords) + qo_bytes);
+                const uint32_t *c = reinterpret_cast<const uint32_t *>(back.p + sizeof(SearchWords) + qo_bytes + hits_bytes);
+                res->qoff[0] = 0;
+                for (uint32_t q = 0; q < nq; ++q) {
+                    res->hits.insert(res->hits.end(), h + q_at[q], h + q_at[q] + c[q]);
+                    res->qoff[q + 1] = res->hits.size();
+                }
+            } else {
+                memcpy(res->qoff.data(), q_at, qo_bytes);
+                res->hits = to_host(fin, (size_t)res->qoff[nq], s);
+            }
+            hits_read = true;
+        }
+    }
+    if (n_sel && sort_rank) {
         const int scb = std::min(31, bits_for(std::max<uint64_t>(65535, max_qlen) * (uint64_t)std::max(1, sc.match)));
         uint32_t *perm = arena.alloc_n<uint32_t>(n_sel);
         sort_records(reinterpret_cast<const uint32_t *>(aln), ALN_WORDS, n_sel,
@@ -2934,6 +3271,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
             DevAln *ranked = arena.alloc_n<DevAln>(nu);
             gather_records(reinterpret_cast<const uint32_t *>(uniq), ALN_WORDS, perm2, nu,
                            reinterpret_cast<uint32_t *>(ranked), s);
+            uint32_t *first = arena.alloc_n<uint32_t>(nq);
             GN_LAUNCH("k_first_of_query", 0, s,
                       k_first_of_query<<<blocks_for(nu), 256, 0, s>>>(reinterpret_cast<const uint32_t *>(ranked), ALN_WORDS, nu, first));
             gn_hit *hits = arena.alloc_n<gn_hit>(nu);
@@ -2947,27 +3285,25 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         }
     }
     timer.mark("rank");
-    uint32_t st = 0, wst = 0;
-    GN_CUDA(cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s));
-    GN_CUDA(cudaMemcpyAsync(&wst, wait_status, 4, cudaMemcpyDeviceToHost, s));
-    res->hits = to_host(fin, n_out, s);
-    GN_REQUIRE((wst & DEV_ERR_TIMEOUT) == 0, GN_ETIMEOUT, "a device-side wait ran out (scan look-back)");
+    if (!hits_read) {
+        res->hits = to_host(fin, n_out, s);
+        pin.fetch(0, words, sizeof(SearchWords));
+        pin.wait();
+        memcpy(&got, pin.p, sizeof(SearchWords));
+        res->qoff.assign(nq + 1, 0);
+        for (uint32_t i = 0; i < n_out; ++i) res->qoff[res->hits[i].query + 1]++;
+        for (uint32_t i = 0; i < nq; ++i) res->qoff[i + 1] += res->qoff[i];
+    }
+    GN_REQUIRE((got.wait_status & DEV_ERR_TIMEOUT) == 0, GN_ETIMEOUT, "a device-side wait ran out (scan look-back)");
 #ifdef GN_CHECKS
     uint32_t cbits = 0;
     GN_CUDA(cudaMemcpyAsync(&cbits, check_bits, 4, cudaMemcpyDeviceToHost, s));
     GN_CUDA(cudaStreamSynchronize(s));
     GN_REQUIRE((cbits & DEV_ERR_BOUNDS) == 0, GN_EINTERNAL, "a device-side bounds check failed (checked build)");
 #endif
-    GN_REQUIRE((st & DEV_ERR_BOUNDS) == 0, GN_EINTERNAL, "a device-side bounds check failed");
-    GN_REQUIRE((st & DEV_ERR_BAND_TOO_WIDE) == 0, GN_ETOOBIG,
+    GN_REQUIRE((got.status & DEV_ERR_BOUNDS) == 0, GN_EINTERNAL, "a device-side bounds check failed");
+    GN_REQUIRE((got.status & DEV_ERR_BAND_TOO_WIDE) == 0, GN_ETOOBIG,
                "an alignment band exceeded 65,535 diagonals or its window 2^32 cells");
-    if (qoff_dev) {
-        res->qoff = to_host(qoff_dev, nq + 1, s);
-    } else {
-        res->qoff.assign(nq + 1, 0);
-        for (uint32_t i = 0; i < n_out; ++i) res->qoff[res->hits[i].query + 1]++;
-        for (uint32_t i = 0; i < nq; ++i) res->qoff[i + 1] += res->qoff[i];
-    }
     timer.mark("output");
     GN_CUDA(cudaStreamSynchronize(s));
     {
