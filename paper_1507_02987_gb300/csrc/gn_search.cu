@@ -17,6 +17,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "gn_internal.cuh"
 
@@ -1232,6 +1233,29 @@ __global__ void k_overlap_sweep(const DevHsp *__restrict__ in, uint32_t n, DevHs
 // length T comes from a 256-bin histogram per byte of the length (two, or three where a
 // query is longer than 65,535 bases), high byte first; the selected records are those
 // longer than T and the first ones of length T.
+
+// The bin of the n-th largest entry of a histogram of 256 bins that holds at least n >= 1, and how
+// many lie above that bin (out[0], out[1]); a warp, eight bins a lane.
+__device__ __forceinline__ void bin_of_nth(const uint32_t *hist, uint32_t n, uint32_t *out) {
+    const int lane = threadIdx.x & 31;
+    uint32_t sum = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum += hist[255 - 8 * lane - i];
+    uint32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (x >= n && x - sum < n) {
+        uint32_t above = x - sum;
+        int b = 255 - 8 * lane;
+        while (above + hist[b] < n) above += hist[b--];
+        out[0] = (uint32_t)b;
+        out[1] = above;
+    }
+}
+
 constexpr int SQ_CAP = 1024;  // largest N this kernel handles
 constexpr int SQ_THREADS = 512;
 
@@ -1242,7 +1266,7 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
     __shared__ uint32_t hist[256];
     __shared__ uint32_t warp_tot[SQ_THREADS / 32];
     __shared__ uint64_t keys[SQ_CAP];
-    __shared__ uint32_t T_s, gt_s;
+    __shared__ uint32_t found[2];
     const uint32_t q = blockIdx.x;
     const uint32_t a = qfirst[q], b = qfirst[q + 1], n = b - a;
     const uint64_t out0 = qout[q];
@@ -1269,16 +1293,10 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
                     atomicAdd(&hist[bin], (uint32_t)__popc(peers));
             }
             __syncthreads();
-            if (threadIdx.x == 0) {
-                uint32_t acc = above;
-                int x = 255;
-                while (acc + hist[x] < N) acc += hist[x--];
-                T_s = (T << 8) | (uint32_t)x;
-                gt_s = acc;
-            }
+            if (threadIdx.x < 32) bin_of_nth(hist, N - above, found);
             __syncthreads();
-            T = T_s;
-            above = gt_s;
+            T = (T << 8) | found[0];
+            above += found[1];
             __syncthreads();
         }
         r_eq = N - above;  // records of length T to take, in array order
@@ -1429,6 +1447,10 @@ __global__ void __launch_bounds__(MB_THREADS) k_merge_block(const DevHsp *__rest
     }
     if (threadIdx.x == 0) *n_out = n_mg;
 }
+
+}  // namespace gn
+#include "gn_merge_groups.cuh"
+namespace gn {
 
 __global__ void k_first_of_query(const uint32_t *__restrict__ recs, int W, uint32_t n, uint32_t *__restrict__ first) {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2275,6 +2297,32 @@ std::vector<T> to_host(const T *d, size_t n, cudaStream_t s) {
     return h;
 }
 
+// A few words from the device, fetched between two kernels and read while the second one runs.
+struct GroupQuestion {
+    HostPool &pool;
+    cudaStream_t s;
+    PinnedBlock pin;
+    cudaEvent_t done = nullptr;
+    GroupQuestion(HostPool &pl, cudaStream_t st) : pool(pl), s(st), pin(pl, 64, st) {}
+    void ask(const uint32_t *dev) {
+        pin.fetch(0, dev, 16);
+        if (!done) done = pool.take_event();
+        if (done) GN_CUDA(cudaEventRecord(done, s));
+    }
+    void answer(uint32_t *out) {
+        if (done) {
+            GN_CUDA(cudaEventSynchronize(done));
+            pin.in_flight = false;
+        } else {
+            pin.wait();
+        }
+        memcpy(out, pin.p, 16);
+    }
+    ~GroupQuestion() {
+        if (done) pool.give_event(done);
+    }
+};
+
 // Resident blocks of a kernel without dynamic shared memory, asked of the driver once per kernel
 // and device (a search asks for five).
 int blocks_per_sm(const void *fn, int threads) {
@@ -2321,6 +2369,8 @@ void allow_max_smem(int device) {
     allow(reinterpret_cast<const void *>(k_bucket_fill<0, 0>));
     allow(reinterpret_cast<const void *>(k_bucket_fill<19, 17>));
     allow(reinterpret_cast<const void *>(k_bucket_group_warp));
+    allow(reinterpret_cast<const void *>(k_merge_groups<1024, MG_BIG / 1024, false>));
+    allow(reinterpret_cast<const void *>(k_merge_groups<1024, MG_BIG / 1024, true>));
     done[device] = true;
 }
 }  // namespace
@@ -2373,6 +2423,7 @@ struct SearchWords {
     uint32_t n_wide, next_wide, next_task, n_long, next_long;
     uint32_t n_strip, strip_band, next_strip;
     uint32_t too_many, pad;
+    uint32_t groups[8];                // groups of a block, of a large block, of no kernel: of the join, of the merge
     unsigned long long next_end, cells[2];
     uint32_t bins[SWO_BINS], placed[SWO_BINS];
 };
@@ -2955,25 +3006,126 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     const int seqb = bits_for(ix->n_seqs ? ix->n_seqs - 1 : 0);
     const int posb = bits_for(ix->max_seq_len);
     const int qposb = std::max(16, bits_for(max_qlen));
+    // Groups of HSPs, their members counted and placed, for the join of long queries' pieces and for
+    // the merge.
+    struct {
+        GroupMap map;
+        uint32_t G = 0;
+        uint32_t *cnt = nullptr, *list = nullptr, *perm = nullptr;
+        uint2 *where = nullptr;
+        uint64_t *off = nullptr;
+        uint32_t words[4];
+    } gr;
+    GroupQuestion asked(ix->host_pool, s);
+    auto count_groups = [&](bool by_count) {
+        const uint64_t per_base = ((uint64_t)n_hsp << 32) / (std::max<uint64_t>(M, 1) * MG_TARGET);
+        gr.map = GroupMap{qstart_d, per_base, 0xFFFFFFFFu / std::max(ix->n_seqs, 1u), nullptr};
+        gr.G = nq + (uint32_t)((M * per_base) >> 32);
+        if (by_count) {
+            gr.G = nq + n_hsp / MG_TARGET;  // the last ones may stay empty
+            uint32_t *seen = arena.alloc_n<uint32_t>(2ull * nq);
+            uint64_t *first = arena.alloc_n<uint64_t>(nq + 1);
+            GN_CUDA(cudaMemsetAsync(seen, 0, 8ull * nq, s));
+            GN_LAUNCH("k_query_parts", n_hsp, s,
+                      k_query_parts<<<blocks_for(n_hsp), 256, 0, s>>>(hsp, n_hsp, seen, seen + nq));
+            void *scr = arena.alloc(scan_scratch_bytes(nq));
+            exclusive_scan_u32(seen + nq, first, nq, scr, s);
+            gr.map.by_count = first;
+        }
+        gr.cnt = arena.alloc_n<uint32_t>(gr.G);
+        gr.where = arena.alloc_n<uint2>(n_hsp);
+        GN_CUDA(cudaMemsetAsync(gr.cnt, 0, 4ull * gr.G, s));
+        GN_LAUNCH("k_group_count", n_hsp, s,
+                  k_group_count<<<blocks_for(n_hsp), 256, 0, s>>>(hsp, n_hsp, gr.map, gr.cnt, gr.where));
+    };
+    auto list_groups = [&](uint32_t *words) {  // by size, which the host learns
+        gr.list = arena.alloc_n<uint32_t>(gr.G);
+        GN_LAUNCH("k_group_lists", gr.G, s, k_group_lists<<<blocks_for(gr.G), 256, 0, s>>>(gr.cnt, gr.G, gr.list, words));
+        asked.ask(words);
+    };
+    auto scan_groups = [&](const uint32_t *cnt) {
+        uint64_t *off = arena.alloc_n<uint64_t>(gr.G + 1ull);
+        void *scr = arena.alloc(scan_scratch_bytes(gr.G));
+        exclusive_scan_u32(cnt, off, gr.G, scr, s);
+        return off;
+    };
+    // The host's answer, and, where a group is too large, groups by the queries' HSPs; then the
+    // members' order.  False: a group is still too large.
+    auto place_groups = [&](uint32_t *words) {
+        asked.answer(gr.words);
+        if (gr.words[2]) {
+            GN_CUDA(cudaMemsetAsync(words, 0, sizeof(gr.words), s));
+            count_groups(true);
+            list_groups(words);
+            asked.answer(gr.words);
+            if (gr.words[2]) return false;
+        }
+        gr.off = scan_groups(gr.cnt);
+        gr.perm = arena.alloc_n<uint32_t>(n_hsp);
+        GN_LAUNCH("k_group_scatter", n_hsp, s,
+                  k_group_scatter<<<blocks_for(n_hsp), 256, 0, s>>>(gr.where, n_hsp, gr.off, gr.perm));
+        return true;
+    };
+    auto run_groups = [&](const MergeGroups &m, const uint32_t *words, auto stitch) {
+        constexpr bool ST = decltype(stitch)::value;
+        constexpr int ME = MG_MID / 256, BE = MG_BIG / 1024;
+        GN_CUDA(cudaMemsetAsync(m.n_out, 0, 4ull * gr.G, s));
+        GN_LAUNCH("k_merge_groups_warp", n_hsp, s, k_merge_groups_warp<ST><<<(gr.G + 7) / 8, 256, 0, s>>>(m, gr.G));
+        if (gr.words[0])
+            GN_LAUNCH("k_merge_groups", n_hsp, s,
+                      k_merge_groups<256, ME, ST><<<gr.words[0], 256, sizeof(MergeSmem<256, ME>), s>>>(m, gr.list, 1, words));
+        if (gr.words[1]) {
+            allow_max_smem(ix->device);
+            GN_LAUNCH("k_merge_groups", n_hsp, s,
+                      k_merge_groups<1024, BE, ST><<<gr.words[1], 1024, sizeof(MergeSmem<1024, BE>), s>>>(m, gr.list + (gr.G - 1), -1,
+                                                                                                      words + 1));
+        }
+    };
+    bool joined_groups = false;  // the HSPs lie by group
     if (segmented && n_hsp) {
         // pieces onto their queries, then one chain per run of pieces sharing seeds
         GN_LAUNCH("k_segment_map", n_hsp, s,
                   k_segment_map<<<blocks_for(n_hsp), 256, 0, s>>>(hsp, n_hsp, seg_parent_d, seg_off_d));
-        uint32_t *perm = arena.alloc_n<uint32_t>(n_hsp);
-        sort_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, n_hsp,
-                     {{W_QI, qib, false}, {W_SEQ, seqb, false}, {W_LEN, 32, false}, {W_QS, qposb, false}},
-                     perm, arena, s);
-        DevHsp *srt = arena.alloc_n<DevHsp>(n_hsp);
-        gather_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, perm, n_hsp,
-                       reinterpret_cast<uint32_t *>(srt), s);
-        DevHsp *chains = arena.alloc_n<DevHsp>(n_hsp);
-        uint32_t *flag = arena.alloc_n<uint32_t>(n_hsp);
-        GN_LAUNCH("k_stitch_sweep", n_hsp, s,
-                  k_stitch_sweep<<<blocks_for(n_hsp), 256, 0, s>>>(srt, n_hsp, (uint32_t)k, p.min_hsp_len, chains,
-                                                                  flag));
+        const int diagb = bits_for((uint64_t)ix->max_seq_len + max_qlen);
+        bool by_groups = seqb + diagb + MG_BITS <= 64;
+        if (by_groups) {
+            count_groups(false);
+            list_groups(words->groups);
+            by_groups = place_groups(words->groups);
+        }
         DevHsp *joined = arena.alloc_n<DevHsp>(n_hsp);
-        n_hsp = compact_records(reinterpret_cast<const uint32_t *>(chains), HSP_WORDS, flag, n_hsp,
-                                reinterpret_cast<uint32_t *>(joined), arena, s);
+        if (by_groups) {
+            DevHsp *chains = arena.alloc_n<DevHsp>(n_hsp);
+            uint32_t *n_chains = arena.alloc_n<uint32_t>(gr.G);
+            run_groups(MergeGroups{hsp, gr.perm, gr.off, gr.cnt, diagb, 2, 0, (uint32_t)max_qlen, (uint32_t)k, p.min_hsp_len, chains, n_chains},
+                       words->groups, std::true_type());
+            uint64_t *to = scan_groups(n_chains);
+            pin.fetch(0, to + gr.G, 8);
+            GN_LAUNCH("k_group_pack", n_hsp, s,
+                      k_group_pack<<<blocks_for(32ull * gr.G), 256, 0, s>>>(chains, gr.off, to, gr.G, gr.map, nq, 0, joined, nullptr, nullptr,
+                                                                            nullptr));
+            pin.wait();
+            n_hsp = (uint32_t)*reinterpret_cast<const uint64_t *>(pin.p);
+            gr.off = to;  // the chains lie by group
+            gr.cnt = n_chains;
+            gr.perm = nullptr;
+            joined_groups = true;
+        } else {
+            uint32_t *perm = arena.alloc_n<uint32_t>(n_hsp);
+            sort_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, n_hsp,
+                         {{W_QI, qib, false}, {W_SEQ, seqb, false}, {W_LEN, 32, false}, {W_QS, qposb, false}},
+                         perm, arena, s);
+            DevHsp *srt = arena.alloc_n<DevHsp>(n_hsp);
+            gather_records(reinterpret_cast<const uint32_t *>(hsp), HSP_WORDS, perm, n_hsp,
+                           reinterpret_cast<uint32_t *>(srt), s);
+            DevHsp *chains = arena.alloc_n<DevHsp>(n_hsp);
+            uint32_t *flag = arena.alloc_n<uint32_t>(n_hsp);
+            GN_LAUNCH("k_stitch_sweep", n_hsp, s,
+                      k_stitch_sweep<<<blocks_for(n_hsp), 256, 0, s>>>(srt, n_hsp, (uint32_t)k, p.min_hsp_len, chains,
+                                                                      flag));
+            n_hsp = compact_records(reinterpret_cast<const uint32_t *>(chains), HSP_WORDS, flag, n_hsp,
+                                    reinterpret_cast<uint32_t *>(joined), arena, s);
+        }
         hsp = joined;
         timer.mark("stitch");
     }
@@ -2987,6 +3139,28 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     const PackedPair seqs{qp.pk, qp.nb, ix->bank.pk, ix->bank.nb, (int64_t)Packed::pk_words(M) - 1,
                           (int64_t)Packed::nb_words(M) - 1, (int64_t)Packed::pk_words(ix->n_bases) - 1,
                           (int64_t)Packed::nb_words(ix->n_bases) - 1};
+    // From here on counts stay on the device (merged HSPs, selected ones, alignments kept): the
+    // buffers are sized by what they can be at most, and the kernels read them there, so that the
+    // phases follow each other without the host.  Only stage outputs and the paths that sort
+    // records over the whole call read them in between.
+    const uint32_t N = p.max_alignments;
+    const char *senv = getenv("GN_SELECT_PATH"), *renv = getenv("GN_RANK_PATH");
+    const bool sort_select = (N > (uint32_t)SQ_CAP) || (N == 0 && keep) || (senv && strcmp(senv, "sort") == 0);
+    bool sort_rank = N > (uint32_t)RQ_CAP || sort_select || (renv && strcmp(renv, "sort") == 0);
+    auto read_count = [&](const uint64_t *dev) {
+        pin.fetch(0, dev, 8);
+        pin.wait();
+        return (uint32_t)*reinterpret_cast<const uint64_t *>(pin.p);
+    };
+    // How the HSPs are merged: in one block, by groups, or in order of the whole call.  Which group
+    // an HSP is in does not change when it is extended, so the groups are counted before, and the
+    // host learns whether all of them fit while the extension runs.
+    const bool merge_block = n_hsp <= MB_CAP && nq <= MB_QUERIES && qib + seqb + qposb <= 64;
+    bool merge_groups = n_hsp && !merge_block && !keep && !sort_select && seqb + qposb + MG_BITS <= 64;
+    if (merge_groups) {
+        if (!joined_groups) count_groups(false);
+        list_groups(words->groups + 4);
+    }
     // a9: extension
     if (n_hsp) {
         // resident warps only, taking HSP ends from a counter
@@ -3005,20 +3179,6 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         if (n_hsp) memcpy(res->st_ext.data(), v.data(), sizeof(DevHsp) * n_hsp);
     }
 
-    // From here on counts stay on the device (merged HSPs, selected ones, alignments kept): the
-    // buffers are sized by what they can be at most, and the kernels read them there, so that the
-    // phases follow each other without the host.  Only stage outputs and the paths that sort
-    // records over the whole call read them in between.
-    const uint32_t N = p.max_alignments;
-    const char *senv = getenv("GN_SELECT_PATH"), *renv = getenv("GN_RANK_PATH");
-    const bool sort_select = (N > (uint32_t)SQ_CAP) || (N == 0 && keep) || (senv && strcmp(senv, "sort") == 0);
-    bool sort_rank = N > (uint32_t)RQ_CAP || sort_select || (renv && strcmp(renv, "sort") == 0);
-    auto read_count = [&](const uint64_t *dev) {
-        pin.fetch(0, dev, 8);
-        pin.wait();
-        return (uint32_t)*reinterpret_cast<const uint64_t *>(pin.p);
-    };
-
     // a10: merge overlapped HSPs; per query, its first box and the prefix sums of what is selected
     uint64_t *n_mg_d = arena.alloc_n<uint64_t>(2), *n_sel_own = n_mg_d + 1;
     DevHsp *merged = arena.alloc_n<DevHsp>(n_hsp);
@@ -3027,10 +3187,24 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     uint32_t n_mg = 0;                               // read only where it is needed
     if (n_hsp) {
         DevHsp *boxes = arena.alloc_n<DevHsp>(n_hsp);
-        if (n_hsp <= MB_CAP && nq <= MB_QUERIES && qib + seqb + qposb <= 64) {
+        if (merge_groups) {
+            if (joined_groups) asked.answer(gr.words);  // no larger than they were
+            else merge_groups = place_groups(words->groups + 4);
+        }
+        if (merge_block) {
             GN_LAUNCH("k_merge_block", n_hsp, s,
                       k_merge_block<<<1, MB_THREADS, 0, s>>>(hsp, n_hsp, (uint32_t)seqb, (uint32_t)qposb, nq, N, keep ? 0 : 1,
                                                              boxes, merged, qfirst, qo, n_mg_d));
+        } else if (merge_groups) {
+            uint32_t *n_boxes = arena.alloc_n<uint32_t>(gr.G), *cnt_sel = arena.alloc_n<uint32_t>(nq);
+            run_groups(MergeGroups{hsp, gr.perm, gr.off, gr.cnt, qposb, max_qlen > 65535 ? 3 : 2, N, 0, 0, 0, boxes, n_boxes},
+                       words->groups + 4, std::false_type());
+            uint64_t *to = scan_groups(n_boxes);
+            GN_LAUNCH("k_group_pack", n_hsp, s,
+                      k_group_pack<<<blocks_for(32ull * gr.G), 256, 0, s>>>(boxes, gr.off, to, gr.G, gr.map, nq, N, merged, qfirst, cnt_sel,
+                                                                            qo));
+            void *scr = arena.alloc(scan_scratch_bytes(nq));
+            if (N) exclusive_scan_u32(cnt_sel, qo, nq, scr, s);
         } else {
             uint32_t *perm = arena.alloc_n<uint32_t>(n_hsp);
             // (qi, seq, qs) order; the sweep takes the records of one qs by (ds, qe)
