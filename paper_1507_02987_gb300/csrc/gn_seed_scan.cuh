@@ -238,10 +238,23 @@ __device__ __forceinline__ void scan_check_ahead(const ScanCtx &c, bool valid, u
             }
         }
         open = head;
-        for (int step = 0; step < SCAN_LANE_STEPS && open; ++step) {  // d: distance of the chain's last hit
-            const int64_t l = link(x, g, d, lo, hi);
-            d += l;
-            open = l != 0;
+        // d: distance of the chain's last hit.  A window holds the next `grid` positions; the walk
+        // goes on in it while all positions in reach lie in it (a window a link: 18 instead of 12 us
+        // for a chain of 30 links, 60 instead of 47 for 1,000 diverged copies on 400 Mbp).
+        const int grid = near ? (64 - c.sh.span) / c.t + 1 : 0;
+        for (int step = 0; step < SCAN_LANE_STEPS && open; ++step) {
+            if (!near) {
+                const int64_t l = link(x, g, d, lo, hi);
+                d += l;
+                open = l != 0;
+                continue;
+            }
+            const uint64_t e = within(equal64_raw(c, x, g, d + c.t), d + c.t, lo, hi);
+            uint32_t at = 0;  // positions past the last hit, from the window's first one
+            for (int j = 0; j < grid && j < (int)at + c.ahead; ++j)
+                if (seed_at(e, j * c.t, keep)) at = j + 1;
+            d += (int64_t)at * c.t;
+            open = (int)at + c.ahead > grid;
         }
     }
     uint32_t todo = __ballot_sync(0xffffffffu, open);
