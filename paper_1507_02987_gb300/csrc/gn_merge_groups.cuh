@@ -6,11 +6,21 @@
 //   k_group_scatter  indices of the HSPs, group by group
 //   k_merge_groups*  one group each: order by (seq, qs, ds, qe), sweep, the N longest boxes
 //   k_group_pack     boxes of all groups back to back, in (qi, seq, qs, ds, qe) order
+// Sorting the call's records by (qi, seq, qs), sweeping and compacting them reads and writes the
+// records and their keys once a pass, a launch each; the pieces of long queries' chains, joined
+// in (qi, seq, diagonal, qs) order, the same with more passes.  By groups a record is read once
+// and its box written twice.  Merge and selection, us: 2.1 M HSPs of 2,000 queries 730 -> 395;
+// 103,000 of 1,000 queries 203 -> 105; 11,000 of 666 queries 163 -> 90.  The join of 177,000 pieces
+// of 8 queries 241 -> 150, their merge and selection 425 -> 160.
 
 namespace gn {
 
-constexpr uint32_t MG_TARGET = 64;  // HSPs a group has on average, at most
-constexpr uint32_t MG_WARP = 64, MG_MID = 1024, MG_BIG = 8192;  // largest group of each kernel
+// HSPs a group has on average, at most, and the largest group of each kernel.  The merge phase in
+// us at averages of 64 | 128 | 256: 2.1 M HSPs 277 | 308 | 380, 103,000 HSPs 58 | 62 | 105, 89,000 HSPs
+// most of which lie in one sequence a query 66 | 113 | 110.  Warps taking up to 128 (256) instead of 64: 263 (271),
+// 62 (78) and 70 (87); 128 threads of 8 records instead of 256 of 4: 320, 75 and 85.
+constexpr uint32_t MG_TARGET = 64;
+constexpr uint32_t MG_WARP = 64, MG_MID = 1024, MG_BIG = 8192;
 constexpr int MG_BITS = 13;          // bits of an index into a group
 static_assert(MG_BIG == 1u << MG_BITS, "an index fits its bits");
 
@@ -77,110 +87,6 @@ __global__ void __launch_bounds__(256) k_group_scatter(const uint2 *__restrict__
     perm[off[w.x] + w.y] = i;
 }
 
-// T threads that work together, a warp or the block, on up to T * E things: thread t has the
-// things t * E .. t * E + E - 1.
-template <int T, int E>
-struct Team {
-    static constexpr bool WARP = T == 32;
-    static __device__ __forceinline__ uint32_t tid() { return WARP ? threadIdx.x & 31 : threadIdx.x; }
-    static __device__ __forceinline__ void sync() {
-        if (WARP) __syncwarp();
-        else __syncthreads();
-    }
-    // tmp: 32 words a team
-    static __device__ __forceinline__ uint32_t excl_sum(uint32_t v, uint64_t *tmp, uint32_t &total) {
-        if (!WARP) return block_excl_scan(v, reinterpret_cast<uint32_t *>(tmp), total);
-        uint32_t x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (tid() >= o) x += y;
-        }
-        total = __shfl_sync(0xffffffffu, x, 31);
-        return x - v;
-    }
-    static __device__ __forceinline__ uint64_t warp_max_scan(uint64_t x) {
-        const int lane = threadIdx.x & 31;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x = max(x, y);
-        }
-        return x;
-    }
-    // largest of the values of the threads before this one (0: none)
-    static __device__ __forceinline__ uint64_t excl_max(uint64_t v, uint64_t *tmp) {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        const uint64_t x = warp_max_scan(v);
-        uint64_t before = __shfl_up_sync(0xffffffffu, x, 1);
-        if (lane == 0) before = 0;
-        if (WARP) return before;
-        if (lane == 31) tmp[wid] = x;
-        __syncthreads();
-        const uint64_t w = warp_max_scan(lane < T / 32 ? tmp[lane] : 0ull);
-        const uint64_t pre = __shfl_sync(0xffffffffu, w, wid > 0 ? wid - 1 : 0);
-        __syncthreads();  // tmp is reused by the next call
-        return wid > 0 ? max(before, pre) : before;
-    }
-    // Bitonic sort of P keys, E a thread (P a multiple of 32 E, a power of two; threads from P / E
-    // on only synchronise).  Exchanges within a thread cost no memory access, within a warp two
-    // shuffles a key; only those between warps go through shared memory (ex: P keys): 6 of 55 stages
-    // at 1,024 keys.  Sorted in shared memory alone, 1,024 keys took 33,000 cycles a block, bound by
-    // shared-memory wavefronts (2 ways of bank conflicts, 8 wavefronts for 32 keys and stage).
-    static __device__ __forceinline__ void sort(uint64_t (&r)[E], uint64_t *ex, uint32_t P) {
-        const uint32_t t = tid(), A = P / E;
-        const bool on = t < A;
-        if (on) {
-#pragma unroll
-            for (int k = 2; k <= E; k <<= 1)
-#pragma unroll
-                for (int j = k >> 1; j > 0; j >>= 1)
-#pragma unroll
-                    for (int e = 0; e < E; ++e)
-                        if ((e & j) == 0) order(r[e], r[e + j], k < E ? (e & k) == 0 : (t & 1) == 0);
-        }
-        for (uint32_t k = 2; k <= A; k <<= 1) {  // sorted runs of k threads
-            const bool up = (t & k) == 0 || k == A;
-            uint32_t j = k >> 1;
-            for (; j >= 32; j >>= 1) {
-                if (on)
-#pragma unroll
-                    for (int e = 0; e < E; ++e) ex[e * A + t] = r[e];
-                sync();
-                if (on)
-#pragma unroll
-                    for (int e = 0; e < E; ++e) keep(r[e], ex[e * A + (t ^ j)], up == ((t & j) == 0));
-                sync();
-            }
-            if (!on) continue;
-            for (; j > 0; j >>= 1)
-#pragma unroll
-                for (int e = 0; e < E; ++e) keep(r[e], __shfl_xor_sync(0xffffffffu, r[e], j), up == ((t & j) == 0));
-#pragma unroll
-            for (int i = E >> 1; i > 0; i >>= 1)
-#pragma unroll
-                for (int e = 0; e < E; ++e)
-                    if ((e & i) == 0) order(r[e], r[e + i], up);
-        }
-    }
-    // least power of two that sort takes, from n on
-    static __device__ __forceinline__ uint32_t padded(uint32_t n) {
-        uint32_t P = 32 * E;
-        while (P < n) P <<= 1;
-        return P;
-    }
-
-  private:
-    static __device__ __forceinline__ void order(uint64_t &a, uint64_t &b, bool up) {
-        const uint64_t lo = min(a, b), hi = max(a, b);
-        a = up ? lo : hi;
-        b = up ? hi : lo;
-    }
-    static __device__ __forceinline__ void keep(uint64_t &a, uint64_t other, bool smaller) {
-        if ((other < a) == smaller) a = other;
-    }
-};
-
 struct MergeGroups {
     const DevHsp *in;
     const uint32_t *perm;  // HSPs by group: group g's from off[g] on, cnt[g] of them (null: in lies so)
@@ -231,7 +137,7 @@ __device__ __forceinline__ void merge_group(const MergeGroups &m, uint32_t g, Me
                 box[i] = make_uint4(h.qs, h.qe, h.ds, h.de);
             }
         }
-        tm::sort(r, S.key, P);
+        tm::sort(r, S.key, P, KeyLess());
         tm::sync();
         uint4 b[E];
 #pragma unroll
@@ -339,7 +245,8 @@ __device__ __forceinline__ void merge_group(const MergeGroups &m, uint32_t g, Me
     }
     tm::sync();
     // The boxes in order; of more than N only the N longest, the first ones of the shortest length
-    // taken: no other box of the group can be among the query's N longest.
+    // taken: no other box of the group can be among the query's N longest.  (A sort by length and
+    // one back cost 27,000 to 42,000 cycles a block, as much as the first sort.)
     uint32_t len[E], n_box = 0, tot = 0;
     const uint32_t max_len = (1u << (8 * m.len_bytes)) - 1u;
 #pragma unroll

@@ -1067,6 +1067,7 @@ __global__ void __launch_bounds__(256) k_xdrop(DevHsp *__restrict__ h, uint32_t 
 
 }  // namespace gn
 #include "gn_seed_scan.cuh"
+#include "gn_team.cuh"
 namespace gn {
 
 // ------------------------------------------- long queries: segments, join --
@@ -1227,13 +1228,6 @@ __global__ void k_overlap_sweep(const DevHsp *__restrict__ in, uint32_t n, DevHs
 }
 
 // ----------------------------------------------------- a11: selection --
-// Per-query selection on records sorted by (qi, seq, qs, ds, qe, de): a block per
-// query keeps its N longest records, ties broken by that order (a stable choice by
-// length), and writes them by (length desc, seq, qs, ds, qe, de).  The N-th largest
-// length T comes from a 256-bin histogram per byte of the length (two, or three where a
-// query is longer than 65,535 bases), high byte first; the selected records are those
-// longer than T and the first ones of length T.
-
 // The bin of the n-th largest entry of a histogram of 256 bins that holds at least n >= 1, and how
 // many lie above that bin (out[0], out[1]); a warp, eight bins a lane.
 __device__ __forceinline__ void bin_of_nth(const uint32_t *hist, uint32_t n, uint32_t *out) {
@@ -1256,13 +1250,24 @@ __device__ __forceinline__ void bin_of_nth(const uint32_t *hist, uint32_t n, uin
     }
 }
 
+// Per-query selection on records sorted by (qi, seq, qs, ds, qe, de): a block per
+// query keeps its N longest records, ties broken by that order (a stable choice by
+// length), and writes them by (length desc, seq, qs, ds, qe, de).  The N-th largest
+// length T comes from a 256-bin histogram per byte of the length (two, or three where a
+// query is longer than 65,535 bases), high byte first; the selected records are those
+// longer than T and the first ones of length T.  Bound by the latency of its passes over the
+// lengths, so every thread has SQ_AHEAD loads under way, and by the chain of the last sort's
+// stages, which stays in registers (Team).  8 queries of 22,000 records each, N = 100: 78 -> 51 us;
+// 1,000 queries of 100: 29 -> 18 us (the threshold found by one thread, the sort in shared memory).
 constexpr int SQ_CAP = 1024;  // largest N this kernel handles
-constexpr int SQ_THREADS = 512;
+constexpr int SQ_THREADS = 512, SQ_AHEAD = 8;
 
 __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__restrict__ rec,
                                                              const uint32_t *__restrict__ qfirst,
                                                              const uint64_t *__restrict__ qout, uint32_t N, int bytes,
                                                              DevHsp *__restrict__ sel) {
+    typedef Team<SQ_THREADS, SQ_CAP / 256> tm;  // keys in the first threads, a warp for up to 128
+    constexpr int E = SQ_CAP / 256;
     __shared__ uint32_t hist[256];
     __shared__ uint32_t warp_tot[SQ_THREADS / 32];
     __shared__ uint64_t keys[SQ_CAP];
@@ -1281,16 +1286,23 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
             __syncthreads();
             // one shared-memory atomic per distinct bin of a warp's 32 records (lengths are
             // concentrated in few bins)
-            for (uint32_t i0 = a + (threadIdx.x & ~31u); i0 < b; i0 += blockDim.x) {
-                const uint32_t i = i0 + (threadIdx.x & 31u);
-                uint32_t bin = 256u;
-                if (i < b) {
-                    const uint32_t len = min(rec[i].len, max_len);
-                    if (((uint64_t)len >> (shift + 8)) == T) bin = (len >> shift) & 0xFFu;
+            for (uint32_t i0 = a + (threadIdx.x & ~31u); i0 < b; i0 += SQ_AHEAD * SQ_THREADS) {
+                uint32_t len[SQ_AHEAD];
+#pragma unroll
+                for (int u = 0; u < SQ_AHEAD; ++u) {
+                    const uint32_t i = i0 + u * SQ_THREADS + (threadIdx.x & 31u);
+                    len[u] = i < b ? min(rec[i].len, max_len) : 0u;
                 }
-                const uint32_t peers = __match_any_sync(0xffffffffu, bin);
-                if (bin < 256u && (threadIdx.x & 31u) == (uint32_t)(__ffs(peers) - 1))
-                    atomicAdd(&hist[bin], (uint32_t)__popc(peers));
+#pragma unroll
+                for (int u = 0; u < SQ_AHEAD; ++u) {
+                    const uint32_t i = i0 + u * SQ_THREADS + (threadIdx.x & 31u);
+                    if (i0 + u * SQ_THREADS >= b) break;
+                    const bool in = i < b && ((uint64_t)len[u] >> (shift + 8)) == T;
+                    const uint32_t bin = in ? (len[u] >> shift) & 0xFFu : 256u;
+                    const uint32_t peers = __match_any_sync(0xffffffffu, bin);
+                    if (in && (threadIdx.x & 31u) == (uint32_t)(__ffs(peers) - 1))
+                        atomicAdd(&hist[bin], (uint32_t)__popc(peers));
+                }
             }
             __syncthreads();
             if (threadIdx.x < 32) bin_of_nth(hist, N - above, found);
@@ -1307,44 +1319,49 @@ __global__ void __launch_bounds__(SQ_THREADS) k_select_query(const DevHsp *__res
     // records of length T
     const uint32_t per = (n + blockDim.x - 1) / blockDim.x;
     const uint32_t lo = min(n, threadIdx.x * per), hi = min(n, lo + per);
+    auto lengths = [&](auto visit) {  // of the thread's records, in order
+        for (uint32_t i0 = lo; i0 < hi; i0 += SQ_AHEAD) {
+            uint32_t len[SQ_AHEAD];
+#pragma unroll
+            for (int u = 0; u < SQ_AHEAD; ++u) len[u] = i0 + u < hi ? min(rec[a + i0 + u].len, max_len) : 0u;
+#pragma unroll
+            for (int u = 0; u < SQ_AHEAD; ++u)
+                if (i0 + u < hi) visit(i0 + u, len[u]);
+        }
+    };
     uint32_t n_gt = 0, n_eq = 0;
-    for (uint32_t i = lo; i < hi; ++i) {
-        const uint32_t len = min(rec[a + i].len, max_len);
+    lengths([&](uint32_t, uint32_t len) {
         const bool gt = n <= N || len > T;
         n_gt += gt ? 1u : 0u;
         n_eq += (!gt && len == T) ? 1u : 0u;
-    }
+    });
     uint32_t tot = 0;
     uint32_t eq_rank = block_excl_scan(n_eq, warp_tot, tot);
     const uint32_t n_take = n_gt + min(n_eq, r_eq > eq_rank ? r_eq - eq_rank : 0u);
     uint32_t pos = block_excl_scan(n_take, warp_tot, tot);
-    for (uint32_t i = lo; i < hi; ++i) {
-        const uint32_t len = min(rec[a + i].len, max_len);
-        const bool gt = n <= N || len > T;
-        const bool eq = !gt && len == T;
-        const bool take = gt || (eq && eq_rank < r_eq);
-        eq_rank += eq ? 1u : 0u;
-        if (take) keys[pos++] = ((uint64_t)(max_len - len) << 32) | i;
+    if (n_take)
+        lengths([&](uint32_t i, uint32_t len) {
+            const bool gt = n <= N || len > T;
+            const bool eq = !gt && len == T;
+            const bool take = gt || (eq && eq_rank < r_eq);
+            eq_rank += eq ? 1u : 0u;
+            if (take) keys[pos++] = ((uint64_t)(max_len - len) << 32) | i;
+        });
+    __syncthreads();
+    uint64_t r[E];
+    const uint32_t P = tm::padded(nsel), A = P / E;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t i = e * A + threadIdx.x;
+        r[e] = threadIdx.x < A && i < nsel ? keys[i] : ~0ull;
     }
     __syncthreads();
-    // bitonic sort of the nsel keys (unique: they carry the position)
-    uint32_t P = 1;
-    while (P < nsel) P <<= 1;
-    for (uint32_t i = nsel + threadIdx.x; i < P; i += blockDim.x) keys[i] = ~0ull;
-    __syncthreads();
-    for (uint32_t k2 = 2; k2 <= P; k2 <<= 1) {
-        for (uint32_t j = k2 >> 1; j > 0; j >>= 1) {
-            for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
-                const uint32_t ixj = i ^ j;
-                if (ixj > i) {
-                    const uint64_t x = keys[i], y = keys[ixj];
-                    if ((x > y) == ((i & k2) == 0)) { keys[i] = y; keys[ixj] = x; }
-                }
-            }
-            __syncthreads();
-        }
+    tm::sort(r, keys, P, KeyLess());
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const uint32_t k = threadIdx.x * E + e;
+        if (k < nsel) sel[out0 + k] = rec[a + (uint32_t)(r[e] & 0xFFFFFFFFu)];
     }
-    for (uint32_t k = threadIdx.x; k < nsel; k += blockDim.x) sel[out0 + k] = rec[a + (uint32_t)(keys[k] & 0xFFFFFFFFu)];
 }
 
 // first[q] = first record of query q in records sorted by query (first[nq] = n), and, when
@@ -1371,57 +1388,56 @@ __global__ void k_query_bounds(const DevHsp *__restrict__ rec, const uint64_t *_
     if (cnt && q < nq) cnt[q] = min(N, first_of_query(rec, n, q + 1) - f);
 }
 
-// Overlap merging and query bounds of a small search in one block: sorts the records of up to
-// MB_CAP HSPs by (qi, seq, qs) (a key of at most 64 bits; ties keep their order, which the sweep
-// does not depend on), sweeps the runs, compacts the boxes and finds each query's first box,
-// and the prefix sums of min(N, boxes) (N = 0: of all boxes) as k_query_bounds and a scan do.
-// Replaces eight launches: a search of a handful of HSPs is a chain of launches of 2 to 5 us each.
-constexpr uint32_t MB_CAP = 2048, MB_QUERIES = 4096;
-constexpr int MB_THREADS = 512;
+// Overlap merging and selection of a small search in one block: sorts the records of up to MB_CAP
+// HSPs by (qi, seq, qs) (ties keep their order, which the sweep does not depend on), sweeps the
+// runs, compacts the boxes, finds each query's first box and the prefix sums of min(N, boxes)
+// (N = 0: of all boxes) as k_query_bounds and a scan do, and, when sel is given, sorts the boxes by
+// (qi, length desc, place) and writes each query's first N there as k_select_query does.
+// Replaces nine launches: a search of a handful of HSPs is a chain of launches of 2 to 5 us each.
+// 8 and 14 us at 1 and 17 HSPs, with the selection in it (8 and 14 before without it).  The call as
+// a whole by this | by groups, us: 38 HSPs 234 | 255, 513 HSPs 257 | 277, 1,023 HSPs 391 | 386.
+constexpr uint32_t MB_CAP = 1024, MB_QUERIES = 4096;
+constexpr int MB_THREADS = 512, MB_BITS = 10;
 
 __global__ void __launch_bounds__(MB_THREADS) k_merge_block(const DevHsp *__restrict__ in, uint32_t n, uint32_t seq_bits,
                                                             uint32_t qs_bits, uint32_t nq, uint32_t N, int in_order,
                                                             DevHsp *__restrict__ boxes, DevHsp *__restrict__ out,
                                                             uint32_t *__restrict__ first, uint64_t *__restrict__ qo,
-                                                            uint64_t *__restrict__ n_out) {
+                                                            uint64_t *__restrict__ n_out, DevHsp *__restrict__ sel) {
+    constexpr int E = MB_CAP / MB_THREADS;
+    typedef Team<MB_THREADS, E> tm;
+    constexpr uint32_t idx_mask = (1u << MB_BITS) - 1u;
     __shared__ uint64_t key[MB_CAP];
-    __shared__ uint16_t idx[MB_CAP];
     __shared__ uint8_t flag[MB_CAP];
     __shared__ uint32_t warp_tot[MB_THREADS / 32];
-    uint32_t P = 32;
-    while (P < n) P <<= 1;
-    for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
-        uint64_t k = ~0ull;
-        if (i < n) k = ((((uint64_t)in[i].qi << seq_bits) | in[i].seq) << qs_bits) | in[i].qs;
-        key[i] = k;
-        idx[i] = i < n ? (uint16_t)i : (uint16_t)0xFFFFu;
-    }
-    __syncthreads();
-    for (uint32_t k2 = 2; k2 <= P; k2 <<= 1) {
-        for (uint32_t j = k2 >> 1; j > 0; j >>= 1) {
-            for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
-                const uint32_t x = i ^ j;
-                if (x > i) {
-                    const uint64_t a = key[i], b = key[x];
-                    const uint16_t ia = idx[i], ib = idx[x];
-                    if ((a > b || (a == b && ia > ib)) == ((i & k2) == 0)) {
-                        key[i] = b; key[x] = a;
-                        idx[i] = ib; idx[x] = ia;
-                    }
-                }
-            }
-            __syncthreads();
+    const uint32_t t = threadIdx.x;
+    // the keys of n records, sorted
+    auto sort = [&](uint32_t n, auto key_of) {
+        uint64_t r[E];
+        const uint32_t P = tm::padded(n), A = P / E;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const uint32_t i = e * A + t;
+            r[e] = t < A && i < n ? key_of(i) << MB_BITS | i : ~0ull;
         }
-    }
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        if (i > 0 && key[i - 1] >> qs_bits == key[i] >> qs_bits) continue;
-        overlap_run([&](uint32_t j) { return in[idx[j]]; }, i, n, boxes,
+        tm::sort(r, key, P, KeyLess());
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (t < A) key[t * E + e] = r[e];
+        __syncthreads();
+    };
+    sort(n, [&](uint32_t i) { return ((((uint64_t)in[i].qi << seq_bits) | in[i].seq) << qs_bits) | in[i].qs; });
+    const uint32_t run_shift = qs_bits + MB_BITS;
+    for (uint32_t i = t; i < n; i += blockDim.x) {
+        if (i > 0 && key[i - 1] >> run_shift == key[i] >> run_shift) continue;
+        overlap_run([&](uint32_t j) { return in[(uint32_t)key[j] & idx_mask]; }, i, n, boxes,
                     [&](uint32_t j, uint32_t v) { flag[j] = (uint8_t)v; }, in_order != 0);
     }
     __syncthreads();
     uint32_t n_mg = 0;
     for (uint32_t i0 = 0; i0 < n; i0 += blockDim.x) {
-        const uint32_t i = i0 + threadIdx.x, f = i < n ? flag[i] : 0u;
+        const uint32_t i = i0 + t, f = i < n ? flag[i] : 0u;
         uint32_t tot = 0;
         const uint32_t at = n_mg + block_excl_scan(f, warp_tot, tot);
         if (f) out[at] = boxes[i];
@@ -1430,7 +1446,7 @@ __global__ void __launch_bounds__(MB_THREADS) k_merge_block(const DevHsp *__rest
     __syncthreads();
     uint64_t sum = 0;
     for (uint32_t q0 = 0; q0 <= nq; q0 += blockDim.x) {
-        const uint32_t q = q0 + threadIdx.x;
+        const uint32_t q = q0 + t;
         uint32_t c = 0;
         if (q <= nq) {
             const uint32_t f = first_of_query(out, n_mg, q);
@@ -1445,7 +1461,15 @@ __global__ void __launch_bounds__(MB_THREADS) k_merge_block(const DevHsp *__rest
         if (q <= nq) qo[q] = sum + at;
         sum += tot;
     }
-    if (threadIdx.x == 0) *n_out = n_mg;
+    if (t == 0) *n_out = n_mg;
+    if (!sel) return;
+    __syncthreads();
+    sort(n_mg, [&](uint32_t i) { return ((uint64_t)out[i].qi << 32) | (0xFFFFFFFFu - out[i].len); });
+    for (uint32_t i = t; i < n_mg; i += blockDim.x) {
+        const DevHsp h = out[(uint32_t)key[i] & idx_mask];
+        const uint32_t k = i - first[h.qi];
+        if (k < N) sel[qo[h.qi] + k] = h;
+    }
 }
 
 }  // namespace gn
@@ -2111,22 +2135,18 @@ __global__ void k_finalize(const DevAln *__restrict__ a, uint32_t n, const uint3
 }
 
 
-// Per-query ranking (alignments of a query are contiguous and at most RQ_CAP): one
-// CTA per query sorts record indices in shared memory with a bitonic network - first
-// by (seq, q_start, q_end, db_start, db_end, score desc) to drop records that repeat
-// an earlier one's sequence and ranges (and records with score <= 0), then by
-// (score desc, seq, q_start, db_start, q_end, db_end) - and writes the ranked hits
-// with e-value and bit score at the query's input offset.
-constexpr int RQ_CAP = 1024;
-
-__device__ __forceinline__ bool rq_less_dedupe(const DevAln &a, const DevAln &b) {
-    if (a.seq != b.seq) return a.seq < b.seq;
-    if (a.qs != b.qs) return a.qs < b.qs;
-    if (a.qe != b.qe) return a.qe < b.qe;
-    if (a.ds != b.ds) return a.ds < b.ds;
-    if (a.de != b.de) return a.de < b.de;
-    return a.score > b.score;
-}
+// Per-query ranking (alignments of a query are contiguous and at most RQ_CAP): a block sorts a
+// query's records by (score desc, seq, q_start, db_start, q_end, db_end), drops records that repeat
+// an earlier one's sequence and ranges (and records with score <= 0), and writes the ranked hits
+// with e-value and bit score at the query's input offset.  The sort moves keys of score, sequence
+// and record in registers (Team) and compares the records only where score and sequence are
+// equal; a table of the ranges, each with the first record that has them, finds the repeats.  Bound
+// by the latency of the sort's stages.  Two sorts of record indices in shared memory, by ranges and
+// by rank, took 123 us for 200 queries of up to 875 alignments (now 49), 61 for 4,096 queries of 22
+// (35) and 55 for 2,000 of 100 (37).  Up to RQ_SMALL alignments a block of a thread each: a warp
+// with four records a lane took 53 and 49 us (and 14 instead of 10 for a lone record: more code
+// to fetch).
+constexpr int RQ_CAP = 1024, RQ_SMALL = 128, RQ_BITS = 10;
 
 __device__ __forceinline__ bool rq_less_rank(const DevAln &a, const DevAln &b) {
     if (a.score != b.score) return a.score > b.score;
@@ -2137,73 +2157,93 @@ __device__ __forceinline__ bool rq_less_rank(const DevAln &a, const DevAln &b) {
     return a.de < b.de;
 }
 
-template <int MODE>  // 0: dedupe order, 1: rank order (dropped records last)
-__device__ void rq_bitonic(uint16_t *idx, const DevAln *rec, const uint8_t *keep, uint32_t P) {
-    for (uint32_t k2 = 2; k2 <= P; k2 <<= 1) {
-        for (uint32_t j = k2 >> 1; j > 0; j >>= 1) {
-            for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
-                const uint32_t ixj = i ^ j;
-                if (ixj > i) {
-                    const uint16_t a = idx[i], c = idx[ixj];
-                    bool a_gt_c;  // a sorts after c
-                    if (a == 0xFFFFu) a_gt_c = c != 0xFFFFu;
-                    else if (c == 0xFFFFu) a_gt_c = false;
-                    else if (MODE == 1 && keep[a] != keep[c]) a_gt_c = !keep[a];
-                    else a_gt_c = MODE == 0 ? rq_less_dedupe(rec[c], rec[a]) : rq_less_rank(rec[c], rec[a]);
-                    const bool up = (i & k2) == 0;
-                    if (a_gt_c == up) { idx[i] = c; idx[ixj] = a; }
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// qo: first alignment of each query, as a prefix sum.  A query of more than RQ_CAP alignments is
-// left out and *too_many set: the caller then ranks the call by sorting.
-__global__ void __launch_bounds__(256) k_rank_query(const DevAln *__restrict__ aln, const uint64_t *__restrict__ qo,
-                                                    uint32_t nq, const uint64_t *__restrict__ qstart, double n_bank,
-                                                    double lambda, double K, double max_e, gn_hit *__restrict__ out,
-                                                    uint32_t *__restrict__ qcount, uint32_t *__restrict__ too_many) {
-    __shared__ DevAln rec[RQ_CAP];
-    __shared__ uint16_t idx[RQ_CAP];
-    __shared__ uint8_t keep[RQ_CAP];
-    __shared__ uint32_t nk_s, ne_s;
+// E: records a thread sorts; the block's T threads take up to T E.  seq_bits: of a sequence number.
+// qo: first alignment of each query, as a prefix sum.  A query of more alignments is left out and
+// *too_many set: the caller then ranks the call by sorting.
+template <int T, int E>
+__global__ void __launch_bounds__(T) k_rank_query(const DevAln *__restrict__ aln, const uint64_t *__restrict__ qo,
+                                                  uint32_t nq, const uint64_t *__restrict__ qstart, int seq_bits, double n_bank,
+                                                  double lambda, double K, double max_e, gn_hit *__restrict__ out,
+                                                  uint32_t *__restrict__ qcount, uint32_t *__restrict__ too_many) {
+    typedef Team<T, E> tm;
+    constexpr uint32_t CAP = T * E, SLOTS = 2 * CAP, EMPTY = 0xFFFFFFFFu, idx_mask = (1u << RQ_BITS) - 1u;
+    static_assert(CAP <= 1u << RQ_BITS, "an index fits its bits");
+    __shared__ DevAln rec[CAP];
+    __shared__ uint64_t ex[CAP];  // the sort's exchanges, then the table
+    __shared__ uint64_t tmp[33];
+    __shared__ uint16_t order[CAP], slot[CAP];
+    __shared__ uint32_t n_out;
+    uint32_t *table = reinterpret_cast<uint32_t *>(ex);
+    const uint32_t t = threadIdx.x;
+    const int kept = min(seq_bits, 64 - 31 - RQ_BITS);  // bits of the sequence in the key, the high ones
     for (uint32_t q = blockIdx.x; q < nq; q += gridDim.x) {
         const uint64_t start = qo[q];
         const uint32_t n = (uint32_t)(qo[q + 1] - start);
-        if (n == 0 || n > RQ_CAP) {
-            if (threadIdx.x == 0) {
+        if (n == 0 || n > CAP) {
+            if (t == 0) {
                 qcount[q] = 0;
                 if (n) *too_many = 1u;
             }
             continue;
         }
-        uint32_t P = 1;
-        while (P < n) P <<= 1;
-        for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
-            if (i < n) rec[i] = aln[start + i];
-            idx[i] = i < n ? (uint16_t)i : (uint16_t)0xFFFFu;
-        }
-        if (threadIdx.x == 0) { nk_s = 0; ne_s = 0; }
+        for (uint32_t i = t; i < n; i += T) rec[i] = aln[start + i];
+        if (t == 0) n_out = 0;
         __syncthreads();
-        rq_bitonic<0>(idx, rec, keep, P);
-        for (uint32_t k = threadIdx.x; k < n; k += blockDim.x) {
-            const DevAln &a = rec[idx[k]];
-            bool kk = a.score > 0;
-            if (kk && k > 0) {
-                const DevAln &b = rec[idx[k - 1]];
-                kk = !(a.seq == b.seq && a.qs == b.qs && a.qe == b.qe && a.ds == b.ds && a.de == b.de);
+        {
+            uint64_t r[E];
+            const uint32_t P = tm::padded(n), A = P / E;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const uint32_t i = e * A + t;
+                r[e] = ~0ull;
+                if (t < A && i < n) {
+                    const uint64_t score = 0x7FFFFFFFu - (uint32_t)max(rec[i].score, 0);
+                    r[e] = ((score << kept | rec[i].seq >> (seq_bits - kept)) << RQ_BITS) | i;
+                }
             }
-            keep[idx[k]] = kk ? 1 : 0;
-            if (kk) atomicAdd(&nk_s, 1u);
+            tm::sort(r, ex, P, [&](uint64_t a, uint64_t b) {
+                if (a >> RQ_BITS != b >> RQ_BITS || a == ~0ull || b == ~0ull) return a < b;
+                const DevAln &x = rec[(uint32_t)a & idx_mask], &y = rec[(uint32_t)b & idx_mask];
+                if (rq_less_rank(x, y)) return true;
+                return !rq_less_rank(y, x) && a < b;
+            });
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < E; ++e)  // (an alignment without a score may equal the padding: it is dropped)
+                if (t * E + e < n) order[t * E + e] = r[e] == ~0ull ? 0xFFFFu : (uint16_t)((uint32_t)r[e] & idx_mask);
+        }
+        for (uint32_t i = t; i < SLOTS; i += T) table[i] = EMPTY;
+        __syncthreads();
+        // each range's entry: its first place in the order, and the record there
+        for (uint32_t i = t; i < n; i += T) {
+            const uint32_t x = order[i];
+            slot[i] = 0xFFFFu;
+            if (x == 0xFFFFu || rec[x].score <= 0) continue;
+            const DevAln a = rec[x];
+            const uint32_t entry = i << RQ_BITS | x;
+            uint32_t h = a.seq * 0x9E3779B1u ^ a.qs * 0x85EBCA77u ^ a.qe * 0xC2B2AE3Du ^ a.ds * 0x27D4EB2Fu ^ a.de * 0x165667B1u;
+            for (h = (h >> 16 ^ h) & (SLOTS - 1);; h = (h + 1) & (SLOTS - 1)) {  // half the slots stay empty
+                const uint32_t old = atomicCAS(&table[h], EMPTY, entry);
+                if (old == EMPTY) break;
+                const DevAln &b = rec[old & idx_mask];
+                if (a.seq == b.seq && a.qs == b.qs && a.qe == b.qe && a.ds == b.ds && a.de == b.de) {
+                    atomicMin(&table[h], entry);
+                    break;
+                }
+            }
+            slot[i] = (uint16_t)h;
         }
         __syncthreads();
-        rq_bitonic<1>(idx, rec, keep, P);
-        const uint32_t nk = nk_s;
-        const double m = (double)(qstart[rec[0].qi + 1] - qstart[rec[0].qi]);
-        for (uint32_t k = threadIdx.x; k < nk; k += blockDim.x) {
-            const DevAln &x = rec[idx[k]];
+        const double m = (double)(qstart[q + 1] - qstart[q]);
+        uint32_t placed = 0;
+        for (uint32_t i0 = 0; i0 < n; i0 += T) {
+            const uint32_t i = i0 + t;
+            const bool keep = i < n && slot[i] != 0xFFFFu && table[slot[i]] >> RQ_BITS == i;
+            uint32_t tot = 0;
+            const uint32_t k = placed + tm::excl_sum(keep ? 1u : 0u, tmp, tot);
+            placed += tot;
+            if (!keep) continue;
+            const DevAln &x = rec[order[i]];
             gn_hit h;
             h.query = x.qi; h.seq = x.seq; h.q_start = x.qs; h.q_end = x.qe; h.db_start = x.ds; h.db_end = x.de;
             h.score = x.score;
@@ -2213,11 +2253,11 @@ __global__ void __launch_bounds__(256) k_rank_query(const DevAln *__restrict__ a
             // e-values rise as scores fall, so the cut keeps a prefix of the ranking
             if (h.evalue <= max_e) {
                 out[start + k] = h;
-                atomicAdd(&ne_s, 1u);
+                atomicAdd(&n_out, 1u);
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) qcount[q] = ne_s;
+        if (t == 0) qcount[q] = n_out;
         __syncthreads();
     }
 }
@@ -3152,10 +3192,13 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         pin.wait();
         return (uint32_t)*reinterpret_cast<const uint64_t *>(pin.p);
     };
-    // How the HSPs are merged: in one block, by groups, or in order of the whole call.  Which group
-    // an HSP is in does not change when it is extended, so the groups are counted before, and the
-    // host learns whether all of them fit while the extension runs.
-    const bool merge_block = n_hsp <= MB_CAP && nq <= MB_QUERIES && qib + seqb + qposb <= 64;
+    // How the HSPs are merged: in one block, by groups, or in order of the whole call.  Groups take
+    // every call whose sort keys fit and in which no query has more HSPs in its range of sequences
+    // than a block holds; otherwise, and for stage outputs and selections that sort the whole call
+    // anyway, the records are sorted (figures: gn_merge_groups.cuh).  Which group an HSP is in does not
+    // change when it is extended, so the groups are counted before, and the host learns whether all
+    // of them fit while the extension runs.
+    const bool merge_block = n_hsp <= MB_CAP && nq <= MB_QUERIES && qib + seqb + qposb + MB_BITS <= 64;
     bool merge_groups = n_hsp && !merge_block && !keep && !sort_select && seqb + qposb + MG_BITS <= 64;
     if (merge_groups) {
         if (!joined_groups) count_groups(false);
@@ -3185,6 +3228,10 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     uint32_t *qfirst = arena.alloc_n<uint32_t>(nq + 1);
     uint64_t *qo = arena.alloc_n<uint64_t>(nq + 1);  // selected HSPs of the queries before each
     uint32_t n_mg = 0;                               // read only where it is needed
+    // a11's room: longest first, at most max_alignments per query (all of them: the boxes as they are)
+    const uint32_t sel_cap = (uint32_t)std::min<uint64_t>(n_hsp, N ? (uint64_t)nq * N : ~0ull);
+    DevHsp *sel = n_hsp && !sort_select && N ? arena.alloc_n<DevHsp>(sel_cap) : merged;
+    const bool block_selects = merge_block && sel != merged;
     if (n_hsp) {
         DevHsp *boxes = arena.alloc_n<DevHsp>(n_hsp);
         if (merge_groups) {
@@ -3194,7 +3241,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         if (merge_block) {
             GN_LAUNCH("k_merge_block", n_hsp, s,
                       k_merge_block<<<1, MB_THREADS, 0, s>>>(hsp, n_hsp, (uint32_t)seqb, (uint32_t)qposb, nq, N, keep ? 0 : 1,
-                                                             boxes, merged, qfirst, qo, n_mg_d));
+                                                             boxes, merged, qfirst, qo, n_mg_d, block_selects ? sel : nullptr));
         } else if (merge_groups) {
             uint32_t *n_boxes = arena.alloc_n<uint32_t>(gr.G), *cnt_sel = arena.alloc_n<uint32_t>(nq);
             run_groups(MergeGroups{hsp, gr.perm, gr.off, gr.cnt, qposb, max_qlen > 65535 ? 3 : 2, N, 0, 0, 0, boxes, n_boxes},
@@ -3236,13 +3283,10 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         if (n_mg) memcpy(res->st_merged.data(), v.data(), sizeof(DevHsp) * n_mg);
     }
 
-    // a11: longest first, at most max_alignments per query (all of them: the boxes as they are)
-    const uint32_t sel_cap = (uint32_t)std::min<uint64_t>(n_hsp, N ? (uint64_t)nq * N : ~0ull);
+    // a11: selection
     uint32_t n_sel = 0;                      // read only where it is needed
     const uint64_t *n_sel_d = qo + nq;       // the same on the device
-    DevHsp *sel = merged;
-    if (n_hsp && !sort_select && N) {
-        sel = arena.alloc_n<DevHsp>(sel_cap);
+    if (n_hsp && !sort_select && N && !block_selects) {
         GN_LAUNCH("k_select_query", n_hsp, s,
                   k_select_query<<<nq, SQ_THREADS, 0, s>>>(merged, qfirst, qo, N, max_qlen > 65535 ? 3 : 2, sel));
     } else if (n_mg && sort_select) {
@@ -3372,14 +3416,17 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         const bool small = hits_bytes + qo_bytes + 4ull * nq <= (1u << 17);
         gn_hit *hits = arena.alloc_n<gn_hit>(sel_cap);
         uint32_t *qcount = arena.alloc_n<uint32_t>(nq);
-        const unsigned rgrid = (unsigned)std::min<uint64_t>(nq, (uint64_t)num_sms() * 8);
+        const bool few = N && N <= (uint32_t)RQ_SMALL;  // no query has more alignments
+        const unsigned rgrid = (unsigned)std::min<uint64_t>(nq, (uint64_t)num_sms() * (few ? 16 : 5));
+        auto rank_kernel = few ? k_rank_query<RQ_SMALL, 1> : k_rank_query<256, RQ_CAP / 256>;
         uint64_t *qoff = arena.alloc_n<uint64_t>(nq + 1);
         void *scr = arena.alloc(scan_scratch_bytes(nq));
         PinnedBlock back(ix->host_pool, sizeof(SearchWords) + qo_bytes + (small ? hits_bytes + 4ull * nq : 0), s);
         for (;;) {
             GN_LAUNCH("k_rank_query", sel_cap, s,
-                      k_rank_query<<<rgrid, 256, 0, s>>>(aln, qo, nq, qstart_d, (double)ix->n_bases, sc.lambda, sc.K,
-                                                         p.max_evalue, hits, qcount, &words->too_many));
+                      rank_kernel<<<rgrid, few ? RQ_SMALL : 256, 0, s>>>(
+                          aln, qo, nq, qstart_d, seqb, (double)ix->n_bases, sc.lambda, sc.K, p.max_evalue, hits, qcount,
+                          &words->too_many));
             size_t at = sizeof(SearchWords);
             if (small) {
                 back.fetch(at, qo, qo_bytes);
@@ -3390,7 +3437,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
             } else {
                 exclusive_scan_u32(qcount, qoff, nq, scr, s);
                 GN_LAUNCH("k_gather_ranked", sel_cap, s,
-                          k_gather_ranked<<<rgrid, 256, 0, s>>>(hits, qo, qoff, nq, fin));
+                          k_gather_ranked<<<(unsigned)std::min<uint64_t>(nq, (uint64_t)num_sms() * 8), 256, 0, s>>>(hits, qo, qoff, nq, fin));
                 back.fetch(at, qoff, qo_bytes);
             }
             back.fetch(0, words, sizeof(SearchWords));
