@@ -31,17 +31,25 @@ constexpr int WIN_CHUNK = 32 * WIN_J;
 // of every valid window, in window order from the chunk's first slot, and the bucket
 // histogram.  One count per chunk and a ballot rank give the slots, so that no flag or slot
 // per window goes through memory (400 Mbp, 36.4 M windows: flags, their scan and the two
-// window passes 0.9 GB, now 0.45 GB).
+// window passes 0.9 GB, now 0.45 GB).  The number of windows, woff[n_seqs], is known to the device
+// only: n_chunks is as many chunks as there can be.  prev (a key's bits above the code are
+// free): the base before the window goes along there, so that its signature needs no look at it.
+constexpr int PREV_SHIFT = 61;
+
 template <bool COUNT>
 __global__ void k_bank_windows(const uint64_t *__restrict__ seq_start, const uint64_t *__restrict__ woff,
-                               uint32_t n_seqs, uint64_t W, const uint32_t *__restrict__ pk,
-                               const uint32_t *__restrict__ nb, SeedShape sh, int t, uint32_t *__restrict__ count,
-                               uint32_t *__restrict__ hist, const uint64_t *__restrict__ first,
-                               uint64_t *__restrict__ keys) {
+                               uint32_t n_seqs, uint64_t n_chunks, const uint32_t *__restrict__ pk,
+                               const uint32_t *__restrict__ nb, SeedShape sh, int t, bool prev,
+                               uint32_t *__restrict__ count, uint32_t *__restrict__ hist,
+                               const uint64_t *__restrict__ first, uint64_t *__restrict__ keys) {
     const int lane = threadIdx.x & 31;
     const uint64_t chunk = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t w0 = chunk * WIN_CHUNK;
-    if (w0 >= W) return;
+    const uint64_t w0 = chunk * WIN_CHUNK, W = woff[n_seqs];
+    if (chunk >= n_chunks) return;
+    if (w0 >= W) {
+        if (COUNT && lane == 0) count[chunk] = 0;
+        return;
+    }
     uint32_t s = 0;
     if (lane == 0) s = dev_upper_index(woff, n_seqs + 1, w0);
     s = __shfl_sync(0xffffffffu, s, 0);
@@ -64,7 +72,9 @@ __global__ void k_bank_windows(const uint64_t *__restrict__ seq_start, const uin
             if (ok) {
                 const uint32_t code = dev_seed_code(pk, g, sh);
                 atomicAdd(&hist[code], 1u);
-                keys[slot + __popc(m & ((1u << lane) - 1u))] = ((uint64_t)code << 32) | g;
+                uint64_t key = ((uint64_t)code << 32) | g;
+                if (prev) key |= (uint64_t)(g > seq_start[s] ? dev_base(pk, nb, g - 1) : SIG_NO_BASE) << PREV_SHIFT;
+                keys[slot + __popc(m & ((1u << lane) - 1u))] = key;
             }
             slot += __popc(m);
         }
@@ -97,25 +107,60 @@ __device__ __forceinline__ uint32_t occurrence_sig(uint64_t g, uint64_t n, const
 }
 
 // Occurrences and their signatures from the sorted keys (keys null: signatures of the
-// occurrences that post already holds).  post and sig: post_alloc_entries words.
+// occurrences that post already holds).  post and sig: post_alloc_entries words.  prev: the keys
+// hold the base before the window, and the signature costs the gather after it alone (build of
+// 400 M occurrences at stride 1: 29.3 -> 23.0 ms).
 __global__ void k_occurrences(const uint64_t *__restrict__ keys, uint64_t n_post, uint32_t *__restrict__ post,
                               uint32_t *__restrict__ sig, uint64_t n, const uint32_t *__restrict__ pk,
-                              const uint32_t *__restrict__ nb, SeqMap sm, SeedShape sh, int t, int kind) {
+                              const uint32_t *__restrict__ nb, SeqMap sm, SeedShape sh, int t, int kind, bool prev) {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_post) return;
-    const uint32_t g = keys ? (uint32_t)keys[i] : post[i];
+    const uint64_t key = keys ? keys[i] : (uint64_t)post[i];
+    const uint32_t g = (uint32_t)key;
     if (keys) post[i] = g;
-    if (sig) sig[i] = occurrence_sig(g, n, pk, nb, sm, sh, t, kind);
+    if (!sig) return;
+    if (prev) {
+        const uint64_t x = (uint64_t)g + (uint64_t)sh.span;
+        sig[i] = (uint32_t)(key >> PREV_SHIFT) | (x <= n ? sig_flank(pk, x) : 0u);
+    } else {
+        sig[i] = occurrence_sig(g, n, pk, nb, sm, sh, t, kind);
+    }
 }
 
-// Room for the signatures; without it searches take the path that does not read them.
-static void alloc_sigs(gn_index *ix, uint64_t &bytes) {
-    const size_t want = sizeof(uint32_t) * post_alloc_entries(ix->n_postings);
-    if (cudaMalloc(&ix->sig_d, want) == cudaSuccess) {
-        bytes += sizeof(uint32_t) * ix->n_postings;
+// Device memory of an index: two blocks, one of what the bank's size decides, one of what the
+// number of occurrences decides.  An allocation or a release is 10 to 100 us of host time; with seven
+// of each, build | release took 354 | 152 us at 1.25 Mbp and 2,954 | 507 us at 400 Mbp, now 281 | 111
+// and 2,780 | 339.
+static void alloc_fixed(gn_index *ix, uint64_t ns, uint64_t n, uint64_t nbk, uint64_t nlut) {
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+        const size_t from = at;
+        at += (bytes + 255) / 256 * 256;
+        return from;
+    };
+    const size_t start = place(8 * (ns + 1)), pk = place(4 * Packed::pk_words(n)), nb = place(4 * Packed::nb_words(n)),
+                 off = place(8 * (nbk + 1)), lut = place(4 * nlut);
+    GN_CUDA(cudaMalloc(&ix->fixed_d, at));
+    ix->seq_start_d = reinterpret_cast<uint64_t *>(ix->fixed_d + start);
+    ix->bank.pk = reinterpret_cast<uint32_t *>(ix->fixed_d + pk);
+    ix->bank.nb = reinterpret_cast<uint32_t *>(ix->fixed_d + nb);
+    ix->off_d = reinterpret_cast<uint64_t *>(ix->fixed_d + off);
+    ix->seq_lut_d = reinterpret_cast<uint32_t *>(ix->fixed_d + lut);
+    ix->device_bytes = 8 * (ns + 1) + 4 * (Packed::pk_words(n) + Packed::nb_words(n)) + 8 * (nbk + 1) + 4 * nlut;
+}
+
+// The occurrences and their signatures; without room for those searches take the path that does
+// not read them.
+static void alloc_occurrences(gn_index *ix) {
+    const size_t want = (sizeof(uint32_t) * post_alloc_entries(ix->n_postings) + 255) / 256 * 256;
+    if (cudaMalloc(&ix->post_d, 2 * want) == cudaSuccess) {
+        ix->sig_d = ix->post_d + want / sizeof(uint32_t);
+        ix->device_bytes += 2 * sizeof(uint32_t) * ix->n_postings;
     } else {
         cudaGetLastError();
+        GN_CUDA(cudaMalloc(&ix->post_d, want));
         ix->sig_d = nullptr;
+        ix->device_bytes += sizeof(uint32_t) * ix->n_postings;
     }
 }
 
@@ -180,20 +225,11 @@ static void index_build_shape(const gn_bank *db, int k, int span, uint32_t keep,
     const SeedShape sh{k, span, keep};
 
     const uint64_t nbk = 1ull << (2 * k);
-    uint64_t bytes = 0;
-    GN_CUDA(cudaMalloc(&ix->seq_start_d, sizeof(uint64_t) * (ns + 1)));
-    bytes += sizeof(uint64_t) * (ns + 1);
-    GN_CUDA(cudaMalloc(&ix->bank.pk, 4 * Packed::pk_words(n)));
-    GN_CUDA(cudaMalloc(&ix->bank.nb, 4 * Packed::nb_words(n)));
-    bytes += 4 * (Packed::pk_words(n) + Packed::nb_words(n));
-    GN_CUDA(cudaMalloc(&ix->off_d, sizeof(uint64_t) * (nbk + 1)));
-    bytes += sizeof(uint64_t) * (nbk + 1);
+    const uint64_t nlut = (n >> SEQ_LUT_SHIFT) + 1;
+    alloc_fixed(ix, ns, n, nbk, nlut);
     GN_CUDA(cudaMemcpyAsync(ix->seq_start_d, ix->seq_start_h.data(), sizeof(uint64_t) * (ns + 1),
                             cudaMemcpyHostToDevice, s));
     // sequence lookup table: the sequence holding each block of 2^SEQ_LUT_SHIFT bases
-    const uint64_t nlut = (n >> SEQ_LUT_SHIFT) + 1;
-    GN_CUDA(cudaMalloc(&ix->seq_lut_d, sizeof(uint32_t) * nlut));
-    bytes += sizeof(uint32_t) * nlut;
     if (ns > 0)
         GN_LAUNCH("k_seq_lut", nlut, s,
                   k_seq_lut<<<(unsigned)((nlut + 255) / 256), 256, 0, s>>>(ix->seq_start_d, ns, n, nlut, ix->seq_lut_d));
@@ -222,18 +258,18 @@ static void index_build_shape(const gn_bank *db, int k, int span, uint32_t keep,
     }
     void *scan_scr = arena.alloc(std::max(scan_scratch_bytes(ns), scan_scratch_bytes(nbk)));
     exclusive_scan_u32(wcnt, woff, ns, scan_scr, s);
-    uint64_t W = 0;
-    GN_CUDA(cudaMemcpyAsync(&W, woff + ns, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    GN_CUDA(cudaStreamSynchronize(s));
 
     // K2: valid windows per chunk and their exclusive scan
-    const uint64_t chunks = (W + WIN_CHUNK - 1) / WIN_CHUNK;
+    const uint64_t w_max = n / (uint64_t)t + ns;  // at most one window a sequence more than its share
+    const uint64_t chunks = (w_max + WIN_CHUNK - 1) / WIN_CHUNK;
     const unsigned grid = (unsigned)std::max<uint64_t>(1, (chunks * 32 + 255) / 256);
+    const SigKind kind = sig_kind(k, span, t);
+    const bool prev = kind == SIG_FLANK && 32 + 2 * k <= PREV_SHIFT;
     uint32_t *ccnt = arena.alloc_n<uint32_t>(chunks);
     uint64_t *coff = arena.alloc_n<uint64_t>(chunks + 1);
-    if (W) {
-        GN_LAUNCH("k_bank_windows_count", W, s,
-                  k_bank_windows<true><<<grid, 256, 0, s>>>(ix->seq_start_d, woff, ns, W, ix->bank.pk, ix->bank.nb, sh, t,
+    if (chunks) {
+        GN_LAUNCH("k_bank_windows_count", w_max, s,
+                  k_bank_windows<true><<<grid, 256, 0, s>>>(ix->seq_start_d, woff, ns, chunks, ix->bank.pk, ix->bank.nb, sh, t, prev,
                                                   ccnt, nullptr, nullptr, nullptr));
     }
     void *scan_scr2 = arena.alloc(scan_scratch_bytes(chunks));
@@ -249,9 +285,9 @@ static void index_build_shape(const gn_bank *db, int k, int span, uint32_t keep,
     GN_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * nbk, s));
     uint64_t *keys = arena.alloc_n<uint64_t>(P);
     uint64_t *keys_alt = arena.alloc_n<uint64_t>(P);
-    if (W) {
-        GN_LAUNCH("k_bank_windows_keys", W, s,
-                  k_bank_windows<false><<<grid, 256, 0, s>>>(ix->seq_start_d, woff, ns, W, ix->bank.pk, ix->bank.nb, sh, t,
+    if (P) {
+        GN_LAUNCH("k_bank_windows_keys", w_max, s,
+                  k_bank_windows<false><<<grid, 256, 0, s>>>(ix->seq_start_d, woff, ns, chunks, ix->bank.pk, ix->bank.nb, sh, t, prev,
                                                    nullptr, hist, coff, keys));
     }
     exclusive_scan_u32(hist, ix->off_d, nbk, scan_scr, s);
@@ -259,31 +295,23 @@ static void index_build_shape(const gn_bank *db, int k, int span, uint32_t keep,
     // K4: stable scatter = stable radix sort of (code, global offset) keys by code
     void *rs = arena.alloc(radix_scratch_bytes(P));
     bool flipped = radix_sort(keys, keys_alt, nullptr, nullptr, P, 32, 32 + 2 * k, rs, s, TAG_INDEX_SORT);
-    GN_CUDA(cudaMalloc(&ix->post_d, sizeof(uint32_t) * post_alloc_entries(P)));
-    bytes += sizeof(uint32_t) * P;
-    alloc_sigs(ix, bytes);
+    alloc_occurrences(ix);
     if (P) {
         GN_LAUNCH("k_occurrences", P, s,
                   k_occurrences<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(flipped ? keys_alt : keys, P, ix->post_d, ix->sig_d, n,
-                                                                         ix->bank.pk, ix->bank.nb, seq_map(ix), sh, t, sig_kind(k, span, t)));
+                                                                         ix->bank.pk, ix->bank.nb, seq_map(ix), sh, t, kind, prev));
     }
     uint32_t wst = 0;
     GN_CUDA(cudaMemcpyAsync(&wst, wait_status, 4, cudaMemcpyDeviceToHost, s));
     arena.release();
     GN_CUDA(cudaStreamSynchronize(s));
     GN_REQUIRE((wst & DEV_ERR_TIMEOUT) == 0, GN_ETIMEOUT, "a device-side wait ran out (scan look-back)");
-    ix->device_bytes = bytes;
 }
 
 void index_free(gn_index *ix) {
     if (!ix) return;
-    cudaFree(ix->seq_start_d);
-    cudaFree(ix->seq_lut_d);
-    cudaFree(ix->bank.pk);
-    cudaFree(ix->bank.nb);
-    cudaFree(ix->off_d);
+    cudaFree(ix->fixed_d);
     cudaFree(ix->post_d);
-    cudaFree(ix->sig_d);
 }
 
 void index_export(const gn_index *ix, uint64_t *bucket_start, uint32_t *post_seq, uint32_t *post_pos) {
@@ -396,15 +424,9 @@ void index_load(const char *path, gn_index *ix) {
     GN_REQUIRE(ix->seq_start_h[0] == 0 && ix->seq_start_h[ns] == n, GN_EINVAL, "index file: bad sequence starts");
     for (uint64_t i = 0; i < ns; ++i)
         GN_REQUIRE(ix->seq_start_h[i + 1] >= ix->seq_start_h[i], GN_EINVAL, "index file: bad sequence starts");
-    uint64_t bytes = 0;
-    GN_CUDA(cudaMalloc(&ix->seq_start_d, sizeof(uint64_t) * (ns + 1)));
-    GN_CUDA(cudaMalloc(&ix->bank.pk, 4 * npk));
-    GN_CUDA(cudaMalloc(&ix->bank.nb, 4 * nnb));
-    GN_CUDA(cudaMalloc(&ix->off_d, 8 * nbk));
-    GN_CUDA(cudaMalloc(&ix->post_d, 4 * post_alloc_entries(np)));
-    GN_CUDA(cudaMalloc(&ix->seq_lut_d, 4 * nlut));
+    alloc_fixed(ix, ns, n, nbk - 1, nlut);
+    alloc_occurrences(ix);
     ix->bank.n = n;
-    bytes += 8 * (ns + 1) + 4 * (npk + nnb) + 8 * nbk + 4 * np + 4 * nlut;
     GN_CUDA(cudaMemcpy(ix->seq_start_d, ix->seq_start_h.data(), 8 * (ns + 1), cudaMemcpyHostToDevice));
     std::vector<uint8_t> buf(IX_CHUNK);
     read_device(f, ix->bank.pk, 4 * npk, buf);
@@ -417,16 +439,14 @@ void index_load(const char *path, gn_index *ix) {
     GN_REQUIRE(last == np, GN_EINVAL, "index file: bucket starts do not end at the occurrence count");
     // the signatures are not in the file: they follow from the occurrences and the bank (the
     // lookup table, unchecked file content, is not walked here)
-    alloc_sigs(ix, bytes);
     if (np && ix->sig_d) {
         GN_LAUNCH("k_occurrences", np, 0,
                   k_occurrences<<<(unsigned)((np + 255) / 256), 256>>>(nullptr, np, ix->post_d, ix->sig_d, n, ix->bank.pk,
                                                                      ix->bank.nb, SeqMap{ix->seq_start_d, nullptr, ix->n_seqs},
                                                                      seed_shape(ix), ix->t,
-                                                                     sig_kind(ix->k, ix->span, ix->t)));
+                                                                     sig_kind(ix->k, ix->span, ix->t), false));
         GN_CUDA(cudaDeviceSynchronize());
     }
-    ix->device_bytes = bytes;
 }
 
 }  // namespace gn

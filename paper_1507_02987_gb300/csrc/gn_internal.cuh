@@ -374,11 +374,12 @@ struct gn_index {
     uint32_t max_seq_len = 0;
     std::vector<uint64_t> seq_start_h;
     uint64_t *seq_start_d = nullptr;  // n_seqs + 1
+    unsigned char *fixed_d = nullptr; // block that holds seq_start_d, bank.pk, bank.nb, off_d and seq_lut_d
     uint32_t *seq_lut_d = nullptr;    // (n_bases >> SEQ_LUT_SHIFT) + 1 entries, see SeqMap
     gn::Packed bank;                  // packed bank + non-base bitmap
     uint64_t *off_d = nullptr;        // 4^k + 1 bucket starts
     uint32_t *post_d = nullptr;       // occurrences: global base offset of the window (post_alloc_entries)
-    uint32_t *sig_d = nullptr;        // occurrence signatures (SigKind), entry for entry; null without room for them
+    uint32_t *sig_d = nullptr;        // occurrence signatures (SigKind), entry for entry, in post_d's block; null without room for them
     uint64_t device_bytes = 0;
     // per-phase device times of the most recent search through this handle
     std::vector<std::pair<const char *, float>> last_phases;
