@@ -153,12 +153,12 @@ GN_API gn_status gn_index_get_info(const gn_index *index, gn_index_info *info);
 
 /* Execution settings that never change results (0 = the library's default): the
  * fill kernel's tile size in hits (default 50,000) and threads per tile (512 or
- * 256), the raw hits planned per hit bucket (default 4,096 with the repeat
- * filter), the lanes that align one HSP in the alignment kernel's grouped path
- * (8, 16 or 32: four, two or one HSP per warp, for bands of up to 40, 48 or 64
- * diagonals; default 8) and the DP-window rows from which an alignment goes to the
- * anti-diagonal wavefront path (default 512).  They belong to an index (they depend
- * on its occurrence lists). */
+ * 256) and the raw hits planned per hit bucket (default 4,096 with the repeat
+ * filter), which only searches that store their hits use; the lanes that align one
+ * HSP in the alignment kernel's grouped path (8, 16 or 32: four, two or one HSP per
+ * warp, for bands of up to 40, 48 or 64 diagonals; default 8) and the DP-window rows
+ * from which an alignment gets a warp of its own (default 512, or 1,024 in searches of
+ * many alignments).  They belong to an index (they depend on its occurrence lists). */
 typedef struct {
     uint32_t tile_hits;
     uint32_t fill_threads;
@@ -179,7 +179,7 @@ GN_API gn_status gn_index_get_tuning(const gn_index *index, gn_tuning *tuning);
  * chosen params to every later search (and to any reference it compares with).  With GN_TUNE_KERNELS it times
  * the search of the sample with several gn_tuning candidates, one group of settings
  * after the other (fill threads and tile size; raw hits per bucket; lanes per HSP
- * and wavefront rows of the alignment kernel), and installs the fastest on the
+ * and long-alignment rows of the alignment kernel), and installs the fastest on the
  * index (and copies it to *tuning if not NULL).  Not to be run
  * concurrently with other searches on the same index.  Errors as gn_search. */
 #define GN_TUNE_BAND 1u
@@ -216,11 +216,10 @@ GN_API gn_status gn_index_export(const gn_index *index, uint64_t *bucket_start, 
 
 /* Searches every query against the index ("Searching process", seven phases):
  * rolling k-mer codes of every query offset; lookup of each code's
- * occurrences (hits); grouping of the hits by (query, diagonal) in per-query
- * diagonal buckets (a repeat filter first drops hits alone on their diagonal;
- * overflowing buckets go through a radix sort) and merging of hits at most D
- * query offsets apart on one (sequence, diagonal) into HSPs of length >=
- * min_hsp_len; X-drop ungapped extension of both HSP ends; merging of
+ * occurrences (hits) and merging of hits at most D query offsets apart on one
+ * (sequence, diagonal) into HSPs of length >= min_hsp_len (a signature beside each
+ * occurrence tells which hits can have another one ahead; searches that it does not
+ * serve group the stored hits by (query, diagonal) in buckets or by a radix sort); X-drop ungapped extension of both HSP ends; merging of
  * overlapped HSPs; selection of the longest max_alignments HSPs per query;
  * banded affine-gap Smith-Waterman of each selected HSP; ranking by score with
  * e-value and bit score.  Queries are independent: results do not depend on

@@ -2462,7 +2462,7 @@ struct SearchWords {
     uint32_t next_tile, next_cand;
     uint32_t n_wide, next_wide, next_task, n_long, next_long;
     uint32_t n_strip, strip_band, next_strip;
-    uint32_t too_many, pad;
+    uint32_t too_many, recs_done;
     uint32_t groups[8];                // groups of a block, of a large block, of no kernel: of the join, of the merge
     unsigned long long next_end, cells[2];
     uint32_t bins[SWO_BINS], placed[SWO_BINS];
@@ -2602,19 +2602,21 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     uint32_t *src = scan ? nullptr : arena.alloc_n<uint32_t>(HM);
     QueryRec *qrec = scan ? arena.alloc_n<QueryRec>(HM) : nullptr;
     const int flank = (int)std::min<uint32_t>(SIG_FLANK_BASES, p.min_hsp_len > (uint32_t)k ? p.min_hsp_len - (uint32_t)k : 0u);
+    const bool recs_sum = scan && HM && HM <= RECS_SUMS;
     if (scan) {
         auto kernel = kind == SIG_FLANK ? k_query_recs<SIG_FLANK> : k_query_recs<SIG_AHEAD>;
         if (HM)
             GN_LAUNCH("k_query_recs", HM, s,
                       kernel<<<blocks_for(HM), 256, 0, s>>>(hstart_d, hnq, HM, hqp.pk, hqp.nb, seed_shape(ix), ix->t,
                                                             (int)links, flank, ix->off_d, qinfo, qrec, cnt,
-                                                            reinterpret_cast<unsigned long long *>(hq_d)));
+                                                            reinterpret_cast<unsigned long long *>(hq_d),
+                                                            recs_sum ? hoff : nullptr, &words->recs_done));
     } else if (HM) {
         GN_LAUNCH("k_query_codes", HM, s,
                   k_query_codes<<<blocks_for(HM), 256, 0, s>>>(hstart_d, hnq, HM, hqp.pk, hqp.nb, seed_shape(ix), ix->off_d, codes, qinfo,
                                                               cnt, src));
     }
-    {
+    if (!recs_sum) {
         void *scr = arena.alloc(scan_scratch_bytes(HM));
         exclusive_scan_u32(cnt, hoff, HM, scr, s);
     }
@@ -3323,7 +3325,16 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     DevAln *aln = arena.alloc_n<DevAln>(any_sel ? sel_cap : 0);
     const SwScore score{sc.match, sc.mismatch, sc.gap_open + sc.gap_extend, sc.gap_extend, 1};
     const bool cut = sc.mismatch < 2 * sc.gap_extend;
-    uint32_t *strip = nullptr;
+    uint32_t *strip = nullptr, *wide = nullptr;
+    uint64_t wide_area = 0;
+    bool wide_done = true;
+    auto align_wide = [&]() {
+        auto kernel = cut ? k_banded_sw_wide<true> : k_banded_sw_wide<false>;
+        GN_LAUNCH("k_banded_sw_wide", wide_area, s,
+                  kernel<<<std::min<uint32_t>((sel_cap + 3) / 4, (uint32_t)num_sms() * 4), 128, 0, s>>>(
+                      sel, wide, &words->n_wide, &words->next_wide, seqs, qstart_d, ix->seq_start_d, score, (int32_t)p.band_w, strip,
+                      &words->n_strip, &words->strip_band, aln));
+    };
     if (any_sel) {
         const uint32_t sms = (uint32_t)num_sms();
         // lanes per HSP of the grouped path (the index's tuning; GN_SW_LANES overrides)
@@ -3358,19 +3369,19 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
             pin.wait();
             memcpy(area, pin.p, 16);
         }
-        uint32_t *wide = arena.alloc_n<uint32_t>(sel_cap);
+        wide = arena.alloc_n<uint32_t>(sel_cap);
         strip = arena.alloc_n<uint32_t>(sel_cap);
         auto sw_kernel = sw_lanes == 16 ? (cut ? k_banded_sw<16, 2, 1, true> : k_banded_sw<16, 2, 1, false>)
                                         : (cut ? k_banded_sw<8, 3, 2, true> : k_banded_sw<8, 3, 2, false>);
-        auto wide_kernel = cut ? k_banded_sw_wide<true> : k_banded_sw_wide<false>;
         GN_LAUNCH("k_banded_sw", area[0], s,
                   sw_kernel<<<std::min<uint32_t>((sel_cap + 3) / 4, sms * 2), 128, 0, s>>>(
                       sel, n_sel_d, sms, seqs, qstart_d, ix->seq_start_d, score, (int32_t)p.band_w, &words->next_task, order, wide,
                       &words->n_wide, &words->n_long, &words->next_long, aln));
-        GN_LAUNCH("k_banded_sw_wide", area[1], s,
-                  wide_kernel<<<std::min<uint32_t>((sel_cap + 3) / 4, sms * 4), 128, 0, s>>>(
-                      sel, wide, &words->n_wide, &words->next_wide, seqs, qstart_d, ix->seq_start_d, score, (int32_t)p.band_w, strip,
-                      &words->n_strip, &words->strip_band, aln));
+        wide_area = area[1];
+        // Small calls at the default band rarely have an alignment for the wide kernel: they wait for
+        // the count (3 of 200 us for an empty launch).
+        wide_done = ordered || 2 * (int64_t)p.band_w + 1 > 64 || keep || sort_rank;
+        if (wide_done) align_wide();
     }
     // bands that no register path holds, once the host knows of them: they are rare, and the rest of
     // the search does not wait for the question
@@ -3443,6 +3454,11 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
             back.fetch(0, words, sizeof(SearchWords));
             back.wait();
             memcpy(&got, back.p, sizeof(SearchWords));
+            if (!wide_done && got.n_wide) {
+                align_wide();
+                wide_done = true;
+                continue;
+            }
             if (strips_done || !got.n_strip) break;
             align_strips(got);
             strips_done = true;
