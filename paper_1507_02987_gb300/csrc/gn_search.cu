@@ -1855,6 +1855,71 @@ __device__ __forceinline__ void sw_row(SwSet<KA + KB> &x, int32_t &F1, uint32_t 
     SF1 = SF;
 }
 
+// Packed cells: score, choice and start cell in one word, for alignments whose rows and scores fit
+// (exactly; sw_fits).  From the top: the score, signed; 3 bits of choice; ROW bits of row and OFF bits
+// of band offset of the start cell.  The choice orders candidates of one score as the recurrence
+// does (a new start 7, the diagonal 6, E opened 5 or extended 4, F opened 1 or extended 0), so that
+// a plain maximum of words selects score and start at once, three candidates in one instruction,
+// where a tracked maximum takes a compare and two selects; a logic operation then clears the
+// choice.  F opens from H, not from H without F: where F won, opening from it can not beat
+// extending it (gap_open <= 0) and has its start.  20 instructions a cell instead of 27, shuffles
+// of one word instead of two, and shorter chains.  us, tracked | packed: one alignment of 400 rows 56 |
+// 47; 200,000 alignments (2,000 queries) 573 | 460, 50,000 at stride 1 220 | 170, 881 M cells of
+// 257 and more diagonals 1,019 | 830.  Alignments that do not fit keep tracked cells (the longest
+// ones of 1,000 queries of up to 10,000 bases are such: 310 | 291).
+template <int OFF, int ROW>
+struct SwPack {
+    static constexpr int CHOICE = OFF + ROW, SCORE = CHOICE + 3;
+    static constexpr int32_t CLEAN = ~(7 << CHOICE), NEG = -(1 << 30), LOW = (1 << SCORE) - 1;
+    int32_t match, mismatch, e_open, e_ext, f_open, f_ext, one;
+    __device__ __forceinline__ explicit SwPack(const SwScore &c)
+        : match(word(c.match, 6)), mismatch(word(c.mismatch, 6)), e_open(word(c.goe, 5)), e_ext(word(c.ge, 4)),
+          f_open(word(c.goe, 1)), f_ext(word(c.ge, 0)), one(c.one) {}
+    static __device__ __forceinline__ int32_t word(int32_t score, int32_t choice) {
+        return (int32_t)((uint32_t)score << SCORE) + (choice << CHOICE);
+    }
+    // rows of the DP window, at most: their starts fit, their scores do, and gaps and mismatches
+    // taken from NEG stay in range
+    static __device__ __forceinline__ bool fits(int64_t rows, const SwScore &c) {
+        const int32_t low = -(1 << (30 - SCORE));
+        return rows < (1 << ROW) && rows * c.match < (1 << (31 - SCORE)) && c.mismatch > low && c.goe > low && c.ge > low;
+    }
+};
+
+// Cell k of the row, as sw_cell; z: the word of a start on the lane's first offset a row on.
+template <class P, int K, bool CUT>
+__device__ __forceinline__ void sp_cell(SwSet<K> &x, int k, uint32_t eq, int32_t E, int32_t &F, int32_t z, const P &c) {
+    const int32_t D = fma_score(x.H[k], eq & (1u << (30 - 2 * k)), c.match, c.mismatch, c.one);
+    const int32_t h = max(__vimax3_s32(D, E, fma_add(z, k, c.one)), F);
+    // a higher score than the best one, whose word with all lower bits set is bstart
+    asm("{ .reg .pred q; setp.gt.s32 q, %3, %2; @q mul.lo.s32 %0, %3, %6; @q mad.lo.s32 %1, %4, %6, %5; @q or.b32 %2, %3, %7; }"
+        : "+r"(x.best), "+r"(x.bcell), "+r"(x.bstart)
+        : "r"(h), "r"(x.cell), "r"(k), "r"(c.one), "n"(P::LOW));
+    const int32_t H = h & P::CLEAN;
+    x.H[k] = H;
+    x.E[k] = max(fma_add(H, c.e_open, c.one), fma_add(E & P::CLEAN, c.e_ext, c.one));
+    if (CUT && !(x.in_band & (1u << (30 - 2 * k)))) x.E[k] = P::NEG;
+    F = max(fma_add(H, c.f_open, c.one), fma_add(F & P::CLEAN, c.f_ext, c.one));
+}
+
+// sw_row on packed cells; SH[0]: the row to come's first offset of the lane, as a start.
+template <class P, int OFF, int G, int KA, int KB, bool NO, bool CUT>
+__device__ __forceinline__ void sp_row(SwSet<KA + KB> &x, int32_t &F1, int sl, const P &c) {
+    constexpr int K = KA + KB;
+    int32_t F = __shfl_up_sync(0xffffffffu, F1, 1);
+    if (sl == 0) F = P::NEG;
+    const uint32_t eq = sw_next_row<K, NO>(x);
+    x.SH[0] += 1u << OFF;
+    const int32_t z = (int32_t)((x.SH[0] & ((1u << P::CHOICE) - 1u)) | (7u << P::CHOICE));
+#pragma unroll
+    for (int k = 0; k < KA; ++k) sp_cell<P, K, CUT>(x, k, eq, x.E[k + 1], F, z, c);
+    int32_t uE = __shfl_down_sync(0xffffffffu, x.E[0], 1);
+    if (sl == G - 1) uE = P::NEG;
+#pragma unroll
+    for (int k = KA; k < K; ++k) sp_cell<P, K, CUT>(x, k, eq, k + 1 < K ? x.E[k + 1] : uE, F, z, c);
+    F1 = F;
+}
+
 // Highest score, then first cell, over the G lanes of a segment; the alignment it stands for.
 template <int G>
 __device__ __forceinline__ void sw_finish(int32_t best, uint32_t cell, uint32_t start, const DevHsp &h, bool on, int32_t w,
@@ -1912,6 +1977,47 @@ __device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const PackedPa
     sw_finish<G>(x.best, x.bcell, x.bstart, h, on, w, res);
 }
 
+// sw_band on packed cells, for HSPs that fit them
+template <int G, int KA, int KB, int OFF, int ROW, bool CUT>
+__device__ __forceinline__ void sp_band(const DevHsp &h, bool on, const PackedPair &q, const uint64_t *__restrict__ qstart,
+                                        const uint64_t *__restrict__ seq_start, const SwScore &score, int32_t w, DevAln &res) {
+    typedef SwPack<OFF, ROW> P;
+    static_assert(G * (KA + KB) <= 1 << OFF, "an offset fits its bits");
+    const int sl = (threadIdx.x & 31) % G;
+    constexpr int K = KA + KB;
+    const P c(score);
+    SwSet<K> x;
+    int32_t T = 0;
+    {
+        SwGeom g{};
+        if (on) {
+            g.set(h, qstart, seq_start, w);
+            T = (int32_t)max(g.qhi - g.qlo, (int64_t)0) + (g.B - 1) / K;
+        }
+        x.start(g, on, K * sl, sl);
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) { x.H[k] = sl == 0 ? k : 0; x.E[k] = P::NEG; }
+    x.bstart = (uint32_t)P::LOW;
+    x.SH[0] = (uint32_t)(-sl * (1 << OFF) + K * sl);
+    if (G < 32) T = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)T);
+    int32_t F1 = P::NEG;
+    for (int32_t t0 = 0; t0 < T; t0 += 16) {
+        const bool no = __any_sync(0xffffffffu, x.load(q));
+        x.q += 16; x.d += 16;
+        const int32_t t1 = min(t0 + 16, T);
+        if (no) {
+#pragma unroll 1
+            for (int32_t t = t0; t < t1; ++t) sp_row<P, OFF, G, KA, KB, true, CUT>(x, F1, sl, c);
+        } else {
+#pragma unroll 1
+            for (int32_t t = t0; t < t1; ++t) sp_row<P, OFF, G, KA, KB, false, CUT>(x, F1, sl, c);
+        }
+    }
+    const uint32_t start = (uint32_t)x.best & ((1u << P::CHOICE) - 1u);
+    sw_finish<G>(x.best >> P::SCORE, x.bcell, (start >> OFF) << SW_SHIFT | (start & ((1u << OFF) - 1u)), h, on, w, res);
+}
+
 // What the number of alignments, known on the device only, decides: see the alignment kernels'
 // launch in search().
 __device__ __forceinline__ bool sw_many(uint32_t n, uint32_t sms) { return n > sms * 64u; }
@@ -1957,7 +2063,10 @@ __global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ se
         DevHsp h{};
         if (!take(j, nl, 64, lane == 0, task, h)) continue;
         DevAln res;
-        sw_band<32, 1, 1, CUT>(h, true, q, qstart, seq_start, c, w, res);
+        if (SwPack<6, 11>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c))
+            sp_band<32, 1, 1, 6, 11, CUT>(h, true, q, qstart, seq_start, c, w, res);
+        else
+            sw_band<32, 1, 1, CUT>(h, true, q, qstart, seq_start, c, w, res);
         if (lane == 0) out[task] = res;
     }
     constexpr uint32_t NT = 32 / G;
@@ -1971,7 +2080,10 @@ __global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ se
         const bool first = lane % G == 0, on = take(base + seg, n, G * (KA + KB), first, task, h);
         if (!__any_sync(0xffffffffu, on)) continue;
         DevAln res;
-        sw_band<G, KA, KB, CUT>(h, on, q, qstart, seq_start, c, w, res);
+        if (__all_sync(0xffffffffu, !on || SwPack<6, 11>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c)))
+            sp_band<G, KA, KB, 6, 11, CUT>(h, on, q, qstart, seq_start, c, w, res);
+        else
+            sw_band<G, KA, KB, CUT>(h, on, q, qstart, seq_start, c, w, res);
         if (on && first) out[task] = res;
     }
 }
@@ -1999,7 +2111,10 @@ __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict
         const int64_t B = dev_band(h, w);
         if (B <= SW_MAX_BAND && (int64_t)h.qe - h.qs + 2 * (int64_t)w <= SW_MAX_ROWS) {
             DevAln res;
-            sw_band<32, 5, 4, CUT>(h, true, q, qstart, seq_start, c, w, res);
+            if (SwPack<9, 9>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c))
+                sp_band<32, 5, 4, 9, 9, CUT>(h, true, q, qstart, seq_start, c, w, res);
+            else
+                sw_band<32, 5, 4, CUT>(h, true, q, qstart, seq_start, c, w, res);
             if (lane == 0) out[task] = res;
         } else if (lane == 0) {
             strip[atomicAdd(strip_count, 1u)] = task;
