@@ -1865,8 +1865,8 @@ __device__ __forceinline__ void sw_row(SwSet<KA + KB> &x, int32_t &F1, uint32_t 
 // extending it (gap_open <= 0) and has its start.  20 instructions a cell instead of 27, shuffles
 // of one word instead of two, and shorter chains.  us, tracked | packed: one alignment of 400 rows 56 |
 // 47; 200,000 alignments (2,000 queries) 573 | 460, 50,000 at stride 1 220 | 170, 881 M cells of
-// 257 and more diagonals 1,019 | 830.  Alignments that do not fit keep tracked cells (the longest
-// ones of 1,000 queries of up to 10,000 bases are such: 310 | 291).
+// 257 and more diagonals 1,019 | 830.  Longer alignments name starts by a table (sp_band); only
+// scores beyond that keep tracked cells.
 template <int OFF, int ROW>
 struct SwPack {
     static constexpr int CHOICE = OFF + ROW, SCORE = CHOICE + 3;
@@ -1878,11 +1878,11 @@ struct SwPack {
     static __device__ __forceinline__ int32_t word(int32_t score, int32_t choice) {
         return (int32_t)((uint32_t)score << SCORE) + (choice << CHOICE);
     }
-    // rows of the DP window, at most: their starts fit, their scores do, and gaps and mismatches
-    // taken from NEG stay in range
-    static __device__ __forceinline__ bool fits(int64_t rows, const SwScore &c) {
+    // rows of the DP window, at most: their starts fit (in the word or by a table), their scores do,
+    // and gaps and mismatches taken from NEG stay in range
+    static __device__ __forceinline__ bool fits(int64_t rows, const SwScore &c, bool table = false) {
         const int32_t low = -(1 << (30 - SCORE));
-        return rows < (1 << ROW) && rows * c.match < (1 << (31 - SCORE)) && c.mismatch > low && c.goe > low && c.ge > low;
+        return (table || rows < (1 << ROW)) && rows * c.match < (1 << (31 - SCORE)) && c.mismatch > low && c.goe > low && c.ge > low;
     }
 };
 
@@ -1977,11 +1977,19 @@ __device__ __forceinline__ void sw_band(const DevHsp &h, bool on, const PackedPa
     sw_finish<G>(x.best, x.bcell, x.bstart, h, on, w, res);
 }
 
-// sw_band on packed cells, for HSPs that fit them
-template <int G, int KA, int KB, int OFF, int ROW, bool CUT>
+// sw_band on packed cells, for HSPs that fit them.  table (null: none; a word for each of the warp's
+// 2 K + 1 cells a lane): the rows of start cells count from the 16 rows at hand, and a start before
+// them is named by its place in the table, where the starts of all cells that still count are
+// put after every 16 rows; with 5 bits of row and as many places a score of 18 (15) bits fits.  A
+// tenth more instructions than without the table.  us, tracked | table, where the longest alignments
+// have over 2,047 rows: 1,000 queries of up to 10,000 bases 291 | 265, 8 long queries 268 | 237.
+template <int G, int KA, int KB, int OFF, int ROW, bool TABLE, bool CUT>
 __device__ __forceinline__ void sp_band(const DevHsp &h, bool on, const PackedPair &q, const uint64_t *__restrict__ qstart,
-                                        const uint64_t *__restrict__ seq_start, const SwScore &score, int32_t w, DevAln &res) {
+                                        const uint64_t *__restrict__ seq_start, const SwScore &score, int32_t w,
+                                        uint32_t *table, DevAln &res) {
     typedef SwPack<OFF, ROW> P;
+    constexpr uint32_t CODE = (1u << P::CHOICE) - 1u, PLACES = TABLE ? 32 * (2 * (KA + KB) + 1) : 0;
+    static_assert(!TABLE || PLACES + (17u << OFF) <= CODE + 1, "places and 17 rows of starts fit");
     static_assert(G * (KA + KB) <= 1 << OFF, "an offset fits its bits");
     const int sl = (threadIdx.x & 31) % G;
     constexpr int K = KA + KB;
@@ -1997,12 +2005,14 @@ __device__ __forceinline__ void sp_band(const DevHsp &h, bool on, const PackedPa
         x.start(g, on, K * sl, sl);
     }
 #pragma unroll
-    for (int k = 0; k < K; ++k) { x.H[k] = sl == 0 ? k : 0; x.E[k] = P::NEG; }
+    for (int k = 0; k < K; ++k) { x.H[k] = sl == 0 ? (int32_t)PLACES + k : 0; x.E[k] = P::NEG; }
     x.bstart = (uint32_t)P::LOW;
     x.SH[0] = (uint32_t)(-sl * (1 << OFF) + K * sl);
     if (G < 32) T = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)T);
-    int32_t F1 = P::NEG;
+    int32_t F1 = P::NEG, best = 0;  // best: the word whose start is best_start
+    uint32_t best_start = 0;
     for (int32_t t0 = 0; t0 < T; t0 += 16) {
+        if (TABLE) x.SH[0] = PLACES + (uint32_t)(K * sl);
         const bool no = __any_sync(0xffffffffu, x.load(q));
         x.q += 16; x.d += 16;
         const int32_t t1 = min(t0 + 16, T);
@@ -2013,9 +2023,35 @@ __device__ __forceinline__ void sp_band(const DevHsp &h, bool on, const PackedPa
 #pragma unroll 1
             for (int32_t t = t0; t < t1; ++t) sp_row<P, OFF, G, KA, KB, false, CUT>(x, F1, sl, c);
         }
+        if constexpr (TABLE) {
+            auto cell_of = [&](int32_t word) {
+                const uint32_t code = (uint32_t)word & CODE, n = code - PLACES;  // n: from PLACES on
+                const uint32_t off = n & ((1u << OFF) - 1u), row = (uint32_t)t0 + (n >> OFF) - off / (uint32_t)K;
+                return code < PLACES ? table[code] : row << SW_SHIFT | off;
+            };
+            uint32_t cell[2 * K + 1];
+#pragma unroll
+            for (int k = 0; k < K; ++k) { cell[2 * k] = cell_of(x.H[k]); cell[2 * k + 1] = cell_of(x.E[k]); }
+            cell[2 * K] = cell_of(F1);
+            if (x.best != best) { best = x.best; best_start = cell_of(best); }
+            __syncwarp();
+            const uint32_t place = (uint32_t)(threadIdx.x & 31) * (2 * K + 1);
+#pragma unroll
+            for (int i = 0; i < 2 * K + 1; ++i) table[place + i] = cell[i];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                x.H[k] = (x.H[k] & ~(int32_t)CODE) | (int32_t)(place + 2 * k);
+                x.E[k] = (x.E[k] & ~(int32_t)CODE) | (int32_t)(place + 2 * k + 1);
+            }
+            F1 = (F1 & ~(int32_t)CODE) | (int32_t)(place + 2 * K);
+            __syncwarp();
+        }
     }
-    const uint32_t start = (uint32_t)x.best & ((1u << P::CHOICE) - 1u);
-    sw_finish<G>(x.best >> P::SCORE, x.bcell, (start >> OFF) << SW_SHIFT | (start & ((1u << OFF) - 1u)), h, on, w, res);
+    if (!TABLE) {
+        const uint32_t start = (uint32_t)x.best & CODE;
+        best_start = (start >> OFF) << SW_SHIFT | (start & ((1u << OFF) - 1u));
+    }
+    sw_finish<G>(x.best >> P::SCORE, x.bcell, best_start, h, on, w, res);
 }
 
 // What the number of alignments, known on the device only, decides: see the alignment kernels'
@@ -2040,6 +2076,7 @@ __global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ se
                                                    uint32_t *__restrict__ wide, uint32_t *__restrict__ wide_count,
                                                    const uint32_t *__restrict__ n_long, uint32_t *__restrict__ next_long,
                                                    DevAln *__restrict__ out) {
+    __shared__ uint32_t table[4][32 * 5];
     const int lane = threadIdx.x & 31, seg = lane / G;
     const uint32_t n = (uint32_t)*n_dev, nl = order ? *n_long : n;  // no order: a warp each
     if (!sw_many(n, sms) && blockIdx.x >= sms) return;  // four warps an SM (see the launch)
@@ -2064,7 +2101,9 @@ __global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ se
         if (!take(j, nl, 64, lane == 0, task, h)) continue;
         DevAln res;
         if (SwPack<6, 11>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c))
-            sp_band<32, 1, 1, 6, 11, CUT>(h, true, q, qstart, seq_start, c, w, res);
+            sp_band<32, 1, 1, 6, 11, false, CUT>(h, true, q, qstart, seq_start, c, w, nullptr, res);
+        else if (SwPack<6, 5>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c, true))
+            sp_band<32, 1, 1, 6, 5, true, CUT>(h, true, q, qstart, seq_start, c, w, table[threadIdx.x >> 5], res);
         else
             sw_band<32, 1, 1, CUT>(h, true, q, qstart, seq_start, c, w, res);
         if (lane == 0) out[task] = res;
@@ -2081,7 +2120,7 @@ __global__ void __launch_bounds__(128) k_banded_sw(const DevHsp *__restrict__ se
         if (!__any_sync(0xffffffffu, on)) continue;
         DevAln res;
         if (__all_sync(0xffffffffu, !on || SwPack<6, 11>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c)))
-            sp_band<G, KA, KB, 6, 11, CUT>(h, on, q, qstart, seq_start, c, w, res);
+            sp_band<G, KA, KB, 6, 11, false, CUT>(h, on, q, qstart, seq_start, c, w, nullptr, res);
         else
             sw_band<G, KA, KB, CUT>(h, on, q, qstart, seq_start, c, w, res);
         if (on && first) out[task] = res;
@@ -2099,6 +2138,7 @@ __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict
                                                         const uint64_t *__restrict__ seq_start, SwScore c, int32_t w,
                                                         uint32_t *__restrict__ strip, uint32_t *__restrict__ strip_count,
                                                         uint32_t *__restrict__ strip_band, DevAln *__restrict__ out) {
+    __shared__ uint32_t table[4][32 * 19];
     const int lane = threadIdx.x & 31;
     const uint32_t n = *wide_count;
     for (;;) {
@@ -2112,7 +2152,9 @@ __global__ void __launch_bounds__(128) k_banded_sw_wide(const DevHsp *__restrict
         if (B <= SW_MAX_BAND && (int64_t)h.qe - h.qs + 2 * (int64_t)w <= SW_MAX_ROWS) {
             DevAln res;
             if (SwPack<9, 9>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c))
-                sp_band<32, 5, 4, 9, 9, CUT>(h, true, q, qstart, seq_start, c, w, res);
+                sp_band<32, 5, 4, 9, 9, false, CUT>(h, true, q, qstart, seq_start, c, w, nullptr, res);
+            else if (SwPack<9, 5>::fits((int64_t)h.qe - h.qs + 2 * (int64_t)w, c, true))
+                sp_band<32, 5, 4, 9, 5, true, CUT>(h, true, q, qstart, seq_start, c, w, table[threadIdx.x >> 5], res);
             else
                 sw_band<32, 5, 4, CUT>(h, true, q, qstart, seq_start, c, w, res);
             if (lane == 0) out[task] = res;
