@@ -2858,7 +2858,8 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     };
     if (scan && HM) {
         auto kernel = kind == SIG_FLANK ? k_seed_scan<SIG_FLANK> : k_seed_scan<SIG_AHEAD>;
-        auto chain = kind == SIG_FLANK ? k_chain<SIG_FLANK> : k_chain<SIG_AHEAD>;
+        const bool edges = !(ix->keep & 1u) || !(ix->keep >> (ix->span - 1));
+        auto chain = kind == SIG_FLANK ? k_chain<SIG_FLANK, false> : edges ? k_chain<SIG_AHEAD, true> : k_chain<SIG_AHEAD, false>;
         const int occ = blocks_per_sm(reinterpret_cast<const void *>(kernel), SCAN_THREADS);
         const int cocc = blocks_per_sm(reinterpret_cast<const void *>(chain), SCAN_THREADS);
         // resident blocks; fewer when the units (four hits each, at least one an offset) do not fill them
