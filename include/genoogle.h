@@ -21,7 +21,8 @@
  *    everything in extension and alignment.
  *  - Limits: bank < 2^32 bases in total; query length < 2^24 bases for gn_search
  *    (over 65,535 in overlapping segments) and < 65,536 for the request loop; at
- *    most 65,536 queries (or query segments) per gn_search call; k in 1..16;
+ *    most 65,536 queries (or query segments) per gn_search call; < 2^32 seed hits
+ *    per query (or segment) and < 2^32 HSPs per call (GN_ETOOBIG); k in 1..16;
  *    stride >= 1.
  */
 #ifndef GENOOGLE_H

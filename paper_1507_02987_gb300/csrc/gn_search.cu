@@ -2543,7 +2543,7 @@ unsigned blocks_for(uint64_t n, unsigned t = 256) { return (unsigned)std::max<ui
 // buckets have.
 bool hit_path_forced() {
     for (const char *v : {"GN_HIT_GROUPING", "GN_TILE_FILTER", "GN_TILE_POS", "GN_TILE_FBITS", "GN_TILE_FBITS2",
-                          "GN_FILL_THREADS", "GN_BUCKET_TARGET", "GN_BUCKET_CAP", "GN_SPILL_ROOM", "GN_MAX_CHUNK_HITS"})
+                          "GN_FILL_THREADS", "GN_BUCKET_TARGET", "GN_BUCKET_CAP", "GN_SPILL_ROOM"})
         if (getenv(v)) return true;
     return false;
 }
@@ -2621,6 +2621,7 @@ struct SearchWords {
     uint32_t n_strip, strip_band, next_strip;
     uint32_t too_many, recs_done;
     uint32_t groups[8];                // groups of a block, of a large block, of no kernel: of the join, of the merge
+    unsigned long long n_units;        // list units of all offsets
     unsigned long long next_end, cells[2];
     uint32_t bins[SWO_BINS], placed[SWO_BINS];
 };
@@ -2805,19 +2806,25 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     timer.mark("query_codes");
 
     // a6-a8 per chunk of queries whose hits fit the budget
-    uint64_t hit_budget = 0;
-    if (!scan) {
+    uint64_t hit_budget = 0, scan_range = SCAN_RANGE;
+    auto free_bytes = []() {
         size_t free_b = 0, total_b = 0;
         GN_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        return free_b;
+    };
+    if (!scan) {
         // bytes per hit of a chunk: hit keys and their ping-pong buffer on the sort path, or the
         // fixed-capacity buckets (up to ~22 B per hit without the repeat filter) and spill lists
-        uint64_t mem_for_hits = (uint64_t)(free_b * 0.55);
+        uint64_t mem_for_hits = (uint64_t)(free_bytes() * 0.55);
         if (o.mem_cap) mem_for_hits = std::min(mem_for_hits, o.mem_cap);
         // (a query chunk holds < 2^32 hits: the fill kernel indexes a tile's hits in 32 bits)
         hit_budget = std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1ull << 20, mem_for_hits / HIT_BYTES));
-        if (const char *e = getenv("GN_MAX_CHUNK_HITS")) {  // smaller chunks (exercises the multi-chunk path)
-            uint64_t v = strtoull(e, nullptr, 10);
-            if (v) hit_budget = std::min<uint64_t>(v, 0xFFFFFFFFull);
+    }
+    if (const char *e = getenv("GN_MAX_CHUNK_HITS")) {  // smaller chunks, or ranges of the scan (exercises several of them)
+        uint64_t v = strtoull(e, nullptr, 10);
+        if (v) {
+            hit_budget = std::min<uint64_t>(v, 0xFFFFFFFFull);
+            scan_range = std::min(std::max<uint64_t>(v / 4, 1), SCAN_RANGE);
         }
     }
     const uint64_t gbits_max = (uint64_t)bits_for(ix->n_bases + QBIAS);
@@ -2825,7 +2832,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
 
     // The scan route sizes its lists from the hits that the list lengths' mean promises (repeats
     // and skewed bases bring more): lists that turn out short are enlarged and their kernel rerun.
-    const uint64_t hits_guess = scan ? (uint64_t)((double)HM * (double)ix->n_postings / std::pow(4.0, ix->k)) : hq[hnq];
+    const uint64_t hits_guess = scan ? (uint64_t)std::min((double)HM * (double)ix->n_postings / std::pow(4.0, ix->k), 4.0 * SCAN_RANGE) : hq[hnq];
     uint32_t hsp_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 14, hits_guess / 64));
     DevHsp *hsp = arena.alloc_n<DevHsp>(hsp_cap);
     uint32_t n_hsp = 0;
@@ -2866,47 +2873,77 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         const uint64_t tiles = (hits_guess / 4 + 2 * HM) / 64 + 1;
         const unsigned grid = (unsigned)std::max<uint64_t>(
             1, std::min<uint64_t>((tiles + SCAN_THREADS / 32 - 1) / (SCAN_THREADS / 32), (uint64_t)num_sms() * occ));
-        // room for candidates: about 1 % of the hits at stride 11
-        uint64_t cand_cap = std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 14, hits_guess / 24));
+        // The scan takes all units in one launch, or ranges of them, each scanned, checked and its HSPs
+        // appended before the next: SCAN_RANGE units at a time, or as many as leave a list of
+        // candidates that memory has room for (55 % of what is free, and no more than the caller grants).
+        // Room for candidates to begin with: about 1 % of the hits at stride 11 are.
+        DeviceArena lists(s);  // enlarged candidate lists
+        auto list_room = [&](uint64_t bytes) {  // candidates that `bytes` hold, within what the caller grants
+            if (o.mem_cap) bytes = std::min(bytes, o.mem_cap);
+            uint64_t room = std::max<uint64_t>(1u << 20, bytes / sizeof(uint2));
+            if (const char *e = getenv("GN_CAND_ROOM")) room = std::max<uint64_t>(4, strtoull(e, nullptr, 10));  // (a unit's)
+            return std::min(room, 4 * SCAN_RANGE);
+        };
+        uint64_t cand_cap = std::min(std::max<uint64_t>(1u << 14, hits_guess / 24), list_room(~0ull));
         uint2 *cand = arena.alloc_n<uint2>(cand_cap);
-        const uint64_t units = g_ktimer ? hq[hnq] : 0;
-        bool scanned = false;
-        for (int attempt = 0;; ++attempt) {
-            if (attempt) {  // n_hsp and next_cand, and the scan's own counters if it runs again
+        uint64_t units = g_ktimer ? hq[hnq] : 0;
+        const uint64_t max_range = scan_range;
+        bool scanned = false;  // the range's candidates are listed
+        int attempt = 0;       // of the range
+        for (uint64_t done = 0, all = 1; done < all; ++attempt) {
+            if (done || attempt) {  // n_hsp and next_cand, and the scan's own counters if it runs again
                 GN_CUDA(cudaMemsetAsync(&words->n_hsp, 0, 4, s));
                 GN_CUDA(cudaMemsetAsync(&words->next_cand, 0, 4, s));
                 if (!scanned) GN_CUDA(cudaMemsetAsync(&words->n_cand, 0, 8, s));
             }
             if (!scanned)
                 GN_LAUNCH("k_seed_scan", units, s,
-                          kernel<<<grid, SCAN_THREADS, 0, s>>>(qrec, hoff, HM, reinterpret_cast<const uint4 *>(ix->sig_d),
+                          kernel<<<grid, SCAN_THREADS, 0, s>>>(qrec, hoff, HM, done, done + scan_range, &words->n_units,
+                                                               reinterpret_cast<const uint4 *>(ix->sig_d),
                                                                post_alloc_entries(ix->n_postings) / 4, flank, cand,
                                                                &words->n_cand, (uint32_t)cand_cap, &words->next_tile));
             const ScanCtx c{qinfo, hstart_d, ix->post_d, ix->bank.pk, ix->bank.nb, hqp.pk, hqp.nb, seed_shape(ix),
-                            ix->t, (int)links, flank, hit_min_len, seq_map(ix), hsp, counter, hsp_cap, status,
+                            ix->t, (int)links, flank, hit_min_len, seq_map(ix), hsp + n_hsp, counter, hsp_cap - n_hsp, status,
                             ix->n_postings, ix->n_bases, HM};
             GN_LAUNCH("k_chain", units, s,
                       chain<<<(unsigned)std::min<uint64_t>((cand_cap + SCAN_THREADS - 1) / SCAN_THREADS, (uint64_t)num_sms() * cocc),
                               SCAN_THREADS, 0, s>>>(c, cand, &words->n_cand, (uint32_t)cand_cap, &words->next_cand));
+            units = 0;  // of the first launch
             pin.fetch(0, words, words_bytes);
             pin.wait();
             const SearchWords *got = reinterpret_cast<const SearchWords *>(pin.p);
             if (hq.empty()) read_hits(reinterpret_cast<const uint64_t *>(pin.p + sizeof(SearchWords)));
-            const uint32_t n_cand = got->n_cand, n_new = got->n_hsp;
-            if (n_cand <= cand_cap && n_new <= hsp_cap) {
-                n_hsp = n_new;
-                break;
-            }
-            GN_REQUIRE(attempt < 3, GN_EINTERNAL, "candidate and HSP list sizing did not converge");
-            GN_REQUIRE(n_new < 0xFFFFFFFFu, GN_ETOOBIG, "more than 2^32 HSPs in one call");
+            all = got->n_units;
+            const uint64_t n_cand = got->n_cand, n_new = got->n_hsp;
+            const uint64_t here = std::min(scan_range, all - done);
             scanned = n_cand <= cand_cap;
-            if (!scanned) {
-                cand_cap = n_cand;
-                cand = arena.alloc_n<uint2>(cand_cap);
+            if (scanned && n_hsp + n_new <= hsp_cap) {
+                n_hsp += (uint32_t)n_new;
+                done += here;
+                if (n_cand < cand_cap / 4) scan_range = std::min(2 * scan_range, max_range);
+                scanned = false;
+                attempt = -1;
+                continue;
             }
-            if (n_new > hsp_cap) {
-                hsp_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull, (uint64_t)n_new + n_new / 4);
-                hsp = arena.alloc_n<DevHsp>(hsp_cap);
+            GN_REQUIRE(attempt < 64, GN_EINTERNAL, "candidate and HSP list sizing did not converge");
+            if (!scanned) {
+                const uint64_t want = done + here < all ? n_cand + n_cand / 4 : n_cand,
+                               room = list_room((uint64_t)(0.55 * free_bytes()));
+                if (n_cand > room) {  // fewer units, as their candidates go; a quarter of the list's length always fits it
+                    cand_cap = std::max(cand_cap, room);
+                    scan_range = std::max<uint64_t>({1, cand_cap / 4, (uint64_t)(0.75 * (double)here * (double)cand_cap / (double)n_cand)});
+                } else {
+                    cand_cap = std::min(want, room);
+                }
+                lists.release();
+                cand = lists.alloc_n<uint2>(cand_cap);
+            } else {
+                const uint64_t need = n_hsp + n_new;
+                GN_REQUIRE(need < (1ull << 32), GN_ETOOBIG, "more than 2^32 HSPs in one call");
+                hsp_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull, need + need / 4);
+                DevHsp *nh = arena.alloc_n<DevHsp>(hsp_cap);
+                if (n_hsp) GN_CUDA(cudaMemcpyAsync(nh, hsp, sizeof(DevHsp) * n_hsp, cudaMemcpyDeviceToDevice, s));
+                hsp = nh;
             }
             GN_CUDA(cudaMemsetAsync(status, 0, 4, s));
         }

@@ -405,10 +405,16 @@ __device__ __forceinline__ void scan_check_flank(const ScanCtx &c, bool valid, u
 constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_STEPS = 4;
 constexpr int SCAN_QUEUE = 64;
+// Units of one launch, at most: candidates and HSPs are counted in 32 bits (in low-complexity
+// sequence every hit is a candidate), and up to 2^31 of them are.
+constexpr uint64_t SCAN_RANGE = 1ull << 29;
 
+// A launch takes the units [u_from, u_to); n_all: where it leaves the number of all units.
 template <int KIND>
 __global__ void __launch_bounds__(SCAN_THREADS, 4) k_seed_scan(const QueryRec *__restrict__ rec,
                                                                const uint64_t *__restrict__ uoff, uint64_t M,
+                                                               uint64_t u_from, uint64_t u_to,
+                                                               unsigned long long *__restrict__ n_all,
                                                                const uint4 *__restrict__ sig4, uint64_t n_units,
                                                                int flank, uint2 *__restrict__ cand,
                                                                uint32_t *__restrict__ cand_count, uint32_t cand_cap,
@@ -418,10 +424,11 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_seed_scan(const QueryRec *_
     const uint32_t lt = (1u << lane) - 1u, le = lt | (1u << lane);
     uint2 *queue = queue_s[wib];
     uint32_t nqueue = 0;
-    const uint64_t total = uoff[M];
+    const uint64_t all = uoff[M], total = min(all, u_to);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_all = all;
     const uint64_t warps = (uint64_t)gridDim.x * (SCAN_THREADS / 32);
     // tiles: eight or more a warp where there is work for that, 64 to 1,024 units
-    const uint64_t R = min((uint64_t)1024, max((uint64_t)64, (uint64_t)((total / (warps * 8) + 31) & ~31ull)));
+    const uint64_t R = min((uint64_t)1024, max((uint64_t)64, (uint64_t)(((total - u_from) / (warps * 8) + 31) & ~31ull)));
     const uint32_t next_mask = KIND == SIG_FLANK ? sig_flank_mask(flank) : 0u;
     auto flush = [&](uint32_t n) {  // the first n (<= 32) queued candidates
         uint32_t at = 0;
@@ -440,7 +447,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_seed_scan(const QueryRec *_
         uint32_t tile = 0;
         if (lane == 0) tile = atomicAdd(next_tile, 1u);
         tile = __shfl_sync(0xffffffffu, tile, 0);
-        const uint64_t u0 = (uint64_t)tile * R;
+        const uint64_t u0 = u_from + (uint64_t)tile * R;
         if (u0 >= total) break;
         const int64_t tile_end = (int64_t)min(R, total - u0);
         // last offset whose units start at or before u0: 32 probes a round
