@@ -2627,6 +2627,9 @@ struct SearchWords {
 };
 static_assert(sizeof(SearchWords) % 8 == 0, "SearchWords is followed by 64-bit words");
 
+// Alignments that a search makes room for without asking how many there are (180 MB).
+constexpr uint32_t SEL_ASK = 1u << 20;
+
 // Segments of a query set: one per MAX_QUERY_LEN bases or part, SEG_STEP apart (see search).
 uint64_t count_segments(const std::vector<uint64_t> &qstart) {
     uint64_t n = 0;
@@ -3426,9 +3429,9 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     uint64_t *qo = arena.alloc_n<uint64_t>(nq + 1);  // selected HSPs of the queries before each
     uint32_t n_mg = 0;                               // read only where it is needed
     // a11's room: longest first, at most max_alignments per query (all of them: the boxes as they are)
-    const uint32_t sel_cap = (uint32_t)std::min<uint64_t>(n_hsp, N ? (uint64_t)nq * N : ~0ull);
-    DevHsp *sel = n_hsp && !sort_select && N ? arena.alloc_n<DevHsp>(sel_cap) : merged;
-    const bool block_selects = merge_block && sel != merged;
+    uint32_t sel_cap = (uint32_t)std::min<uint64_t>(n_hsp, N ? (uint64_t)nq * N : ~0ull);
+    const bool block_selects = merge_block && n_hsp && !sort_select && N;
+    DevHsp *sel = block_selects ? arena.alloc_n<DevHsp>(sel_cap) : merged;
     if (n_hsp) {
         DevHsp *boxes = arena.alloc_n<DevHsp>(n_hsp);
         if (merge_groups) {
@@ -3483,7 +3486,12 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     // a11: selection
     uint32_t n_sel = 0;                      // read only where it is needed
     const uint64_t *n_sel_d = qo + nq;       // the same on the device
+    // The buffers from here on take about 170 bytes an alignment: where they would take more than
+    // SEL_ASK of them, many more perhaps than there are boxes, the host waits for the number
+    // (20 us of a search that takes milliseconds).
+    if (n_hsp && !sort_select && sel_cap > SEL_ASK) sel_cap = read_count(n_sel_d);
     if (n_hsp && !sort_select && N && !block_selects) {
+        sel = arena.alloc_n<DevHsp>(sel_cap);
         GN_LAUNCH("k_select_query", n_hsp, s,
                   k_select_query<<<nq, SQ_THREADS, 0, s>>>(merged, qfirst, qo, N, max_qlen > 65535 ? 3 : 2, sel));
     } else if (n_mg && sort_select) {
@@ -3508,7 +3516,10 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         n_sel_d = n_sel_own;
     }
     timer.mark("select");
-    if (n_hsp && (keep || sort_rank)) n_sel = (n_mg || !sort_select) ? read_count(n_sel_d) : 0;
+    if (n_hsp && (keep || sort_rank)) {
+        n_sel = (n_mg || !sort_select) ? read_count(n_sel_d) : 0;
+        sel_cap = n_sel;
+    }
     if (keep) {
         std::vector<DevHsp> v = to_host(sel, n_sel, s);
         res->st_sel.resize(n_sel);
