@@ -137,7 +137,11 @@ GN_API gn_status gn_default_params(gn_scoring *scoring, gn_params *params);
  * cross sequences), a histogram over the 4^k buckets, an exclusive scan of it
  * and a stable scatter that keeps each bucket's occurrences in ascending
  * (sequence, position) order.  The packed bank and the index stay resident in
- * device memory until gn_index_free.  k in 1..16, stride >= 1.
+ * device memory until gn_index_free.  Beside each occurrence the index keeps a
+ * 4-byte signature that speeds the seed lookup up, as long as an eighth of the
+ * device's memory stays free with them (or as many bytes as the environment
+ * variable GN_SIGNATURE_RESERVE names); without them searches give the same
+ * results, more slowly.  The same holds for gn_index_load.  k in 1..16, stride >= 1.
  * Errors: GN_EINVAL (bad k/stride/bank), GN_ETOOBIG (bank >= 2^32 bases),
  * GN_ENOMEM, GN_ECUDA. */
 GN_API gn_status gn_index_build(const gn_bank *db, int k, int stride, void *cuda_stream, gn_index **out);

@@ -54,3 +54,23 @@ def test_all_alignments_of_many_hsps_that_merge(gn):  # noqa: F811
         assert_ranked_equal(res.query(i), ref[i].ranked, f"query {i}")
     assert used[0] <= used[1] + 200 * boxes + (16 << 20), (used, boxes)
     ix.close()
+
+
+def test_signatures_leave_memory_free(gn, monkeypatch, tmp_path):  # noqa: F811
+    """An index whose signatures would not leave the reserve free does without them, built or
+    loaded: 4 bytes an occurrence less, the same hits."""
+    bank = synth.make_bank("mid", n_seqs=2000)
+    qs = synth.make_queries("mid", bank, n=20)
+    ix = gn.Index.from_bank(bank)
+    path = str(tmp_path / "ix.gnx")
+    ix.save(path)
+    info, want = ix.info(), gn.search(ix, qs.start, qs.bases).all()
+    ix.close()
+    for reserve, saved in ((1 << 50, 4 * info.n_postings), (0, 0)):
+        monkeypatch.setenv("GN_SIGNATURE_RESERVE", str(reserve))
+        for make in (lambda: gn.Index.from_bank(bank), lambda: gn.Index.load(path)):
+            ix = make()
+            assert ix.info().device_bytes == info.device_bytes - saved
+            got = gn.search(ix, qs.start, qs.bases).all()
+            assert all(np.array_equal(a, b) for a, b in zip(got, want))
+            ix.close()
