@@ -3432,7 +3432,8 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
     uint32_t sel_cap = (uint32_t)std::min<uint64_t>(n_hsp, N ? (uint64_t)nq * N : ~0ull);
     const bool block_selects = merge_block && n_hsp && !sort_select && N;
     DevHsp *sel = block_selects ? arena.alloc_n<DevHsp>(sel_cap) : merged;
-    if (n_hsp) {
+    // in_order: boxes of one query start in the order by which equally long ones are selected
+    auto merge_boxes = [&](int in_order) {
         DevHsp *boxes = arena.alloc_n<DevHsp>(n_hsp);
         if (merge_groups) {
             if (joined_groups) asked.answer(gr.words);  // no larger than they were
@@ -3440,7 +3441,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         }
         if (merge_block) {
             GN_LAUNCH("k_merge_block", n_hsp, s,
-                      k_merge_block<<<1, MB_THREADS, 0, s>>>(hsp, n_hsp, (uint32_t)seqb, (uint32_t)qposb, nq, N, keep ? 0 : 1,
+                      k_merge_block<<<1, MB_THREADS, 0, s>>>(hsp, n_hsp, (uint32_t)seqb, (uint32_t)qposb, nq, N, in_order,
                                                              boxes, merged, qfirst, qo, n_mg_d, block_selects ? sel : nullptr));
         } else if (merge_groups) {
             uint32_t *n_boxes = arena.alloc_n<uint32_t>(gr.G), *cnt_sel = arena.alloc_n<uint32_t>(nq);
@@ -3462,7 +3463,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
                            reinterpret_cast<uint32_t *>(srt), s);
             uint32_t *flag = arena.alloc_n<uint32_t>(n_hsp);
             GN_LAUNCH("k_overlap_sweep", n_hsp, s,
-                      k_overlap_sweep<<<blocks_for(n_hsp), 256, 0, s>>>(srt, n_hsp, boxes, flag, keep ? 0 : 1));
+                      k_overlap_sweep<<<blocks_for(n_hsp), 256, 0, s>>>(srt, n_hsp, boxes, flag, in_order));
             const uint64_t *count = compact_records_async(reinterpret_cast<const uint32_t *>(boxes), HSP_WORDS, flag, n_hsp,
                                                           reinterpret_cast<uint32_t *>(merged), arena, s);
             GN_CUDA(cudaMemcpyAsync(n_mg_d, count, 8, cudaMemcpyDeviceToDevice, s));
@@ -3474,14 +3475,17 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
                 exclusive_scan_u32(cnt_sel, qo, nq, scr, s);
             }
         }
-    }
-    timer.mark("overlap_merge");
-    if (n_hsp && (keep || sort_select)) n_mg = read_count(n_mg_d);
-    if (keep) {
+    };
+    if (n_hsp && keep) {  // the stage's boxes are in the sweep's order
+        merge_boxes(0);
+        n_mg = read_count(n_mg_d);
         std::vector<DevHsp> v = to_host(merged, n_mg, s);
         res->st_merged.resize(n_mg);
         if (n_mg) memcpy(res->st_merged.data(), v.data(), sizeof(DevHsp) * n_mg);
     }
+    if (n_hsp) merge_boxes(1);
+    timer.mark("overlap_merge");
+    if (n_hsp && sort_select && !keep) n_mg = read_count(n_mg_d);
 
     // a11: selection
     uint32_t n_sel = 0;                      // read only where it is needed
