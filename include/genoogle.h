@@ -183,9 +183,11 @@ GN_API gn_status gn_index_get_tuning(const gn_index *index, gn_tuning *tuning);
  * cost that grows with the band.  w changes results, so the caller passes the
  * chosen params to every later search (and to any reference it compares with).  With GN_TUNE_KERNELS it times
  * the search of the sample with several gn_tuning candidates, one group of settings
- * after the other (fill threads and tile size; raw hits per bucket; lanes per HSP
- * and long-alignment rows of the alignment kernel), and installs the fastest on the
- * index (and copies it to *tuning if not NULL).  Not to be run
+ * after the other (for searches that store their hits, fill threads and tile size and
+ * raw hits per bucket; lanes per HSP and long-alignment rows of the alignment kernel),
+ * and installs the fastest on the index (and copies it to *tuning if not NULL).  Rows
+ * that depend on the number of alignments, the default, stay unless fixed ones are
+ * faster; they are reported as 512, and gn_index_set_tuning fixes them.  Not to be run
  * concurrently with other searches on the same index.  Errors as gn_search. */
 #define GN_TUNE_BAND 1u
 #define GN_TUNE_KERNELS 2u

@@ -366,6 +366,7 @@ struct gn_index {
     int k = 0, t = 0;
     int span = 0;        // bases a seed covers (k without a mask)
     gn_tuning tuning{};  // result-invariant execution settings (0 = defaults)
+    bool rows_by_count = false;  // the autotuner kept the default rule for tuning.sw_wave_rows
     uint32_t keep = 0;   // kept positions of a seed (all k bits without a mask)
     int device = 0;
     uint32_t n_seqs = 0;
@@ -429,6 +430,8 @@ struct SearchOptions {
 // Query i -> queries 2i (as given) and 2i + 1 (reverse complement) in device memory from arena.
 void both_strands(const uint8_t *qbases_dev, const std::vector<uint64_t> &qstart_h, DeviceArena &arena,
                   cudaStream_t s, const uint8_t **out_bases, std::vector<uint64_t> &out_start);
+// Whether a search with these (resolved) parameters chains its hits from signatures.
+bool takes_scan(const gn_index *ix, const gn_params &p);
 // Device-resident query set: bases (ASCII) on the device, starts on the host.
 void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t> &qstart, const SearchOptions &o,
             cudaStream_t s, gn_results *res);

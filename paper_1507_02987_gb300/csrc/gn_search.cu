@@ -2630,6 +2630,21 @@ static_assert(sizeof(SearchWords) % 8 == 0, "SearchWords is followed by 64-bit w
 // Alignments that a search makes room for without asking how many there are (180 MB).
 constexpr uint32_t SEL_ASK = 1u << 20;
 
+// Seed lookup and chaining take one of two routes to the same HSPs.  The signature scan
+// (gn_seed_scan.cuh) reads each occurrence's signature once and stores no hit; it serves
+// searches in which a chain needs two hits (min_hsp_len > span) at most SIG_FIELDS windows
+// apart (with SIG_FLANK: windows that overlap or touch), the distances a signature holds.
+// Everything else, and a search for which a hit-storing path is forced, goes through the
+// buckets or the global sort below.  Where both serve, the scan is faster at every size
+// measured (scan and chains against fill, grouping and the sort of its spills): one query of
+// 2,000 bases on 4 Gbp 29 against 36 us; 4,096 short queries on 400 Mbp 0.18 against 0.60 ms;
+// 2,000 queries on 4 Gbp 1.46 against 3.70 ms; 500 queries at stride 1 0.13 against 3.2 ms.
+bool takes_scan(const gn_index *ix, const gn_params &p) {
+    const uint32_t links = p.max_hit_distance / (uint32_t)ix->t;  // windows from one hit to the next, at most
+    return ix->sig_d && p.min_hsp_len > (uint32_t)ix->span && !(p.flags & GN_FLAG_KEEP_HITS) && !hit_path_forced() && links >= 1 &&
+           links <= (uint32_t)(sig_kind(ix->k, ix->span, ix->t) == SIG_FLANK ? ix->k : SIG_FIELDS);
+}
+
 // Segments of a query set: one per MAX_QUERY_LEN bases or part, SEG_STEP apart (see search).
 uint64_t count_segments(const std::vector<uint64_t> &qstart) {
     uint64_t n = 0;
@@ -2742,20 +2757,10 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         hqp.nb = arena.alloc_n<uint32_t>(Packed::nb_words(HM));
         pack_bases(sb, HM, hqp, s);
     }
-    // Seed lookup and chaining take one of two routes to the same HSPs.  The signature scan
-    // (gn_seed_scan.cuh) reads each occurrence's signature once and stores no hit; it serves
-    // searches in which a chain needs two hits (min_hsp_len > span) at most SIG_FIELDS windows
-    // apart (with SIG_FLANK: windows that overlap or touch), the distances a signature holds.
-    // Everything else, and a search for which a hit-storing path is forced, goes through the
-    // buckets or the global sort below.  Where both serve, the scan is faster at every size
-    // measured (scan and chains against fill, grouping and the sort of its spills): one query of
-    // 2,000 bases on 4 Gbp 29 against 36 us; 4,096 short queries on 400 Mbp 0.18 against 0.60 ms;
-    // 2,000 queries on 4 Gbp 1.46 against 3.70 ms; 500 queries at stride 1 0.13 against 3.2 ms.
     const int singles = p.min_hsp_len <= (uint32_t)k ? 1 : 0;
     const SigKind kind = sig_kind(ix->k, ix->span, ix->t);
     const uint32_t links = p.max_hit_distance / (uint32_t)ix->t;  // windows from one hit to the next, at most
-    const bool scan = ix->sig_d && !singles && !keep_hits && !hit_path_forced() &&
-                      (kind == SIG_FLANK ? links >= 1 && links <= (uint32_t)k : links >= 1 && links <= (uint32_t)SIG_FIELDS);
+    const bool scan = takes_scan(ix, p);
     uint32_t *codes = scan ? nullptr : arena.alloc_n<uint32_t>(HM);
     uint32_t *qinfo = arena.alloc_n<uint32_t>(HM);
     uint32_t *cnt = arena.alloc_n<uint32_t>(HM);  // list lengths; scan route: list units
@@ -3559,7 +3564,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         // 613.  So rows from 512 at 4 warps an SM, from 1,024 at 8 with more than 64 alignments an
         // SM (sw_long_rows, sw_many: the device knows the number), and with no more alignments
         // than warps each gets its own, in any order (sw_lanes = 32 asks for that).
-        uint32_t sw_long = ix->tuning.sw_wave_rows;
+        uint32_t sw_long = ix->rows_by_count ? 0u : ix->tuning.sw_wave_rows;
         if (const char *e = getenv("GN_SW_LONG_ROWS")) sw_long = (uint32_t)std::max(1l, strtol(e, nullptr, 10));
         if (sw_lanes == 32) sw_long = 1;
         const bool ordered = sel_cap > sms * 4 || getenv("GN_SW_LONG_ROWS");
