@@ -87,12 +87,13 @@ HSP_DTYPE = np.dtype([("query", "<u4"), ("seq", "<u4"), ("q_start", "<u4"), ("q_
 STAGE_HIT_DTYPE = np.dtype([("query", "<u4"), ("qpos", "<u4"), ("seq", "<u4"), ("pos", "<u4")])
 
 _lib = None
+_quick = None  # polls that do not wait, called without giving the interpreter lock up
 _lock = threading.Lock()
 
 
 def load():
     """Loads the CUDA library; raises if it has not been built."""
-    global _lib
+    global _lib, _quick
     with _lock:
         if _lib is not None:
             return _lib
@@ -151,6 +152,10 @@ def load():
             f = getattr(lib, name)
             f.restype = res
             f.argtypes = args
+        _quick = ctypes.PyDLL(path)
+        for name in ("gn_serve_poll", "gn_serve_poll_any"):
+            f = getattr(_quick, name)
+            f.restype, f.argtypes = sig[name]
         _lib = lib
         return lib
 
@@ -321,10 +326,16 @@ def gn_serve_submit(s: int, bases: bytes) -> int:
     return t.value
 
 
+# A finished request is fetched without giving the interpreter lock up: that is a lookup under the
+# server's lock, and where one thread submits while another collects, handing the interpreter to and
+# fro for each call costs more than the calls.  4,000 requests submitted at once (4 Gbp): 400 Mbp/s
+# and 99 % within 34 ms where every poll is a hand-over, 770 and 17 where only waiting polls are.
 def gn_serve_poll(s: int, ticket: int, timeout_ms: int):
     """Returns a results handle, or None on GN_ETIMEOUT."""
-    r = ctypes.c_void_p()
-    st = load().gn_serve_poll(ctypes.c_void_p(s), ticket, timeout_ms, ctypes.byref(r))
+    lib, r = load(), ctypes.c_void_p()
+    st = _quick.gn_serve_poll(s, ticket, 0, ctypes.byref(r))
+    if st == GN_ETIMEOUT and timeout_ms:
+        st = lib.gn_serve_poll(s, ticket, timeout_ms, ctypes.byref(r))
     if st == GN_ETIMEOUT:
         return None
     _check(st)
@@ -334,9 +345,11 @@ def gn_serve_poll(s: int, ticket: int, timeout_ms: int):
 def gn_serve_poll_any(s: int, timeout_ms: int):
     """(ticket, results handle) of the oldest finished request, or None on GN_ETIMEOUT.
     A failed request raises GnError."""
-    r = ctypes.c_void_p()
+    lib, r = load(), ctypes.c_void_p()
     t = ctypes.c_uint64()
-    st = load().gn_serve_poll_any(ctypes.c_void_p(s), timeout_ms, ctypes.byref(t), ctypes.byref(r))
+    st = _quick.gn_serve_poll_any(s, 0, ctypes.byref(t), ctypes.byref(r))
+    if st == GN_ETIMEOUT and timeout_ms:
+        st = lib.gn_serve_poll_any(s, timeout_ms, ctypes.byref(t), ctypes.byref(r))
     if st == GN_ETIMEOUT:
         return None
     _check(st)

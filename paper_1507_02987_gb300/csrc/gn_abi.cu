@@ -282,21 +282,32 @@ static void serve_worker(gn_server *sv) {
             }
             search(const_cast<gn_index *>(sv->ix), b, qstart, o, s, &all);
         });
-        if (st != GN_OK) err = g_last_error;
+        // Each request's result is made before the lock is taken, under which submissions and polls
+        // wait: what is left there is to link the finished entries in.
+        std::map<uint64_t, gn_results *> done;
+        if (st == GN_OK) {
+            st = guarded([&] {
+                for (size_t i = 0; i < batch.size(); ++i) {
+                    auto r = std::make_unique<gn_results>();
+                    r->n_queries = 1;
+                    r->qoff = {0, all.qoff[i + 1] - all.qoff[i]};
+                    r->hits.assign(all.hits.begin() + all.qoff[i], all.hits.begin() + all.qoff[i + 1]);
+                    for (auto &h : r->hits) h.query = 0;
+                    done.emplace_hint(done.end(), batch[i].ticket, r.get());
+                    r.release();
+                }
+            });
+        }
+        if (st != GN_OK) {
+            err = g_last_error;
+            for (auto &d : done) delete d.second;
+            done.clear();
+        }
         {
             std::lock_guard<std::mutex> lk(sv->mu);
-            for (size_t i = 0; i < batch.size(); ++i) {
-                if (st != GN_OK) {
-                    sv->failed[batch[i].ticket] = {st, err};
-                    continue;
-                }
-                gn_results *r = new gn_results();
-                r->n_queries = 1;
-                r->qoff = {0, all.qoff[i + 1] - all.qoff[i]};
-                r->hits.assign(all.hits.begin() + all.qoff[i], all.hits.begin() + all.qoff[i + 1]);
-                for (auto &h : r->hits) h.query = 0;
-                sv->done[batch[i].ticket] = r;
-            }
+            if (st == GN_OK) sv->done.merge(done);
+            else
+                for (auto &r : batch) sv->failed[r.ticket] = {st, err};
             sv->in_use -= taken;
             sv->running -= 1;
         }
@@ -715,7 +726,7 @@ gn_status gn_serve_poll(gn_server *sv, uint64_t ticket, uint32_t timeout_ms, gn_
     *out = nullptr;
     std::unique_lock<std::mutex> lk(sv->mu);
     auto ready = [&] { return sv->done.count(ticket) || sv->failed.count(ticket); };
-    if (!sv->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms), ready)) {
+    if (!(timeout_ms ? sv->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms), ready) : ready())) {
         g_last_error = "not done yet";
         return GN_ETIMEOUT;
     }
@@ -739,7 +750,7 @@ gn_status gn_serve_poll_any(gn_server *sv, uint32_t timeout_ms, uint64_t *ticket
     *ticket = 0;
     std::unique_lock<std::mutex> lk(sv->mu);
     auto ready = [&] { return !sv->done.empty() || !sv->failed.empty(); };
-    if (!sv->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms), ready)) {
+    if (!(timeout_ms ? sv->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms), ready) : ready())) {
         g_last_error = "nothing done yet";
         return GN_ETIMEOUT;
     }
