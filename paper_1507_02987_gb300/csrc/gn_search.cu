@@ -2645,6 +2645,9 @@ bool takes_scan(const gn_index *ix, const gn_params &p) {
            links <= (uint32_t)(sig_kind(ix->k, ix->span, ix->t) == SIG_FLANK ? ix->k : SIG_FIELDS);
 }
 
+// Candidates that a list is enlarged to without asking for the free memory (256 MB).
+constexpr uint64_t CAND_ASK = 1ull << 25;
+
 // Segments of a query set: one per MAX_QUERY_LEN bases or part, SEG_STEP apart (see search).
 uint64_t count_segments(const std::vector<uint64_t> &qstart) {
     uint64_t n = 0;
@@ -2936,7 +2939,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
             GN_REQUIRE(attempt < 64, GN_EINTERNAL, "candidate and HSP list sizing did not converge");
             if (!scanned) {
                 const uint64_t want = done + here < all ? n_cand + n_cand / 4 : n_cand,
-                               room = list_room((uint64_t)(0.55 * free_bytes()));
+                               room = list_room(want > CAND_ASK ? (uint64_t)(0.55 * free_bytes()) : ~0ull);
                 if (n_cand > room) {  // fewer units, as their candidates go; a quarter of the list's length always fits it
                     cand_cap = std::max(cand_cap, room);
                     scan_range = std::max<uint64_t>({1, cand_cap / 4, (uint64_t)(0.75 * (double)here * (double)cand_cap / (double)n_cand)});
