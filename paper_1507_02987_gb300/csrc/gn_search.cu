@@ -2615,13 +2615,14 @@ void both_strands(const uint8_t *qbases_dev, const std::vector<uint64_t> &qstart
 // Words that a search's kernels write and its host code reads.
 struct SearchWords {
     uint32_t wait_status, status;
-    uint32_t n_hsp, n_cand;            // HSPs and candidates of the signature scan
-    uint32_t next_tile, next_cand;
+    uint32_t n_hsp, next_cand;         // of the signature scan's range: HSPs, candidates,
+    unsigned long long n_cand;         // and list units of all offsets
+    uint32_t next_tile, scan_pad;
+    unsigned long long n_units;
     uint32_t n_wide, next_wide, next_task, n_long, next_long;
     uint32_t n_strip, strip_band, next_strip;
     uint32_t too_many, recs_done;
     uint32_t groups[8];                // groups of a block, of a large block, of no kernel: of the join, of the merge
-    unsigned long long n_units;        // list units of all offsets
     unsigned long long next_end, cells[2];
     uint32_t bins[SWO_BINS], placed[SWO_BINS];
 };
@@ -2843,7 +2844,7 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
 
     // The scan route sizes its lists from the hits that the list lengths' mean promises (repeats
     // and skewed bases bring more): lists that turn out short are enlarged and their kernel rerun.
-    const uint64_t hits_guess = scan ? (uint64_t)std::min((double)HM * (double)ix->n_postings / std::pow(4.0, ix->k), 4.0 * SCAN_RANGE) : hq[hnq];
+    const uint64_t hits_guess = scan ? (uint64_t)std::min((double)HM * (double)ix->n_postings / std::pow(4.0, ix->k), (double)CAND_MAX) : hq[hnq];
     uint32_t hsp_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFFFull, std::max<uint64_t>(1u << 14, hits_guess / 64));
     DevHsp *hsp = arena.alloc_n<DevHsp>(hsp_cap);
     uint32_t n_hsp = 0;
@@ -2887,13 +2888,14 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         // The scan takes all units in one launch, or ranges of them, each scanned, checked and its HSPs
         // appended before the next: SCAN_RANGE units at a time, or as many as leave a list of
         // candidates that memory has room for (55 % of what is free, and no more than the caller grants).
-        // Room for candidates to begin with: about 1 % of the hits at stride 11 are.
+        // A range costs a host wait and the ends of two kernels: 8.7 G hits at stride 1 took 7.60 ms in
+        // five and 7.39 in one.  Room for candidates to begin with: about 1 % of the hits at stride 11 are.
         DeviceArena lists(s);  // enlarged candidate lists
         auto list_room = [&](uint64_t bytes) {  // candidates that `bytes` hold, within what the caller grants
             if (o.mem_cap) bytes = std::min(bytes, o.mem_cap);
             uint64_t room = std::max<uint64_t>(1u << 20, bytes / sizeof(uint2));
             if (const char *e = getenv("GN_CAND_ROOM")) room = std::max<uint64_t>(4, strtoull(e, nullptr, 10));  // (a unit's)
-            return std::min(room, 4 * SCAN_RANGE);
+            return std::min(room, CAND_MAX);
         };
         uint64_t cand_cap = std::min(std::max<uint64_t>(1u << 14, hits_guess / 24), list_room(~0ull));
         uint2 *cand = arena.alloc_n<uint2>(cand_cap);
@@ -2902,11 +2904,8 @@ void search(gn_index *ix, const uint8_t *qbases_dev, const std::vector<uint64_t>
         bool scanned = false;  // the range's candidates are listed
         int attempt = 0;       // of the range
         for (uint64_t done = 0, all = 1; done < all; ++attempt) {
-            if (done || attempt) {  // n_hsp and next_cand, and the scan's own counters if it runs again
-                GN_CUDA(cudaMemsetAsync(&words->n_hsp, 0, 4, s));
-                GN_CUDA(cudaMemsetAsync(&words->next_cand, 0, 4, s));
-                if (!scanned) GN_CUDA(cudaMemsetAsync(&words->n_cand, 0, 8, s));
-            }
+            if (done || attempt)  // n_hsp and next_cand; n_cand and next_tile too if the scan runs again
+                GN_CUDA(cudaMemsetAsync(&words->n_hsp, 0, scanned ? 8 : 20, s));
             if (!scanned)
                 GN_LAUNCH("k_seed_scan", units, s,
                           kernel<<<grid, SCAN_THREADS, 0, s>>>(qrec, hoff, HM, done, done + scan_range, &words->n_units,

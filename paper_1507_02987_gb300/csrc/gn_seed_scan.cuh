@@ -405,9 +405,10 @@ __device__ __forceinline__ void scan_check_flank(const ScanCtx &c, bool valid, u
 constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_STEPS = 4;
 constexpr int SCAN_QUEUE = 64;
-// Units of one launch, at most: candidates and HSPs are counted in 32 bits (in low-complexity
-// sequence every hit is a candidate), and up to 2^31 of them are.
-constexpr uint64_t SCAN_RANGE = 1ull << 29;
+// Units of one launch, at most (a call's limits are checked after the first; a tile's number has 32
+// bits), and candidates of one list, at most: in low-complexity sequence every hit is a
+// candidate, so they are counted in 64 bits, and listed, checked and made HSPs of in 32.
+constexpr uint64_t SCAN_RANGE = 1ull << 32, CAND_MAX = 1ull << 31;
 
 // A launch takes the units [u_from, u_to); n_all: where it leaves the number of all units.
 template <int KIND>
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_seed_scan(const QueryRec *_
                                                                unsigned long long *__restrict__ n_all,
                                                                const uint4 *__restrict__ sig4, uint64_t n_units,
                                                                int flank, uint2 *__restrict__ cand,
-                                                               uint32_t *__restrict__ cand_count, uint32_t cand_cap,
+                                                               unsigned long long *__restrict__ cand_count, uint32_t cand_cap,
                                                                uint32_t *__restrict__ next_tile) {
     __shared__ uint2 queue_s[SCAN_THREADS / 32][SCAN_QUEUE];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -431,8 +432,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_seed_scan(const QueryRec *_
     const uint64_t R = min((uint64_t)1024, max((uint64_t)64, (uint64_t)(((total - u_from) / (warps * 8) + 31) & ~31ull)));
     const uint32_t next_mask = KIND == SIG_FLANK ? sig_flank_mask(flank) : 0u;
     auto flush = [&](uint32_t n) {  // the first n (<= 32) queued candidates
-        uint32_t at = 0;
-        if (lane == 0) at = atomicAdd(cand_count, n);
+        unsigned long long at = 0;
+        if (lane == 0) at = atomicAdd(cand_count, (unsigned long long)n);
         at = __shfl_sync(0xffffffffu, at, 0) + lane;
         __syncwarp();
         if ((uint32_t)lane < n && at < cand_cap) cand[at] = queue[lane];
@@ -533,10 +534,10 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_seed_scan(const QueryRec *_
 // Checks the candidates of the scan, 32 to a warp from a counter.
 template <int KIND, bool EDGES>
 __global__ void __launch_bounds__(SCAN_THREADS) k_chain(const __grid_constant__ ScanCtx c, const uint2 *__restrict__ cand,
-                                                        const uint32_t *__restrict__ cand_count, uint32_t cand_cap,
+                                                        const unsigned long long *__restrict__ cand_count, uint32_t cand_cap,
                                                         uint32_t *__restrict__ next) {
     const int lane = threadIdx.x & 31;
-    const uint32_t n = min(*cand_count, cand_cap);
+    const uint32_t n = (uint32_t)min(*cand_count, (unsigned long long)cand_cap);
     for (;;) {
         uint32_t at = 0;
         if (lane == 0) at = atomicAdd(next, 32u);
