@@ -492,8 +492,9 @@ class Results:
         return gn_results_get(self.handle, i)
 
     def all(self) -> list[np.ndarray]:
-        """Every query's hits, cut from one copy of all of them (4,096 queries: 0.9 ms; 12 ms with a
-        call and a copy for each)."""
+        """Every query's hits, as views of one copy of all of them (4,096 queries: 0.9 ms; 12 ms with a
+        call and a copy for each): one query's array keeps the others' memory alive; copy it, or
+        take query(i), to keep it alone."""
         hits, start = gn_results_all(self.handle)
         return [hits[a:b] for a, b in zip(start, start[1:])]
 
